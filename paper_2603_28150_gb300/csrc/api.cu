@@ -177,8 +177,11 @@ size_t ws_walk(pat_plan* pp, unsigned char* base, bool with_io, int64_t lean_sli
   const Layout& L = p.L;
   const bool lean = lean_slices > 0;
   const size_t cs = 2 * L.rsize;
-  const int64_t smax = lean ? lean_slices : (int64_t)L.max_batch * std::max(L.nz, L.nt);
-  const size_t xy = lean ? 0 : (size_t)smax * spectrum_row_cap(L) * cs;
+  const int64_t per = std::max(L.nz, L.nt);
+  const int64_t smax = lean ? lean_slices : (int64_t)L.max_batch * per;
+  // a volume's slices rounded up to whole quads where the plan may fold
+  const int64_t rows = L.fp64 || L.px != L.py ? smax : (int64_t)L.max_batch * ((per + 3) / 4 * 4);
+  const size_t xy = lean ? 0 : (size_t)rows * spectrum_row_cap(L) * cs;
   const size_t tb = (size_t)smax * L.tslice * cs;
   const size_t vol = lean ? 0 : (size_t)L.max_batch * L.nz * L.ny * L.nx * L.rsize;
   const size_t dat = lean ? 0 : (size_t)L.max_batch * L.nt * L.ny * L.nx * L.rsize;
@@ -343,15 +346,12 @@ cudaError_t forward_dev(const Plan& p, const void* rho, void* d, int batch, cuda
                         const void* sub, double* sumsq, int groups, double* group_sums) {
   const Layout& L = p.L;
   const int64_t plane = (int64_t)L.ny * L.nx, scan = (int64_t)L.my * L.mx;
-  const bool sl = tc_slots(p, batch);
-  const int64_t row = sl ? slot_row(L) : L.Kpad;
-  const int* slot = sl ? p.fold_slot : nullptr;
-  cudaError_t e = launch_spectrum(p, rho, plane, L.nx, L.ny, p.X, row, batch * L.nz, s,
-                                  no_sampling(), slot);
+  const SpecRow zr = spec_row(p, batch, L.nz), tr = spec_row(p, batch, L.nt);
+  cudaError_t e = launch_spectrum(p, rho, plane, L.nx, L.ny, p.X, zr, batch * L.nz, s);
   if (e != cudaSuccess) return e;
-  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s)) != cudaSuccess) return e;
-  return launch_image(p, p.Y, row, d, scan, batch * L.nt, sub, sumsq, s, groups, group_sums,
-                      sampling_of(L), slot);
+  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s, zr.quad > 0)) != cudaSuccess) return e;
+  return launch_image(p, p.Y, tr, d, scan, batch * L.nt, sub, sumsq, s, groups, group_sums,
+                      sampling_of(L));
 }
 
 cudaError_t gradient_dev(const Plan& p, const void* x, const void* y, void* grad, int batch,
@@ -359,38 +359,31 @@ cudaError_t gradient_dev(const Plan& p, const void* x, const void* y, void* grad
                          const FistaStep* step) {
   const Layout& L = p.L;
   const int64_t plane = (int64_t)L.ny * L.nx, scan = (int64_t)L.my * L.mx;
-  const bool sl = tc_slots(p, batch);
-  const int64_t row = sl ? slot_row(L) : L.Kpad;
-  const int* slot = sl ? p.fold_slot : nullptr;
+  const SpecRow zr = spec_row(p, batch, L.nz), tr = spec_row(p, batch, L.nt);
+  const bool quad = zr.quad > 0;
   // with a step that leaves the row transform of the next x in T, stage i
   // here is its column pass alone
   cudaError_t e = (step && step->next_T)
-                      ? launch_spectrum_cols(p, L.ny, p.X, row, batch * L.nz, s, slot)
-                      : launch_spectrum(p, x, plane, L.nx, L.ny, p.X, row, batch * L.nz, s,
-                                        no_sampling(), slot);
+                      ? launch_spectrum_cols(p, L.ny, p.X, zr, batch * L.nz, s)
+                      : launch_spectrum(p, x, plane, L.nx, L.ny, p.X, zr, batch * L.nz, s);
   if (e != cudaSuccess) return e;
-  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s)) != cudaSuccess) return e;
-  if ((e = launch_residual(p, p.Y, row, y, scan, batch * L.nt, sumsq, s, groups, group_sums,
-                           sampling_of(L), slot, p.Y, row)) != cudaSuccess)
+  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s, quad)) != cudaSuccess) return e;
+  if ((e = launch_residual(p, p.Y, tr, y, scan, batch * L.nt, sumsq, s, groups, group_sums,
+                           sampling_of(L), p.Y)) != cudaSuccess)
     return e;
-  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s)) != cudaSuccess) return e;
-  if (step) return launch_image_step(p, p.X, row, batch * L.nz, *step, s, slot);
-  return launch_image(p, p.X, row, grad, plane, batch * L.nz, nullptr, nullptr, s, 0, nullptr,
-                      no_sampling(), slot);
+  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s, quad)) != cudaSuccess) return e;
+  if (step) return launch_image_step(p, p.X, zr, batch * L.nz, *step, s);
+  return launch_image(p, p.X, zr, grad, plane, batch * L.nz, nullptr, nullptr, s);
 }
 
 cudaError_t adjoint_dev(const Plan& p, const void* d, void* rho, int batch, cudaStream_t s) {
   const Layout& L = p.L;
   const int64_t plane = (int64_t)L.ny * L.nx, scan = (int64_t)L.my * L.mx;
-  const bool sl = tc_slots(p, batch);
-  const int64_t row = sl ? slot_row(L) : L.Kpad;
-  const int* slot = sl ? p.fold_slot : nullptr;
-  cudaError_t e = launch_spectrum(p, d, scan, L.nx, L.ny, p.Y, row, batch * L.nt, s,
-                                  sampling_of(L), slot);
+  const SpecRow zr = spec_row(p, batch, L.nz), tr = spec_row(p, batch, L.nt);
+  cudaError_t e = launch_spectrum(p, d, scan, L.nx, L.ny, p.Y, tr, batch * L.nt, s, sampling_of(L));
   if (e != cudaSuccess) return e;
-  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s)) != cudaSuccess) return e;
-  return launch_image(p, p.X, row, rho, plane, batch * L.nz, nullptr, nullptr, s, 0, nullptr,
-                      no_sampling(), slot);
+  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s, zr.quad > 0)) != cudaSuccess) return e;
+  return launch_image(p, p.X, zr, rho, plane, batch * L.nz, nullptr, nullptr, s);
 }
 
 cudaError_t instantiate_counted(cudaGraph_t graph, cudaGraphExec_t* exec, int* kernels) {
@@ -983,7 +976,9 @@ int pat_stage_spectrum(pat_plan* plan, const void* in, void* out, int slices, pa
   const Layout& L = plan->p.L;
   if (slices < 0 || slices > L.max_batch * std::max(L.nz, L.nt))
     return fail(PAT_ERR_ARG, "slices must be in [0, max_batch * max(nz, nt)]");
-  PAT_CUDA(launch_spectrum(plan->p, in, (int64_t)L.ny * L.nx, L.nx, L.ny, out, L.K, slices,
+  SpecRow sr;
+  sr.stride = L.K;
+  PAT_CUDA(launch_spectrum(plan->p, in, (int64_t)L.ny * L.nx, L.nx, L.ny, out, sr, slices,
                            (cudaStream_t)stream));
   return PAT_OK;
   PAT_GUARD_END
@@ -996,7 +991,9 @@ int pat_stage_image(pat_plan* plan, const void* in, void* out, int slices, pat_s
   const Layout& L = plan->p.L;
   if (slices < 0 || slices > L.max_batch * std::max(L.nz, L.nt))
     return fail(PAT_ERR_ARG, "slices must be in [0, max_batch * max(nz, nt)]");
-  PAT_CUDA(launch_image(plan->p, in, L.K, out, (int64_t)L.ny * L.nx, slices, nullptr, nullptr,
+  SpecRow sr;
+  sr.stride = L.K;
+  PAT_CUDA(launch_image(plan->p, in, sr, out, (int64_t)L.ny * L.nx, slices, nullptr, nullptr,
                         (cudaStream_t)stream));
   return PAT_OK;
   PAT_GUARD_END

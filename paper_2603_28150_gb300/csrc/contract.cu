@@ -21,6 +21,7 @@ namespace pat {
 namespace {
 
 constexpr int kWarps = 8;
+constexpr int64_t kFoldCtas = 304;  // two CTAs on each of 152 SMs
 
 template <typename R, bool CPLX>
 struct Elem;  // table element type and z per 16-byte group
@@ -212,92 +213,261 @@ __global__ void __launch_bounds__(kWarps * 32, (sizeof(R) == 4 && !CPLX && VB ==
 // whose bin indices come from `members` ([block][lane][4], -1 = absent). CTA j
 // reads stored chunk chunk[j] of 32 rows (chunk j when `chunk` is NULL): with
 // radial sharing the CTAs of one radius group read the same chunk at about
-// the same time, so DRAM delivers it once and L2 serves the others. One
-// volume per blockIdx.y; every volume streams the (folded) table once.
-constexpr int kRT = 4;   // forward: time samples per register block
-constexpr int kTC = 32;  // adjoint: time samples per shared D tile
+// the same time, so DRAM delivers it once and L2 serves the others; the
+// volumes of a batch are neighbouring CTAs for the same reason.
+//
+// The members of a block's representatives are scattered over the half
+// spectrum, so with one row of bins per slice every access is an 8-byte piece
+// of a 32-byte sector. QUAD spectra interleave four slices ([slice / 4][bin]
+// [slice % 4], see SpecRow): a lane's four time samples (depths) of one bin
+// are one whole sector. The spectra of a block are staged in shared memory in
+// the same quads, [member][quad][lane] with the 16-byte halves of a quad
+// swizzled so that a warp's 16-byte reads touch every bank once.
+//
+// Measured per launch (one GB300, forward / adjoint): 128^2 -> 256^2 x 64 x
+// 256, 0.40 GB stored: 93 / 90 us, from 110 / 113 with bin rows and the table
+// loaded into registers; 256^2 -> 512^2 x 128 x 512, 5.8 GB: 1250 / 1233 from
+// 2270 / 1915; 202^2 -> 512^2 x 17 x 201: 147 / 173 from 507 / 316; five
+// volumes at 64^2 -> 128^2 x 32 x 128: 35 / 39 from 57 / 76. Without the table
+// copies the 128^2 launch takes 70 / 62 us and without the multiply-adds 80 /
+// 88: shared-memory and L1 traffic (the spectra, the ring and the 32-line
+// stores of scattered sectors) and the table stream overlap only in part.
+constexpr int kFoldThreads = 512;  // most threads of a CTA (caps the registers at 128)
 
-// Forward: warp w takes the time blocks w, w + 8, ... of kRT samples; per
-// z-group it loads kRT table float4s and the 4 members' X from shared memory.
-__global__ void __launch_bounds__(kWarps * 32, 2)
-    k_fold_fwd(const float4* __restrict__ table, const int4* __restrict__ members,
-               const int* __restrict__ chunk, const cx<float>* __restrict__ X,
-               cx<float>* __restrict__ Y, int nz, int nt, int nzg, int64_t Kpad) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<float>* xs = reinterpret_cast<cx<float>*>(smem_raw);  // [4][nzp][32]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t ub = blockIdx.x;
-  const int b = blockIdx.y, nzp = nzg * 4;
-  const int4 mem = members[ub * 32 + lane];
-  const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
-  const cx<float>* Xb = X + (int64_t)b * nz * Kpad;
-  pdl_wait();
-  for (int z = warp; z < nzp; z += kWarps) {
+// 16-byte slot of half h (slices 2h, 2h + 1) of a lane's quad in its 1 KB row.
+__device__ __forceinline__ int quad_slot(int lane, int h) {
+  return (2 * lane + h) ^ ((lane >> 2) & 1);
+}
+
+// Starts the copy of quads [q0, q0 + nq) of the four members' spectra into
+// dst[4][rows][64] (16-byte slots); slices at or past n and absent members
+// become zero. in: this volume's spectra.
+template <bool QUAD>
+__device__ __forceinline__ void stage_quads(float4* dst, int rows, const cx<float>* in,
+                                            const int* bins, int q0, int nq, int n, int64_t Kpad,
+                                            int lane, int warp, int nwarps) {
+  for (int q = warp; q < nq; q += nwarps) {
 #pragma unroll
-    for (int m = 0; m < 4; ++m)
-      xs[(m * nzp + z) * 32 + lane] =
-          (bins[m] >= 0 && z < nz) ? Xb[(int64_t)z * Kpad + bins[m]] : mk<float>(0.f, 0.f);
+    for (int m = 0; m < 4; ++m) {
+      const bool ok = bins[m] >= 0;
+      const int64_t bin = ok ? bins[m] : 0;
+      float4* row = dst + (m * rows + q) * 64;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(row + quad_slot(lane, h));
+        const int s = 4 * (q0 + q) + 2 * h;  // first slice of this half
+        if constexpr (QUAD) {
+          const int bytes = ok ? 8 * max(0, min(2, n - s)) : 0;
+          const cx<float>* src = in + ((int64_t)(q0 + q) * Kpad + bin) * 4 + 2 * h;
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d),
+                       "l"(bytes ? src : in), "r"(bytes)
+                       : "memory");
+        } else {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int bytes = ok && s + i < n ? 8 : 0;
+            const cx<float>* src = in + (int64_t)(s + i) * Kpad + bin;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d + 8 * i),
+                         "l"(bytes ? src : in), "r"(bytes)
+                         : "memory");
+          }
+        }
+      }
+    }
   }
-  __syncthreads();
-  const int64_t cb = chunk ? chunk[ub] : ub;
-  const float4* tb = table + cb * nt * (int64_t)nzg * 32 + lane;
-  for (int t0 = warp * kRT; t0 < nt; t0 += kWarps * kRT) {
-    cx<float> acc[kRT][4];
-#pragma unroll
-    for (int r = 0; r < kRT; ++r)
-#pragma unroll
-      for (int m = 0; m < 4; ++m) acc[r][m] = mk<float>(0.f, 0.f);
-#pragma unroll 4
-    for (int g = 0; g < nzg; ++g) {
-      float hv[kRT][4];
-#pragma unroll
-      for (int r = 0; r < kRT; ++r) {
-        float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (t0 + r < nt) h = ld_stream(tb + ((int64_t)(t0 + r) * nzg + g) * 32);
-        hv[r][0] = h.x;
-        hv[r][1] = h.y;
-        hv[r][2] = h.z;
-        hv[r][3] = h.w;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        cx<float> x[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) x[m] = xs[(m * nzp + g * 4 + q) * 32 + lane];
-#pragma unroll
-        for (int r = 0; r < kRT; ++r)
-#pragma unroll
-          for (int m = 0; m < 4; ++m) mac(acc[r][m], hv[r][q], x[m]);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < kRT; ++r) {
-      const int t = t0 + r;
-      if (t >= nt) break;
-#pragma unroll
-      for (int m = 0; m < 4; ++m)
-        if (bins[m] >= 0) Y[((int64_t)b * nt + t) * Kpad + bins[m]] = acc[r][m];
-    }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Stores the values of four consecutive slices 4q .. 4q + 3 of one bin.
+template <bool QUAD>
+__device__ __forceinline__ void store_quad(cx<float>* out, int q, int bin, int n, int64_t Kpad,
+                                           cx<float> a, cx<float> b, cx<float> c, cx<float> d) {
+  if constexpr (QUAD) {  // slices at or past n are padding that no reader uses
+    float4* o = reinterpret_cast<float4*>(out + ((int64_t)q * Kpad + bin) * 4);
+    o[0] = make_float4(a.x, a.y, b.x, b.y);
+    o[1] = make_float4(c.x, c.y, d.x, d.y);
+  } else {
+    cx<float>* o = out + (int64_t)(4 * q) * Kpad + bin;
+    if (4 * q < n) o[0] = a;
+    if (4 * q + 1 < n) o[Kpad] = b;
+    if (4 * q + 2 < n) o[2 * Kpad] = c;
+    if (4 * q + 3 < n) o[3 * Kpad] = d;
   }
 }
 
-// Adjoint: warp w of z-chunk c owns z-groups c*8*GPW + w + j*8; the 4 members'
-// D values of kTC samples are staged in shared memory and reused by all warps.
-template <int GPW>
-__global__ void __launch_bounds__(kWarps * 32, 2)
+// Adds what store_quad wrote to a .. d.
+template <bool QUAD>
+__device__ __forceinline__ void add_quad(const cx<float>* out, int q, int bin, int n, int64_t Kpad,
+                                         cx<float>& a, cx<float>& b, cx<float>& c, cx<float>& d) {
+  const cx<float>* o = QUAD ? out + ((int64_t)q * Kpad + bin) * 4 : out + (int64_t)(4 * q) * Kpad + bin;
+  const int64_t st = QUAD ? 1 : Kpad;
+  a = cadd(a, o[0]);
+  if (4 * q + 1 < n) b = cadd(b, o[st]);
+  if (4 * q + 2 < n) c = cadd(c, o[2 * st]);
+  if (4 * q + 3 < n) d = cadd(d, o[3 * st]);
+}
+
+// Complex values per volume of a spectrum of n slices.
+template <bool QUAD>
+__device__ __forceinline__ int64_t vol_len(int n, int64_t Kpad) {
+  return (QUAD ? (int64_t)((n + 3) / 4) * 4 : (int64_t)n) * Kpad;
+}
+
+// 16-byte asynchronous copy of a table float4 (zero when !ok).
+__device__ __forceinline__ void cp_table(float4* dst, const float4* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(ok ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Forward: a warp takes blocks of T time samples and walks the z-groups; the
+// T table float4s of a step sit in the warp's ring of R slots, copied ahead by
+// the lanes that read them (no barrier: a lane reads its own copies), so the
+// table bytes in flight do not cost registers.
+// grid (batch, nrb, splits of the time blocks), tb time blocks per split.
+template <bool QUAD, int T, int R>
+__global__ void __launch_bounds__(kFoldThreads, 1)
+    k_fold_fwd(const float4* __restrict__ table, const int4* __restrict__ members,
+               const int* __restrict__ chunk, const cx<float>* __restrict__ X,
+               cx<float>* __restrict__ Y, int nz, int nt, int nzg, int64_t Kpad, int tb, int gc) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  float4* xs = reinterpret_cast<float4*>(smem_raw);  // [4][gc][64]
+  float4* ring = xs + 4 * gc * 64 + warp * (R * T * 32) + lane;
+  const int64_t ub = blockIdx.y;
+  const int b = blockIdx.x;
+  const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32 + lane;
+  const int bk0 = blockIdx.z * tb + warp;
+  const int bend = min((nt + T - 1) / T, (int)(blockIdx.z + 1) * tb);
+  for (int g0 = 0; g0 < nzg; g0 += gc) {  // z-groups whose spectra fit: one pass up to gc groups
+    const int g1 = min(nzg, g0 + gc);
+    int pbk = bk0, pg = g0;  // next step to copy
+    auto copy_ahead = [&](int slot) {
+      if (pbk < bend) {
+        const float4* src = tbl + ((int64_t)pbk * T * nzg + pg) * 32;
+#pragma unroll
+        for (int r = 0; r < T; ++r)
+          cp_table(ring + (slot * T + r) * 32, src + (int64_t)r * nzg * 32, pbk * T + r < nt);
+        if (++pg == g1) {
+          pg = g0;
+          pbk += nwarps;
+        }
+      }
+      cp_commit();
+    };
+#pragma unroll
+    for (int i = 0; i < R - 1; ++i) copy_ahead(i);  // the table is constant: no wait needed
+    {
+      const int4 mem = members[ub * 32 + lane];
+      const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
+      if (g0 == 0) pdl_wait();
+      stage_quads<QUAD>(xs, gc, X + b * vol_len<QUAD>(nz, Kpad), bins, g0, g1 - g0, nz, Kpad,
+                        lane, warp, nwarps);
+    }
+    cp_wait<0>();
+    __syncthreads();
+    int slot = 0;
+    for (int bk = bk0; bk < bend; bk += nwarps) {
+      cx<float> acc[T][4];
+#pragma unroll
+      for (int r = 0; r < T; ++r)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[r][m] = mk<float>(0.f, 0.f);
+#pragma unroll 1
+      for (int g = 0; g < g1 - g0; ++g) {
+        copy_ahead((slot + R - 1) % R);
+        cp_wait<R - 1>();
+        float4 h[T];
+#pragma unroll
+        for (int r = 0; r < T; ++r) h[r] = ring[(slot * T + r) * 32];
+        slot = (slot + 1) % R;
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          float4 x[4];
+#pragma unroll
+          for (int m = 0; m < 4; ++m) x[m] = xs[(m * gc + g) * 64 + quad_slot(lane, hf)];
+#pragma unroll
+          for (int r = 0; r < T; ++r)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              mac(acc[r][m], hf ? h[r].z : h[r].x, mk<float>(x[m].x, x[m].y));
+              mac(acc[r][m], hf ? h[r].w : h[r].y, mk<float>(x[m].z, x[m].w));
+            }
+        }
+      }
+      const int4 mem = __ldg(members + ub * 32 + lane);
+      const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
+      cx<float>* Yb = Y + b * vol_len<QUAD>(nt, Kpad);
+#pragma unroll
+      for (int r = 0; r < T; r += 4) {
+        const int q = (bk * T + r) / 4;
+        if (4 * q >= nt) break;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          if (bins[m] < 0) continue;
+          if (g0 > 0) add_quad<QUAD>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m],
+                                     acc[r + 2][m], acc[r + 3][m]);
+          store_quad<QUAD>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m], acc[r + 2][m],
+                           acc[r + 3][m]);
+        }
+      }
+    }
+    if (g1 < nzg) __syncthreads();  // the spectra and rings are free
+  }
+}
+
+// Adjoint: warp (zi, ti) of zw x tw owns the z-groups zc zw GPW + zi + j zw
+// (j < GPW) and the quads ti, ti + tw, ...; the 4 members' D of SQ tw quads
+// are staged in shared memory (two buffers, the next stage's copies in flight
+// during the current one) and reused by all warps; the table comes through
+// the warp's ring as in the forward. With tw > 1 the warps' partial sums of
+// one z-group meet in shared memory at the end, in the order of ti. grid
+// (z-chunks x batch, nrb).
+template <bool QUAD, int GPW, int SQ, int R>
+__global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_adj(const float4* __restrict__ table, const int4* __restrict__ members,
                const int* __restrict__ chunk, const cx<float>* __restrict__ D,
-               cx<float>* __restrict__ Z, int nz, int nt, int nzg, int64_t Kpad) {
-  __shared__ cx<float> ds[kTC][4][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t ub = blockIdx.x;
-  const int b = blockIdx.y;
-  const int gbase = blockIdx.z * kWarps * GPW + warp;
+               cx<float>* __restrict__ Z, int nz, int nt, int nzg, int64_t Kpad, int nzc, int zw,
+               int tw) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int tq = SQ * tw;                            // quads per stage
+  float4* ds = reinterpret_cast<float4*>(smem_raw);  // [2][4][tq][64]
+  float4* ring = ds + 2 * 4 * tq * 64 + warp * (R * 4 * GPW * 32) + lane;
+  const int64_t ub = blockIdx.y;
+  const int zc = blockIdx.x % nzc, b = blockIdx.x / nzc;
+  const int zi = warp % zw, ti = warp / zw;
+  const int gbase = zc * zw * GPW + zi;
+  const float4* tbl =
+      table + ((int64_t)(chunk ? chunk[ub] : ub) * nt * nzg + gbase) * 32 + lane;
+  const int ntq = (nt + 3) / 4, nst = (ntq + tq - 1) / tq;
+  int pq = ti;  // next quad to copy
+  auto copy_ahead = [&](int slot) {
+    if (pq < ntq) {
+      const float4* src = tbl + (int64_t)pq * 4 * nzg * 32;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int j = 0; j < GPW; ++j) {
+          const bool ok = 4 * pq + r < nt && gbase + j * zw < nzg;
+          cp_table(ring + ((slot * 4 + r) * GPW + j) * 32,
+                   ok ? src + ((int64_t)r * nzg + j * zw) * 32 : table, ok);
+        }
+      pq += tw;
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int i = 0; i < R - 1; ++i) copy_ahead(i);
   const int4 mem = members[ub * 32 + lane];
   const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
-  const cx<float>* Db = D + (int64_t)b * nt * Kpad;
-  const int64_t cb = chunk ? chunk[ub] : ub;
-  const float4* tb = table + cb * nt * (int64_t)nzg * 32 + lane;
+  const cx<float>* Db = D + b * vol_len<QUAD>(nt, Kpad);
   cx<float> acc[GPW][4][4];
 #pragma unroll
   for (int j = 0; j < GPW; ++j)
@@ -306,84 +476,183 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
 #pragma unroll
       for (int m = 0; m < 4; ++m) acc[j][q][m] = mk<float>(0.f, 0.f);
   pdl_wait();
-  for (int t0 = 0; t0 < nt; t0 += kTC) {
-    __syncthreads();
-    for (int tt = warp; tt < kTC; tt += kWarps) {
-      const int t = t0 + tt;
+  stage_quads<QUAD>(ds, tq, Db, bins, 0, min(tq, ntq), nt, Kpad, lane, warp, nwarps);
+  cp_wait<0>();
+  int slot = 0;
+  for (int st = 0; st < nst; ++st) {
+    const int q0 = st * tq;
+    // this stage's D: SQ ring groups were committed after its copies
+    if (st > 0) cp_wait<SQ>();
+    __syncthreads();  // and every warp is done with the other buffer
+    if (st + 1 < nst)
+      stage_quads<QUAD>(ds + ((st + 1) & 1) * 4 * tq * 64, tq, Db, bins, q0 + tq,
+                        min(tq, ntq - q0 - tq), nt, Kpad, lane, warp, nwarps);
+    const float4* dst = ds + (st & 1) * 4 * tq * 64;
+#pragma unroll 1
+    for (int i = 0; i < SQ; ++i) {
+      const int q = ti + i * tw;
+      copy_ahead((slot + R - 1) % R);
+      cp_wait<R - 1>();
+      if (q0 + q < ntq) {
+        float4 h[4][GPW];
 #pragma unroll
-      for (int m = 0; m < 4; ++m)
-        ds[tt][m][lane] =
-            (bins[m] >= 0 && t < nt) ? Db[(int64_t)t * Kpad + bins[m]] : mk<float>(0.f, 0.f);
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int j = 0; j < GPW; ++j) h[r][j] = ring[((slot * 4 + r) * GPW + j) * 32];
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            const float4 d = dst[(m * tq + q) * 64 + quad_slot(lane, hf)];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              const cx<float> dv = k ? mk<float>(d.z, d.w) : mk<float>(d.x, d.y);
+#pragma unroll
+              for (int j = 0; j < GPW; ++j) {
+                const float4 hv = h[2 * hf + k][j];
+                mac(acc[j][0][m], hv.x, dv);
+                mac(acc[j][1][m], hv.y, dv);
+                mac(acc[j][2][m], hv.z, dv);
+                mac(acc[j][3][m], hv.w, dv);
+              }
+            }
+          }
+      }
+      slot = (slot + 1) % R;
+    }
+  }
+  if (tw > 1) {
+    cp_wait<0>();
+    __syncthreads();  // the staging buffers and rings are free
+    cx<float>* red = reinterpret_cast<cx<float>*>(smem_raw);  // [(ti - 1) zw + zi][GPW 16][32]
+    if (ti > 0) {
+      cx<float>* r = red + ((ti - 1) * zw + zi) * (GPW * 16 * 32) + lane;
+#pragma unroll
+      for (int j = 0; j < GPW; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int m = 0; m < 4; ++m) r[((j * 4 + q) * 4 + m) * 32] = acc[j][q][m];
     }
     __syncthreads();
-    const int tn = min(kTC, nt - t0);
-    // 8 samples per step: their GPW x 8 table loads are issued together
-    for (int tt = 0; tt < tn; tt += 8) {
-      float4 h[8][GPW];
+    if (ti == 0)
+      for (int k = 1; k < tw; ++k) {
+        const cx<float>* r = red + ((k - 1) * zw + zi) * (GPW * 16 * 32) + lane;
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
-#pragma unroll
-        for (int j = 0; j < GPW; ++j) {
-          const int g = gbase + j * kWarps;
-          h[r][j] = (g < nzg && tt + r < tn)
-                        ? ld_stream(tb + ((int64_t)(t0 + tt + r) * nzg + g) * 32)
-                        : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        cx<float> d[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) d[m] = ds[(tt + r) & (kTC - 1)][m][lane];
-#pragma unroll
-        for (int j = 0; j < GPW; ++j) {
-          const float hq[4] = {h[r][j].x, h[r][j].y, h[r][j].z, h[r][j].w};
+        for (int j = 0; j < GPW; ++j)
 #pragma unroll
           for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int m = 0; m < 4; ++m) mac(acc[j][q][m], hq[q], d[m]);
-        }
+            for (int m = 0; m < 4; ++m)
+              acc[j][q][m] = cadd(acc[j][q][m], r[((j * 4 + q) * 4 + m) * 32]);
       }
-    }
   }
+  if (ti != 0) return;
+  cx<float>* Zb = Z + b * vol_len<QUAD>(nz, Kpad);
 #pragma unroll
   for (int j = 0; j < GPW; ++j) {
-    const int g = gbase + j * kWarps;
+    const int g = gbase + j * zw;
+    if (g >= nzg) break;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int z = g * 4 + q;
-      if (g < nzg && z < nz) {
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-          if (bins[m] >= 0) Z[((int64_t)b * nz + z) * Kpad + bins[m]] = acc[j][q][m];
-      }
+    for (int m = 0; m < 4; ++m)
+      if (bins[m] >= 0)
+        store_quad<QUAD>(Zb, g, bins[m], nz, Kpad, acc[j][0][m], acc[j][1][m], acc[j][2][m],
+                         acc[j][3][m]);
+  }
+}
+
+constexpr size_t kSmemCta = 227 * 1024;  // most shared memory of a CTA (and of an SM's CTAs)
+
+template <bool QUAD, int T, int R>
+cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc, cudaStream_t s) {
+  const Layout& L = p.L;
+  constexpr size_t ring = (size_t)R * T * 512;  // bytes per warp
+  const size_t xbytes = (size_t)gc * 4096;
+  const bool two = 2 * (xbytes + 8 * ring) <= kSmemCta;
+  const int nwarps = two ? 8 : (int)std::min<size_t>(16, (kSmemCta - xbytes) / ring);
+  const size_t smem = xbytes + nwarps * ring;
+  auto fn = k_fold_fwd<QUAD, T, R>;
+  cudaError_t e = cudaFuncSetAttribute((const void*)fn,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // Splits of the time blocks over CTAs, by waves of CTAs x (blocks of the
+  // busiest warp + the CTA's load of its SM + its prologue): the order of the
+  // measured times at 71 to 1059 blocks (64^2: 10.1 us in 2, 16 in 1; 128^2:
+  // 93 us in 1, 99 in 2; 5 volumes at 64^2: 35 us in 2, 39 in 1).
+  const int nb = (L.nt + T - 1) / T, slots = two ? (int)kFoldCtas : (int)kFoldCtas / 2;
+  const int64_t ctas = L.nrb * batch;
+  int tb = nb;
+  double best = 1e300;
+  for (int split = 1; split <= 8; split *= 2) {
+    const int n = (nb + split - 1) / split, parts = (nb + n - 1) / n;
+    const double cost = (double)((ctas * parts + slots - 1) / slots) *
+                        ((n + nwarps - 1) / nwarps + 0.1 * n + 0.5);
+    if (cost < best) {
+      best = cost;
+      tb = n;
     }
   }
+  dim3 grid((unsigned)batch, (unsigned)L.nrb, (unsigned)((nb + tb - 1) / tb));
+  return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
+                    reinterpret_cast<const int4*>(p.rb_members),
+                    static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(X),
+                    static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad, tb, gc);
 }
 
+template <bool QUAD>
 cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s) {
   const Layout& L = p.L;
-  const size_t smem = sizeof(cx<float>) * 4 * (size_t)L.nzg * 4 * 32;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_fold_fwd,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  dim3 grid((unsigned)L.nrb, (unsigned)batch);
-  return launch_pdl(k_fold_fwd, grid, dim3(kWarps * 32), smem, s,
-                    static_cast<const float4*>(p.table), reinterpret_cast<const int4*>(p.rb_members),
-                    static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(X),
-                    static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad);
+  if ((size_t)L.nzg * 4096 > kSmemCta) return cudaErrorInvalidValue;  // more than 224 depths
+  // the spectra of up to 128 depths are resident at a time, more take another pass
+  const int gc = std::min(L.nzg, 32);
+  // Blocks of 8 samples read the spectra half as often as blocks of 4, but
+  // their ring leaves room for two CTAs per SM only up to 48 depths (three
+  // volumes at 96^2 x 45: 78 against 84 us); at 64 depths two CTAs with
+  // blocks of 4 are faster than one of 16 warps with blocks of 8 (93 / 101 us).
+  if (2 * ((size_t)gc * 4096 + 64 * 1024) <= kSmemCta)
+    return fold_fwd_t<QUAD, 8, 2>(p, X, Y, batch, gc, s);
+  return fold_fwd_t<QUAD, 4, 3>(p, X, Y, batch, gc, s);
 }
 
+template <bool QUAD, int GPW, int SQ, int R>
+cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw, int tw,
+                       cudaStream_t s) {
+  const Layout& L = p.L;
+  const int nzc = (L.nzg + zw * GPW - 1) / (zw * GPW), nwarps = zw * tw;
+  const size_t ring = (size_t)nwarps * R * 4 * GPW * 512;
+  const size_t smem = std::max<size_t>(2 * 4096 * (size_t)SQ * tw + ring,
+                                       (size_t)(tw - 1) * zw * GPW * 4096);
+  auto fn = k_fold_adj<QUAD, GPW, SQ, R>;
+  cudaError_t e = cudaFuncSetAttribute((const void*)fn,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  dim3 grid((unsigned)(nzc * batch), (unsigned)L.nrb);
+  return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
+                    reinterpret_cast<const int4*>(p.rb_members),
+                    static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(D),
+                    static_cast<cx<float>*>(Z), L.nz, L.nt, L.nzg, L.Kpad, nzc, zw, tw);
+}
+
+// Two z-groups per warp and up to 8 warps along z; fewer along z leave warps
+// for the time samples. Grids with less than about one CTA per SM split the
+// z-groups over more CTAs (64^2 x 32: 12.7 us in two, 17 in one; 32^2 x 16:
+// 5.7 us in four of one group per warp, 13 in one).
+template <bool QUAD>
 cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s) {
   const Layout& L = p.L;
-  constexpr int GPW = 2;
-  dim3 grid((unsigned)L.nrb, (unsigned)batch,
-            (unsigned)((L.nzg + kWarps * GPW - 1) / (kWarps * GPW)));
-  return launch_pdl(k_fold_adj<GPW>, grid, dim3(kWarps * 32), 0, s,
-                    static_cast<const float4*>(p.table), reinterpret_cast<const int4*>(p.rb_members),
-                    static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(D),
-                    static_cast<cx<float>*>(Z), L.nz, L.nt, L.nzg, L.Kpad);
+  const int64_t ctas = L.nrb * batch;
+  const int units = (L.nzg + 1) / 2;
+  int nzc = (units + 7) / 8;
+  int zw = (units + nzc - 1) / nzc;
+  while (zw > 1 && 2 * ctas * nzc <= 200) {
+    zw = (zw + 1) / 2;
+    nzc = (units + zw - 1) / zw;
+  }
+  if (zw == 1 && 2 * ctas * nzc <= 200) return fold_adj_t<QUAD, 1, 1, 4>(p, D, Z, batch, 1, 8, s);
+  static constexpr int kTw[8] = {8, 4, 2, 2, 1, 1, 1, 1};
+  const int tw = kTw[zw - 1];
+  return tw <= 2 ? fold_adj_t<QUAD, 2, 2, 2>(p, D, Z, batch, zw, tw, s)
+                 : fold_adj_t<QUAD, 2, 1, 2>(p, D, Z, batch, zw, tw, s);
 }
 
 template <typename R, bool CPLX, int VB>
@@ -479,19 +748,21 @@ cudaError_t launch_from_slots(const Plan& p, const void* in, void* out, int64_t 
   return cudaGetLastError();
 }
 
-cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s) {
+cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s,
+                                bool quad) {
   if (p.tc_fwd && p.tc_min_batch > 0 && batch >= p.tc_min_batch)
     return tc_contract(p, p.tc_fwd, p.tc_adj, X, Y, batch, false, p.tc_err, s);
-  if (p.L.fold) return fold_fwd(p, X, Y, batch, s);
+  if (p.L.fold) return quad ? fold_fwd<true>(p, X, Y, batch, s) : fold_fwd<false>(p, X, Y, batch, s);
   if (p.L.fp64)
     return p.L.real ? fwd_vb<double, false>(p, X, Y, batch, s) : fwd_vb<double, true>(p, X, Y, batch, s);
   return p.L.real ? fwd_vb<float, false>(p, X, Y, batch, s) : fwd_vb<float, true>(p, X, Y, batch, s);
 }
 
-cudaError_t launch_contract_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s) {
+cudaError_t launch_contract_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s,
+                                bool quad) {
   if (p.tc_adj && p.tc_min_batch > 0 && batch >= p.tc_min_batch)
     return tc_contract(p, p.tc_fwd, p.tc_adj, D, Z, batch, true, p.tc_err, s);
-  if (p.L.fold) return fold_adj(p, D, Z, batch, s);
+  if (p.L.fold) return quad ? fold_adj<true>(p, D, Z, batch, s) : fold_adj<false>(p, D, Z, batch, s);
   if (p.L.fp64)
     return p.L.real ? adj_vb<double, false>(p, D, Z, batch, s) : adj_vb<double, true>(p, D, Z, batch, s);
   return p.L.real ? adj_vb<float, false>(p, D, Z, batch, s) : adj_vb<float, true>(p, D, Z, batch, s);

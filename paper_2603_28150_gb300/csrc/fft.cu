@@ -9,8 +9,7 @@ namespace {
 
 template <typename R>
 cudaError_t spectrum_t(const Plan& p, const R* in, int64_t in_stride, int nx_in, int ny_in,
-                       cx<R>* out, int64_t out_stride, int S, cudaStream_t st, Samp sm,
-                       const int* slot) {
+                       cx<R>* out, const SpecRow& sr, int S, cudaStream_t st, Samp sm) {
   const Layout& L = p.L;
   const int tstride = ny_in + (ny_in & 1);
   const int64_t tslice = (int64_t)(L.px / 2 + 1) * tstride;
@@ -24,8 +23,8 @@ cudaError_t spectrum_t(const Plan& p, const R* in, int64_t in_stride, int nx_in,
   };
   if ((e = row()) != cudaSuccess) return e;
   auto col = [&]() -> cudaError_t {
-    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_fwd(T, tstride, tslice, ny_in, L.px / 2 + 1, S, out, out_stride,
-                                        twy, st, slot)))
+    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_fwd(T, tstride, tslice, ny_in, L.px / 2 + 1, S, out, sr, twy,
+                                        st)))
   };
   return col();
 }
@@ -43,21 +42,21 @@ cudaError_t spectrum_rows_t(const Plan& p, const R* in, int64_t in_stride, int n
 }
 
 template <typename R>
-cudaError_t spectrum_cols_t(const Plan& p, int ny_in, cx<R>* out, int64_t out_stride, int S,
-                            cudaStream_t st, const int* slot) {
+cudaError_t spectrum_cols_t(const Plan& p, int ny_in, cx<R>* out, const SpecRow& sr, int S,
+                            cudaStream_t st) {
   const Layout& L = p.L;
   const int tstride = ny_in + (ny_in & 1);
   const int64_t tslice = (int64_t)(L.px / 2 + 1) * tstride;
   cx<R>* T = static_cast<cx<R>*>(p.T);
   const cx<R>* twy = static_cast<const cx<R>*>(p.twy);
-  PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_fwd(T, tstride, tslice, ny_in, L.px / 2 + 1, S, out, out_stride,
-                                      twy, st, slot)))
+  PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_fwd(T, tstride, tslice, ny_in, L.px / 2 + 1, S, out, sr, twy,
+                                      st)))
 }
 
 template <typename R>
-cudaError_t image_t(const Plan& p, const cx<R>* in, int64_t in_stride, R* out, int64_t out_stride,
+cudaError_t image_t(const Plan& p, const cx<R>* in, const SpecRow& sr, R* out, int64_t out_stride,
                     int S, const R* sub, double* sumsq, cudaStream_t st, int groups,
-                    double* group_sums, Samp sm, const int* slot) {
+                    double* group_sums, Samp sm) {
   const Layout& L = p.L;
   cx<R>* T = static_cast<cx<R>*>(p.T);
   const cx<R>* twx = static_cast<const cx<R>*>(p.twx);
@@ -67,8 +66,8 @@ cudaError_t image_t(const Plan& p, const cx<R>* in, int64_t in_stride, R* out, i
   const bool grouped = groups > 0 && group_sums != nullptr;
   double* partials = (sumsq || grouped) ? p.red : nullptr;
   auto col = [&]() -> cudaError_t {
-    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_inv(in, in_stride, L.px / 2 + 1, S, T, L.tstride, L.tslice, L.ny,
-                                        twy, st, slot)))
+    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_inv(in, sr, L.px / 2 + 1, S, T, L.tstride, L.tslice, L.ny,
+                                        twy, st)))
   };
   if ((e = col()) != cudaSuccess) return e;
   auto row = [&]() -> cudaError_t {
@@ -88,10 +87,9 @@ cudaError_t image_t(const Plan& p, const cx<R>* in, int64_t in_stride, R* out, i
 // residual row pass in place, column forward pass into out; ||r||^2 summed as
 // image_t does.
 template <typename R>
-cudaError_t residual_t(const Plan& p, const cx<R>* in, int64_t in_stride, const R* y,
+cudaError_t residual_t(const Plan& p, const cx<R>* in, const SpecRow& sr, const R* y,
                        int64_t y_stride, int S, double* sumsq, cudaStream_t st, int groups,
-                       double* group_sums, Samp sm, const int* slot, cx<R>* out,
-                       int64_t out_stride) {
+                       double* group_sums, Samp sm, cx<R>* out) {
   const Layout& L = p.L;
   cx<R>* T = static_cast<cx<R>*>(p.T);
   const cx<R>* twx = static_cast<const cx<R>*>(p.twx);
@@ -101,8 +99,8 @@ cudaError_t residual_t(const Plan& p, const cx<R>* in, int64_t in_stride, const 
   const bool grouped = groups > 0 && group_sums != nullptr;
   double* partials = (sumsq || grouped) ? p.red : nullptr;
   auto col = [&]() -> cudaError_t {
-    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_inv(in, in_stride, L.px / 2 + 1, S, T, L.tstride, L.tslice, L.ny,
-                                        twy, st, slot)))
+    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_inv(in, sr, L.px / 2 + 1, S, T, L.tstride, L.tslice, L.ny,
+                                        twy, st)))
   };
   if ((e = col()) != cudaSuccess) return e;
   auto row = [&]() -> cudaError_t {
@@ -117,23 +115,23 @@ cudaError_t residual_t(const Plan& p, const cx<R>* in, int64_t in_stride, const 
                      cudaSuccess)
     return e;
   auto colf = [&]() -> cudaError_t {
-    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_fwd(T, L.tstride, L.tslice, L.ny, L.px / 2 + 1, S, out,
-                                        out_stride, twy, st, slot)))
+    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_fwd(T, L.tstride, L.tslice, L.ny, L.px / 2 + 1, S, out, sr,
+                                        twy, st)))
   };
   return colf();
 }
 
 template <typename R>
-cudaError_t image_step_t(const Plan& p, const cx<R>* in, int64_t in_stride, int S,
-                         const FistaStep& f, cudaStream_t st, const int* slot) {
+cudaError_t image_step_t(const Plan& p, const cx<R>* in, const SpecRow& sr, int S,
+                         const FistaStep& f, cudaStream_t st) {
   const Layout& L = p.L;
   cx<R>* T = static_cast<cx<R>*>(p.T);
   const cx<R>* twx = static_cast<const cx<R>*>(p.twx);
   const cx<R>* twy = static_cast<const cx<R>*>(p.twy);
   cudaError_t e;
   auto col = [&]() -> cudaError_t {
-    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_inv(in, in_stride, L.px / 2 + 1, S, T, L.tstride, L.tslice, L.ny,
-                                        twy, st, slot)))
+    PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_inv(in, sr, L.px / 2 + 1, S, T, L.tstride, L.tslice, L.ny,
+                                        twy, st)))
   };
   if ((e = col()) != cudaSuccess) return e;
   const int64_t plane = (int64_t)L.ny * L.nx;
@@ -154,60 +152,55 @@ cudaError_t launch_spectrum_rows(const Plan& p, const void* in, int64_t in_strid
   return spectrum_rows_t<float>(p, static_cast<const float*>(in), in_stride, nx_in, ny_in, S, s);
 }
 
-cudaError_t launch_spectrum_cols(const Plan& p, int ny_in, void* out, int64_t out_stride, int S,
-                                 cudaStream_t s, const int* slot) {
+cudaError_t launch_spectrum_cols(const Plan& p, int ny_in, void* out, const SpecRow& sr, int S,
+                                 cudaStream_t s) {
   if (S <= 0) return cudaSuccess;
-  if (p.L.fp64)
-    return spectrum_cols_t<double>(p, ny_in, static_cast<cx<double>*>(out), out_stride, S, s, slot);
-  return spectrum_cols_t<float>(p, ny_in, static_cast<cx<float>*>(out), out_stride, S, s, slot);
+  if (p.L.fp64) return spectrum_cols_t<double>(p, ny_in, static_cast<cx<double>*>(out), sr, S, s);
+  return spectrum_cols_t<float>(p, ny_in, static_cast<cx<float>*>(out), sr, S, s);
 }
 
-cudaError_t launch_image_step(const Plan& p, const void* in, int64_t in_stride, int S,
-                              const FistaStep& f, cudaStream_t s, const int* slot) {
+cudaError_t launch_image_step(const Plan& p, const void* in, const SpecRow& sr, int S,
+                              const FistaStep& f, cudaStream_t s) {
   if (S <= 0) return cudaSuccess;
   if (p.L.fp64)
-    return image_step_t<double>(p, static_cast<const cx<double>*>(in), in_stride, S, f, s, slot);
-  return image_step_t<float>(p, static_cast<const cx<float>*>(in), in_stride, S, f, s, slot);
+    return image_step_t<double>(p, static_cast<const cx<double>*>(in), sr, S, f, s);
+  return image_step_t<float>(p, static_cast<const cx<float>*>(in), sr, S, f, s);
 }
 
-cudaError_t launch_residual(const Plan& p, const void* in, int64_t in_stride, const void* y,
+cudaError_t launch_residual(const Plan& p, const void* in, const SpecRow& sr, const void* y,
                             int64_t y_stride, int S, double* sumsq, cudaStream_t s, int groups,
-                            double* group_sums, Samp sm, const int* slot, void* out,
-                            int64_t out_stride) {
+                            double* group_sums, Samp samp, void* out) {
   if (S <= 0) return cudaSuccess;
   if (p.L.fp64)
-    return residual_t<double>(p, static_cast<const cx<double>*>(in), in_stride,
+    return residual_t<double>(p, static_cast<const cx<double>*>(in), sr,
                               static_cast<const double*>(y), y_stride, S, sumsq, s, groups,
-                              group_sums, sm, slot, static_cast<cx<double>*>(out), out_stride);
-  return residual_t<float>(p, static_cast<const cx<float>*>(in), in_stride,
-                           static_cast<const float*>(y), y_stride, S, sumsq, s, groups, group_sums,
-                           sm, slot, static_cast<cx<float>*>(out), out_stride);
+                              group_sums, samp, static_cast<cx<double>*>(out));
+  return residual_t<float>(p, static_cast<const cx<float>*>(in), sr, static_cast<const float*>(y),
+                           y_stride, S, sumsq, s, groups, group_sums, samp,
+                           static_cast<cx<float>*>(out));
 }
 
 cudaError_t launch_spectrum(const Plan& p, const void* in, int64_t in_stride, int nx_in, int ny_in,
-                            void* out, int64_t out_stride, int S, cudaStream_t s, Samp sm,
-                            const int* slot) {
+                            void* out, const SpecRow& sr, int S, cudaStream_t s, Samp samp) {
   if (S <= 0) return cudaSuccess;
   if (p.L.fp64)
     return spectrum_t<double>(p, static_cast<const double*>(in), in_stride, nx_in, ny_in,
-                              static_cast<cx<double>*>(out), out_stride, S, s, sm, slot);
+                              static_cast<cx<double>*>(out), sr, S, s, samp);
   return spectrum_t<float>(p, static_cast<const float*>(in), in_stride, nx_in, ny_in,
-                           static_cast<cx<float>*>(out), out_stride, S, s, sm, slot);
+                           static_cast<cx<float>*>(out), sr, S, s, samp);
 }
 
-cudaError_t launch_image(const Plan& p, const void* in, int64_t in_stride, void* out,
+cudaError_t launch_image(const Plan& p, const void* in, const SpecRow& sr, void* out,
                          int64_t out_stride, int S, const void* sub, double* sumsq,
-                         cudaStream_t s, int groups, double* group_sums, Samp sm,
-                         const int* slot) {
+                         cudaStream_t s, int groups, double* group_sums, Samp samp) {
   if (S <= 0) return cudaSuccess;
   if (p.L.fp64)
-    return image_t<double>(p, static_cast<const cx<double>*>(in), in_stride,
-                           static_cast<double*>(out), out_stride, S,
-                           static_cast<const double*>(sub), sumsq, s, groups, group_sums, sm,
-                           slot);
-  return image_t<float>(p, static_cast<const cx<float>*>(in), in_stride, static_cast<float*>(out),
+    return image_t<double>(p, static_cast<const cx<double>*>(in), sr, static_cast<double*>(out),
+                           out_stride, S, static_cast<const double*>(sub), sumsq, s, groups,
+                           group_sums, samp);
+  return image_t<float>(p, static_cast<const cx<float>*>(in), sr, static_cast<float*>(out),
                         out_stride, S, static_cast<const float*>(sub), sumsq, s, groups,
-                        group_sums, sm, slot);
+                        group_sums, samp);
 }
 
 }  // namespace pat

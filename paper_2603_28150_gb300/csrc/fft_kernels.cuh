@@ -56,7 +56,14 @@ struct Shape {
   // padded vector stride: the extra element puts consecutive vectors in
   // different banks for the transposed (vector-major) accesses of the row kernels
   static constexpr int VSTR = P + P / 16 + 1;
+  // stride of a column kernel on quad spectra, whose neighbouring threads are
+  // four slices by consecutive elements: 4 (mod 8) elements apart, so four
+  // slices x four elements touch the 16 8-byte banks once
+  static constexpr int VSTR_Q = (P + P / 16 + 3) / 8 * 8 + 4;
 };
+
+// Column kernels on the three spectrum layouts of SpecRow.
+enum { kRows = 0, kSlots = 1, kQuads = 2 };
 
 // Radix of pass S and the product of the radices before it.
 template <int P, int S>
@@ -389,9 +396,10 @@ __device__ __forceinline__ cx<R>* setup_smem(const cx<R>* tw_g, cx<R>** tw_s) {
   return tw + TP::N;
 }
 
-template <typename R, int P>
+template <typename R, int P, int MODE = kRows>
 constexpr size_t smem_bytes() {
-  return sizeof(cx<R>) * (size_t)(TwPlan<P>::N + Shape<P>::VPB * Shape<P>::VSTR);
+  return sizeof(cx<R>) * (size_t)(TwPlan<P>::N + Shape<P>::VPB * (MODE == kQuads ? Shape<P>::VSTR_Q
+                                                                                 : Shape<P>::VSTR));
 }
 
 // Compact index of sensor coordinate c on a scan axis (offset o, stride st,
@@ -605,34 +613,74 @@ __device__ __forceinline__ void slot_store_pair(cx<R>* dst, int s0, int s1, cx<R
   }
 }
 
+// The column (slice s, kx) of each of a block's vectors, and where its
+// spectrum lives. Rows and slots: consecutive vectors are consecutive columns,
+// a vector's threads are neighbours. Quads: the block holds the four slices of
+// VPB / 4 columns, and four neighbouring threads hold one element of the four
+// slices (one 32-byte sector).
+template <typename R, int P, int MODE>
+struct ColMap {
+  using SH = Shape<P>;
+  static constexpr int VS = MODE == kQuads ? SH::VSTR_Q : SH::VSTR;
+  int v, tid;
+  bool ok;
+  int64_t s, kx;
+  int64_t base;  // offset of element 0 (rows, quads) or of the slice's row (slots)
+  static constexpr int STEP = MODE == kQuads ? 4 : 1;
+  __device__ __forceinline__ ColMap(int ncols, int64_t nvec, int64_t stride, int quad) {
+    // 32-bit quotients (slices x columns < 2^31): no 64-bit division
+    if constexpr (MODE == kQuads) {
+      const int sl = threadIdx.x & 3, c = threadIdx.x / (4 * SH::TPV);
+      tid = (threadIdx.x >> 2) % SH::TPV;
+      v = 4 * c + sl;
+      const unsigned g = blockIdx.x * (SH::VPB / 4) + c;  // (volume, quad, column)
+      const unsigned nq = (unsigned)(quad + 3) / 4;
+      const unsigned vq = g / (unsigned)ncols;
+      const unsigned vol = vq / nq;
+      const int sv = 4 * (int)(vq - vol * nq) + sl;  // slice within the volume
+      ok = g < nvec && sv < quad;
+      kx = ok ? (int64_t)(g - vq * (unsigned)ncols) : 0;
+      s = ok ? (int64_t)vol * quad + sv : 0;
+      base = ok ? ((int64_t)vq * stride + kx * P) * 4 + sl : 0;
+    } else {
+      v = threadIdx.x / SH::TPV;
+      tid = threadIdx.x % SH::TPV;
+      const unsigned g = blockIdx.x * SH::VPB + v;
+      ok = g < nvec;
+      const unsigned gq = ok ? g / (unsigned)ncols : 0u;
+      s = gq;
+      kx = ok ? (int64_t)(g - gq * (unsigned)ncols) : 0;
+      base = s * stride + (MODE == kRows ? kx * P : 0);
+    }
+  }
+};
+
 // Stage i, column pass: T[s][kx][0..n_in) zero-padded to P, FFT over y,
-// written to out[s][kx][0..P) (slice stride out_stride), or with `slot` to
+// written to the spectrum `out` (row stride out_stride); with kSlots to
 // out[s][slot[kx * P + ky]] (the representative-slot layout; the transform
 // then lands in the work vector and leaves as mirror pairs).
-template <typename R, int P, bool SLOT, bool ZIN>
+template <typename R, int P, int MODE, bool ZIN>
 __global__ void __launch_bounds__(kThreads) k_col_fwd(const cx<R>* __restrict__ T, int tstride,
                                                       int64_t tslice, int n_in, int ncols,
                                                       int64_t nvec, cx<R>* __restrict__ out,
-                                                      int64_t out_stride,
+                                                      int64_t out_stride, int quad,
                                                       const cx<R>* __restrict__ tw_g,
                                                       const int* __restrict__ slot) {
   using SH = Shape<P>;
+  using CM = ColMap<R, P, MODE>;
   cx<R>* tw;
   cx<R>* bufs = setup_smem<R, P>(tw_g, &tw);
-  const int v = threadIdx.x / SH::TPV, tid = threadIdx.x % SH::TPV;
-  const int64_t g = (int64_t)blockIdx.x * SH::VPB + v;
-  const bool ok = g < nvec;
-  // 32-bit quotient (nvec = slices x columns < 2^31): no 64-bit division
-  const unsigned gq = ok ? (unsigned)g / (unsigned)ncols : 0u;
-  const int64_t s = gq, kx = ok ? (int64_t)((unsigned)g - gq * (unsigned)ncols) : 0;
-  const cx<R>* src = T + s * tslice + kx * tstride;
-  cx<R>* dst = out + s * out_stride;
-  const int* sl = SLOT ? slot + kx * P : nullptr;
+  const CM c(ncols, nvec, out_stride, quad);
+  const bool ok = c.ok;
+  const int tid = c.tid;
+  const cx<R>* src = T + c.s * tslice + c.kx * tstride;
+  cx<R>* dst = out + c.base;
+  cx<R>* b = bufs + c.v * CM::VS;
   pdl_wait();
   __syncthreads();
   auto ld = [&](int y) -> cx<R> { return (ok && y < n_in) ? src[y] : mk<R>(0, 0); };
-  if constexpr (SLOT) {
-    cx<R>* b = bufs + v * SH::VSTR;
+  if constexpr (MODE == kSlots) {
+    const int* sl = slot + c.kx * P;
     NoStore<R> ns;
     run_passes<R, P, 0, false, true, false, ZIN>(b, tw, tid, ld, ns);  // ends with a barrier
     if (ok) {
@@ -650,44 +698,40 @@ __global__ void __launch_bounds__(kThreads) k_col_fwd(const cx<R>* __restrict__ 
     }
   } else {
     auto st = [&](int y, cx<R> val) {
-      if (ok) dst[kx * P + y] = val;
+      if (ok) dst[y * CM::STEP] = val;
     };
-    run_passes<R, P, 0, false, true, true, ZIN>(bufs + v * SH::VSTR, tw, tid, ld, st);
+    run_passes<R, P, 0, false, true, true, ZIN>(b, tw, tid, ld, st);
   }
 }
 
-// Stage iii, column pass: in[s][kx][0..P) (or with `slot`, in[s][slot[kx * P +
-// ky]]) inverse FFT over ky, rows [0, n_out) kept (crop) into T[s][kx][y].
-template <typename R, int P, bool SLOT, bool HOUT>
+// Stage iii, column pass: the spectrum `in` inverse FFT over ky, rows
+// [0, n_out) kept (crop) into T[s][kx][y].
+template <typename R, int P, int MODE, bool HOUT>
 __global__ void __launch_bounds__(kThreads) k_col_inv(const cx<R>* __restrict__ in,
-                                                      int64_t in_stride, int ncols, int64_t nvec,
-                                                      cx<R>* __restrict__ T, int tstride,
-                                                      int64_t tslice, int n_out,
+                                                      int64_t in_stride, int quad, int ncols,
+                                                      int64_t nvec, cx<R>* __restrict__ T,
+                                                      int tstride, int64_t tslice, int n_out,
                                                       const cx<R>* __restrict__ tw_g,
                                                       const int* __restrict__ slot) {
-  using SH = Shape<P>;
+  using CM = ColMap<R, P, MODE>;
   cx<R>* tw;
   cx<R>* bufs = setup_smem<R, P>(tw_g, &tw);
-  const int v = threadIdx.x / SH::TPV, tid = threadIdx.x % SH::TPV;
-  const int64_t g = (int64_t)blockIdx.x * SH::VPB + v;
-  const bool ok = g < nvec;
-  // 32-bit quotient (nvec = slices x columns < 2^31): no 64-bit division
-  const unsigned gq = ok ? (unsigned)g / (unsigned)ncols : 0u;
-  const int64_t s = gq, kx = ok ? (int64_t)((unsigned)g - gq * (unsigned)ncols) : 0;
-  const cx<R>* src = in + s * in_stride;
-  const int* sl = SLOT ? slot + kx * P : nullptr;
-  cx<R>* dst = T + s * tslice + kx * tstride;
+  const CM c(ncols, nvec, in_stride, quad);
+  const bool ok = c.ok;
+  const cx<R>* src = in + c.base;
+  const int* sl = MODE == kSlots ? slot + c.kx * P : nullptr;
+  cx<R>* dst = T + c.s * tslice + c.kx * tstride;
   pdl_wait();
   __syncthreads();
   auto ld = [&](int y) -> cx<R> {
-    return ok ? src[SLOT ? __ldg(sl + y) : kx * P + y] : mk<R>(0, 0);
+    return ok ? src[MODE == kSlots ? __ldg(sl + y) : y * CM::STEP] : mk<R>(0, 0);
   };
   auto st = [&](int y, cx<R> val) {
     if (ok && y < n_out) dst[y] = val;
   };
   // (slot-mapped columns load element by element here: gathering mirror
   // pairs as 16-byte loads through the work vector measured slower)
-  run_passes<R, P, 0, true, true, true, false, HOUT>(bufs + v * SH::VSTR, tw, tid, ld, st);
+  run_passes<R, P, 0, true, true, true, false, HOUT>(bufs + c.v * CM::VS, tw, c.tid, ld, st);
 }
 
 // Stage iii row pass, first half: the half spectra A = T[kx][y0], B =
@@ -1034,35 +1078,61 @@ cudaError_t FftLen<R, P>::row_r2c(const R* in, int64_t in_stride, int nx_in, int
                     T, tstride, tslice, tw, sm);
 }
 
-template <typename R, int P>
-cudaError_t FftLen<R, P>::col_fwd(const cx<R>* T, int tstride, int64_t tslice, int n_in, int ncols, int S,
-                                  cx<R>* out, int64_t out_stride, const cx<R>* tw, cudaStream_t st,
-                                  const int* slot) {
+namespace {
+template <typename R, int P, int MODE>
+cudaError_t col_fwd_t(const cx<R>* T, int tstride, int64_t tslice, int n_in, int ncols, int S,
+                      cx<R>* out, const SpecRow& sr, const cx<R>* tw, cudaStream_t st) {
   using SH = Shape<P>;
   const bool zin = 2 * n_in <= P;
-  auto fn = slot ? (zin ? k_col_fwd<R, P, true, true> : k_col_fwd<R, P, true, false>)
-                 : (zin ? k_col_fwd<R, P, false, true> : k_col_fwd<R, P, false, false>);
-  cudaError_t e = set_smem_attr<R, P>((const void*)fn);
+  auto fn = zin ? k_col_fwd<R, P, MODE, true> : k_col_fwd<R, P, MODE, false>;
+  constexpr size_t smem = smem_bytes<R, P, MODE>();
+  cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
   if (e != cudaSuccess) return e;
-  const int64_t nvec = (int64_t)S * ncols;
-  const int64_t blocks = (nvec + SH::VPB - 1) / SH::VPB;
-  return launch_pdl(fn, dim3((unsigned)blocks), dim3(kThreads), smem_bytes<R, P>(), st,
-                    T, tstride, tslice, n_in, ncols, nvec, out, out_stride, tw, slot);
+  // quads: units of four slices (the last of a volume may hold fewer)
+  const int64_t units = MODE == kQuads ? (int64_t)(S / sr.quad) * ((sr.quad + 3) / 4) : S;
+  constexpr int per = MODE == kQuads ? SH::VPB / 4 : SH::VPB;
+  const int64_t nvec = units * ncols, blocks = (nvec + per - 1) / per;
+  return launch_pdl(fn, dim3((unsigned)blocks), dim3(kThreads), smem, st, T, tstride, tslice, n_in,
+                    ncols, nvec, out, sr.stride, sr.quad, tw, sr.slot);
+}
+
+template <typename R, int P, int MODE>
+cudaError_t col_inv_t(const cx<R>* in, const SpecRow& sr, int ncols, int S, cx<R>* T, int tstride,
+                      int64_t tslice, int n_out, const cx<R>* tw, cudaStream_t st) {
+  using SH = Shape<P>;
+  const bool hout = 2 * n_out <= P;  // rows [P/2, P) are cropped away
+  auto fn = hout ? k_col_inv<R, P, MODE, true> : k_col_inv<R, P, MODE, false>;
+  constexpr size_t smem = smem_bytes<R, P, MODE>();
+  cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  const int64_t units = MODE == kQuads ? (int64_t)(S / sr.quad) * ((sr.quad + 3) / 4) : S;
+  constexpr int per = MODE == kQuads ? SH::VPB / 4 : SH::VPB;
+  const int64_t nvec = units * ncols, blocks = (nvec + per - 1) / per;
+  return launch_pdl(fn, dim3((unsigned)blocks), dim3(kThreads), smem, st, in, sr.stride, sr.quad,
+                    ncols, nvec, T, tstride, tslice, n_out, tw, sr.slot);
+}
+}  // namespace
+
+template <typename R, int P>
+cudaError_t FftLen<R, P>::col_fwd(const cx<R>* T, int tstride, int64_t tslice, int n_in, int ncols, int S,
+                                  cx<R>* out, const SpecRow& sr, const cx<R>* tw, cudaStream_t st) {
+  if constexpr (sizeof(R) == 4) {  // double-precision plans do not fold
+    if (sr.quad) return col_fwd_t<R, P, kQuads>(T, tstride, tslice, n_in, ncols, S, out, sr, tw, st);
+  }
+  return sr.slot ? col_fwd_t<R, P, kSlots>(T, tstride, tslice, n_in, ncols, S, out, sr, tw, st)
+                 : col_fwd_t<R, P, kRows>(T, tstride, tslice, n_in, ncols, S, out, sr, tw, st);
 }
 
 template <typename R, int P>
-cudaError_t FftLen<R, P>::col_inv(const cx<R>* in, int64_t in_stride, int ncols, int S, cx<R>* T, int tstride,
-                                  int64_t tslice, int n_out, const cx<R>* tw, cudaStream_t st, const int* slot) {
-  using SH = Shape<P>;
-  const bool hout = 2 * n_out <= P;  // rows [P/2, P) are cropped away
-  auto fn = slot ? (hout ? k_col_inv<R, P, true, true> : k_col_inv<R, P, true, false>)
-                 : (hout ? k_col_inv<R, P, false, true> : k_col_inv<R, P, false, false>);
-  cudaError_t e = set_smem_attr<R, P>((const void*)fn);
-  if (e != cudaSuccess) return e;
-  const int64_t nvec = (int64_t)S * ncols;
-  const int64_t blocks = (nvec + SH::VPB - 1) / SH::VPB;
-  return launch_pdl(fn, dim3((unsigned)blocks), dim3(kThreads), smem_bytes<R, P>(), st,
-                    in, in_stride, ncols, nvec, T, tstride, tslice, n_out, tw, slot);
+cudaError_t FftLen<R, P>::col_inv(const cx<R>* in, const SpecRow& sr, int ncols, int S, cx<R>* T, int tstride,
+                                  int64_t tslice, int n_out, const cx<R>* tw, cudaStream_t st) {
+  if constexpr (sizeof(R) == 4) {
+    if (sr.quad) return col_inv_t<R, P, kQuads>(in, sr, ncols, S, T, tstride, tslice, n_out, tw, st);
+  }
+  return sr.slot ? col_inv_t<R, P, kSlots>(in, sr, ncols, S, T, tstride, tslice, n_out, tw, st)
+                 : col_inv_t<R, P, kRows>(in, sr, ncols, S, T, tstride, tslice, n_out, tw, st);
 }
 
 template <typename R, int P>

@@ -11,13 +11,12 @@ struct FftLen {
   // stage i row pass: real rows of in -> half spectra T[s][kx][y]
   static cudaError_t row_r2c(const R* in, int64_t in_stride, int nx_in, int ny_in, cx<R>* T, int tstride,
                              int64_t tslice, int S, const cx<R>* tw, cudaStream_t st, Samp sm);
-  // stage i column pass: T -> X[s][kx][ky] (or the slot layout with `slot`)
+  // stage i column pass: T -> the spectrum `out` laid out as `sr` says
   static cudaError_t col_fwd(const cx<R>* T, int tstride, int64_t tslice, int n_in, int ncols, int S,
-                             cx<R>* out, int64_t out_stride, const cx<R>* tw, cudaStream_t st,
-                             const int* slot);
+                             cx<R>* out, const SpecRow& sr, const cx<R>* tw, cudaStream_t st);
   // stage iii column pass: spectrum -> T, rows cropped to n_out
-  static cudaError_t col_inv(const cx<R>* in, int64_t in_stride, int ncols, int S, cx<R>* T, int tstride,
-                             int64_t tslice, int n_out, const cx<R>* tw, cudaStream_t st, const int* slot);
+  static cudaError_t col_inv(const cx<R>* in, const SpecRow& sr, int ncols, int S, cx<R>* T, int tstride,
+                             int64_t tslice, int n_out, const cx<R>* tw, cudaStream_t st);
   // stage iii row pass: T -> real image (optionally minus `sub`, squares summed)
   static cudaError_t row_c2r(const cx<R>* T, int tstride, int64_t tslice, int nx_out, int ny_out, R* out,
                              int64_t out_stride, int S, const R* sub, double* partials, const cx<R>* tw,

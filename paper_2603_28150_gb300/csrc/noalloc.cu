@@ -127,8 +127,10 @@ extern "C" int pat_spectrum_noalloc(const float* in, int nx, int ny, int px, int
     view.T = s->scratch;
     view.twx = s->twiddles + twiddle_offset(px);
     view.twy = s->twiddles + twiddle_offset(py);
-    PAT_CUDA(launch_spectrum(view, in, (int64_t)nx * ny, nx, ny, out,
-                             (int64_t)(px / 2 + 1) * py, slices, (cudaStream_t)stream));
+    SpecRow sr;
+    sr.stride = (int64_t)(px / 2 + 1) * py;
+    PAT_CUDA(launch_spectrum(view, in, (int64_t)nx * ny, nx, ny, out, sr, slices,
+                             (cudaStream_t)stream));
     return PAT_OK;
   } catch (...) {
     return fail(PAT_ERR_CUDA, "unexpected internal error");

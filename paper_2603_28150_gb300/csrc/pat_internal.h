@@ -175,7 +175,7 @@ struct Plan {
   void* twx = nullptr;    // device cx<real_t>[px]: exp(-2 pi i k / px)
   void* twy = nullptr;    // device cx<real_t>[py]
   // workspace (device)
-  void* X = nullptr;      // [max_batch][max(nz, nt)][Kpad] complex  (X or Z or D)
+  void* X = nullptr;      // [max_batch][max(nz, nt)][Kpad] complex  (X or Z or D; see SpecRow)
   void* Y = nullptr;      // [max_batch][max(nz, nt)][Kpad] complex  (Y or D or Z)
   void* T = nullptr;      // [max_batch * max(nz, nt)][tslice] complex
   void* vol_a = nullptr;  // [max_batch][nz][ny][nx] real: FISTA momentum point y_k
@@ -317,28 +317,38 @@ int cuda_fail(cudaError_t e, const char* what);
 // ----------------------------------------------------------------------------
 // Launchers (each returns cudaError_t of the launch).
 // ----------------------------------------------------------------------------
+// Where the spectra of a run of slices live: one row of `stride` complex
+// values per slice (bin k at k, or at slot[k] with `slot`), or with quad > 0
+// (slices per volume) four slices interleaved: volume v's slice s, bin k at
+// ((v ceil(quad / 4) + s / 4) stride + k) 4 + s % 4. A bin's four slices are
+// then one 32-byte sector, which the contraction of a folded table needs (its
+// bins are scattered), and a column of four slices stays contiguous.
+struct SpecRow {
+  int64_t stride = 0;
+  const int* slot = nullptr;
+  int quad = 0;
+};
 // FFT stages. `in`/`out` element type follows L.fp64.
 // Stage i: real slices [S][ny][nx] (slice stride in_stride elements, row
 // length nx_in valid of px, ny_in valid rows of py) -> spectra [S][px/2+1][py]
-// with slice stride out_stride complex elements.
+// laid out as `sr` says.
 cudaError_t launch_spectrum(const Plan& p, const void* in, int64_t in_stride, int nx_in, int ny_in,
-                            void* out, int64_t out_stride, int S, cudaStream_t s,
-                            Samp samp = no_sampling(), const int* slot = nullptr);
+                            void* out, const SpecRow& sr, int S, cudaStream_t s,
+                            Samp samp = no_sampling());
 // Stage iii: spectra [S][px/2+1][py] -> real [S][ny][nx] (crop), optionally
 // out = image - sub (sub has out's layout) with sum of squares added to
 // *sumsq (FP64, via the plan's reduction scratch when sumsq != nullptr).
-cudaError_t launch_image(const Plan& p, const void* in, int64_t in_stride, void* out,
+cudaError_t launch_image(const Plan& p, const void* in, const SpecRow& sr, void* out,
                          int64_t out_stride, int S, const void* sub, double* sumsq,
                          cudaStream_t s, int groups = 0, double* group_sums = nullptr,
-                         Samp samp = no_sampling(), const int* slot = nullptr);
+                         Samp samp = no_sampling());
 // Stage iii then stage i on the data side of the gradient (Eq. 15): spectra
-// of H x (rows of in_stride) -> spectra of r = S H x - y (rows of out_stride;
-// out may be in), y [S][my][mx] with slice stride y_stride; ||r||^2 as in
-// launch_image. The residual image is never stored.
-cudaError_t launch_residual(const Plan& p, const void* in, int64_t in_stride, const void* y,
+// of H x -> spectra of r = S H x - y (both laid out as `sr` says; out may be
+// in), y [S][my][mx] with slice stride y_stride; ||r||^2 as in launch_image.
+// The residual image is never stored.
+cudaError_t launch_residual(const Plan& p, const void* in, const SpecRow& sr, const void* y,
                             int64_t y_stride, int S, double* sumsq, cudaStream_t s, int groups,
-                            double* group_sums, Samp samp, const int* slot, void* out,
-                            int64_t out_stride);
+                            double* group_sums, Samp samp, void* out);
 // FISTA step (Eq. 14-15) fused into the last stage of the gradient: with g =
 // H*(S H y_k - d) at a voxel, x_k = max(y_k - g/L - lambda/L, 0) and
 // y_{k+1} = x_k + beta_k (x_k - x_{k-1}), scal = {1/L, lambda/L}, beta_k =
@@ -360,18 +370,21 @@ struct FistaStep {
 };
 // Stage iii over the depth slices of `S` = batch * nz spectra with the FISTA
 // step in place of the gradient store.
-cudaError_t launch_image_step(const Plan& p, const void* in, int64_t in_stride, int S,
-                              const FistaStep& f, cudaStream_t s, const int* slot);
+cudaError_t launch_image_step(const Plan& p, const void* in, const SpecRow& sr, int S,
+                              const FistaStep& f, cudaStream_t s);
 // Stage i split in its two passes: rows of the real slices into the plan's T,
 // and the column pass from T (launch_spectrum runs both).
 cudaError_t launch_spectrum_rows(const Plan& p, const void* in, int64_t in_stride, int nx_in,
                                  int ny_in, int S, cudaStream_t s);
-cudaError_t launch_spectrum_cols(const Plan& p, int ny_in, void* out, int64_t out_stride, int S,
-                                 cudaStream_t s, const int* slot);
+cudaError_t launch_spectrum_cols(const Plan& p, int ny_in, void* out, const SpecRow& sr, int S,
+                                 cudaStream_t s);
 // Contractions over the resident table (tensor cores when the plan has the
-// split tables and batch >= tc_min_batch).
-cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s);
-cudaError_t launch_contract_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s);
+// split tables and batch >= tc_min_batch). quad: the spectra of a folded plan
+// on the CUDA cores are in quads (SpecRow), else one row of Kpad bins a slice.
+cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s,
+                                bool quad = false);
+cudaError_t launch_contract_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s,
+                                bool quad = false);
 
 // The batched tensor-core contraction of a folded plan reads and writes
 // spectra in the representative-slot layout (rows of 4 * Upad complex
@@ -380,6 +393,17 @@ inline bool tc_slots(const Plan& p, int batch) {
   return p.tc_fwd && p.L.fold && p.tc_min_batch > 0 && batch >= p.tc_min_batch;
 }
 inline int64_t slot_row(const Layout& L) { return 4 * L.Upad; }
+// Layout of the plan's own spectra of `n` slices per volume at this batch:
+// slots for the folded tensor-core path, quads for the folded CUDA-core path
+// (whole sectors for its scattered bins: see contract.cu), else rows of Kpad.
+inline SpecRow spec_row(const Plan& p, int batch, int n) {
+  SpecRow r;
+  const bool sl = tc_slots(p, batch);
+  r.stride = sl ? slot_row(p.L) : p.L.Kpad;
+  r.slot = sl ? p.fold_slot : nullptr;
+  r.quad = !sl && p.L.fold ? n : 0;
+  return r;
+}
 // [S][Kpad] bins -> [S][4 Upad] slots and back (single precision).
 cudaError_t launch_to_slots(const Plan& p, const void* in, void* out, int64_t S, cudaStream_t s);
 cudaError_t launch_from_slots(const Plan& p, const void* in, void* out, int64_t S,

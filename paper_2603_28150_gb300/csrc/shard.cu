@@ -293,8 +293,9 @@ int pat_shard_spectrum(pat_plan* plan, int side, const float* in, void* send, pa
     const Plan& p = plan->p;
     const Layout& L = p.L;
     const int n = (side ? L.nt : L.nz) / p.shard_world;
-    PAT_CUDA(launch_spectrum(p, in, (int64_t)L.ny * L.nx, L.nx, L.ny, send, p.shard_W, n,
-                             (cudaStream_t)stream, no_sampling(), side ? p.shard_tmap : p.shard_zmap));
+    const SpecRow sr{p.shard_W, side ? p.shard_tmap : p.shard_zmap, 0};
+    PAT_CUDA(launch_spectrum(p, in, (int64_t)L.ny * L.nx, L.nx, L.ny, send, sr, n,
+                             (cudaStream_t)stream));
     return PAT_OK;
   } catch (...) {
     return fail(PAT_ERR_CUDA, "unexpected internal error");
@@ -347,8 +348,8 @@ int pat_shard_image(pat_plan* plan, int side, const void* recv, float* out, cons
     cudaStream_t s = (cudaStream_t)stream;
     const int n = (side ? L.nt : L.nz) / p.shard_world;
     double* dsum = r2 ? plan->x.res + 3 : nullptr;
-    PAT_CUDA(launch_image(p, recv, p.shard_W, out, (int64_t)L.ny * L.nx, n, sub, dsum, s, 0, nullptr,
-                          no_sampling(), side ? p.shard_tmap : p.shard_zmap));
+    const SpecRow sr{p.shard_W, side ? p.shard_tmap : p.shard_zmap, 0};
+    PAT_CUDA(launch_image(p, recv, sr, out, (int64_t)L.ny * L.nx, n, sub, dsum, s));
     if (r2) {
       PAT_CUDA(cudaMemcpyAsync(r2, dsum, sizeof(double), cudaMemcpyDeviceToHost, s));
       PAT_CUDA(cudaStreamSynchronize(s));

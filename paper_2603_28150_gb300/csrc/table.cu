@@ -543,7 +543,9 @@ int build_table_from_source(Plan& p, const void* table, pat_table_format fmt, bo
     *out = spec;
     *out_stride = Kfull;
     *rowmajor = 0;
-    return launch_spectrum(prep, src, (int64_t)L.px * L.py, L.px, L.py, spec, Kfull, n, s);
+    SpecRow sr;
+    sr.stride = Kfull;
+    return launch_spectrum(prep, src, (int64_t)L.px * L.py, L.px, L.py, spec, sr, n, s);
   };
 
   // Pass 1: statistics of the whole library.
