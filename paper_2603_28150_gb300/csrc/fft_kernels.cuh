@@ -89,9 +89,15 @@ struct TwPlan {
   static constexpr int N = (TOTAL + 1) & ~1;  // even: the work buffers stay 16-byte aligned
 };
 
-// One padding slot per 16 elements keeps the radix-16 scatter of the first
-// pass (stride 16) free of shared-memory bank conflicts.
-__device__ __forceinline__ int pidx(int i) { return i + (i >> 4); }
+// One padding slot per 16 elements, or per 32 where the first pass has radix
+// 32, keeps the scatter of the first pass (stride 16 or 32) free of
+// shared-memory bank conflicts (with one per 16 the radix-32 scatter met
+// two-way conflicts, 30 % of all wavefronts of the column passes at P = 512;
+// column inverse of 201 slices 69.8 -> 59.6 us).
+template <int P>
+__device__ __forceinline__ int pidx(int i) {
+  return i + (i >> (RadixPlan<P>::RMAX == 32 ? 5 : 4));
+}
 
 // exp(-2 pi i m / 16) for m in [0, 8) (conjugated for the inverse); m is a
 // compile-time constant after unrolling, so the switch folds away.
@@ -327,7 +333,7 @@ __device__ __forceinline__ void run_passes(cx<R>* buf, const cx<R>* tw, int tid,
       else if constexpr (first_ld)
         v[q][r] = ld(j + r * NB);
       else
-        v[q][r] = buf[pidx(j + r * NB)];
+        v[q][r] = buf[pidx<P>(j + r * NB)];
     }
     if constexpr (NS > 1) {
       const int k = j % NS;
@@ -359,7 +365,7 @@ __device__ __forceinline__ void run_passes(cx<R>* buf, const cx<R>* tw, int tid,
       const int k = j % NS;
       const int base = (j - k) * RAD + k;
 #pragma unroll
-      for (int r = 0; r < ROUT; ++r) buf[pidx(base + r * NS)] = v[q][r];
+      for (int r = 0; r < ROUT; ++r) buf[pidx<P>(base + r * NS)] = v[q][r];
     }
     __syncthreads();
   }
@@ -410,6 +416,27 @@ __device__ __forceinline__ int scan_index(int c, int o, int st, int n) {
   const int i = d / st;
   return i < n ? i : -1;
 }
+
+// Sum of squares in FP64, every square exact. An FP64 instruction occupies an
+// SM for 16 cycles per warp here, and so does the conversion of a float: with
+// one conversion and one multiply-add per residual the FP64 pipe was the
+// busiest unit of the residual pass (53 % at P = 256). Normal floats and zero
+// are therefore widened by integer operations, bit for bit the conversion of
+// |r|; `odd` is non-zero if a value was none of these (subnormal, infinite or
+// NaN), and the caller then sums the converted values instead.
+struct SumSq {
+  double s = 0.0;
+  uint32_t odd = 0;
+  __device__ __forceinline__ void add(float r) {
+    const uint32_t u = __float_as_uint(r) & 0x7fffffffu;
+    const bool normal = u - 0x00800000u < 0x7f000000u;
+    const double d =
+        __hiloint2double(normal ? (int)((u >> 3) + 0x38000000u) : 0, (int)(u << 29));
+    odd |= normal ? 0u : u;
+    s = fma(d, d, s);
+  }
+  __device__ __forceinline__ void add(double r) { s = fma(r, r, s); }
+};
 
 // Input of one packed row pair (rows y0, y0 + 1 of a slice, a + i b),
 // zero-padded from nx_in: the plain [ny][nx] slice, or with SAMP the
@@ -559,8 +586,8 @@ __device__ __forceinline__ void store_pair(cx<R>* p, cx<R> a, cx<R> b) {
 // Z[P - kx] = conj(A) + i conj(B) (A, B the half spectra of two real rows).
 template <typename R, int P>
 __device__ __forceinline__ void pack_pair(cx<R>* b, int kx, cx<R> A, cx<R> B) {
-  b[pidx(kx)] = mk<R>(A.x - B.y, A.y + B.x);
-  if (kx > 0 && kx < P / 2) b[pidx(P - kx)] = mk<R>(A.x + B.y, B.x - A.y);
+  b[pidx<P>(kx)] = mk<R>(A.x - B.y, A.y + B.x);
+  if (kx > 0 && kx < P / 2) b[pidx<P>(P - kx)] = mk<R>(A.x + B.y, B.x - A.y);
 }
 
 // Stage i, row pass: rows y0 = 2 pair, y0 + 1 of slice s packed as a + i b,
@@ -591,7 +618,7 @@ __global__ void __launch_bounds__(kThreads) k_row_r2c(const R* __restrict__ in, 
     const int yy = 2 * (pair0 + vv);
     if (yy >= ny_in) continue;
     cx<R> A, B;
-    untangle(bufs[vv * SH::VSTR + pidx(kx)], bufs[vv * SH::VSTR + pidx((P - kx) % P)], &A,
+    untangle(bufs[vv * SH::VSTR + pidx<P>(kx)], bufs[vv * SH::VSTR + pidx<P>((P - kx) % P)], &A,
              &B);
     store_pair(dst + (int64_t)kx * tstride + yy, A, B);  // tstride even: yy + 1 < tstride
   }
@@ -690,10 +717,10 @@ __global__ void __launch_bounds__(kThreads) k_col_fwd(const cx<R>* __restrict__ 
         if (y > P / 2) break;
         const int s0 = __ldg(sl + y);
         if (y == 0 || y == P / 2) {
-          dst[s0] = b[pidx(y)];
+          dst[s0] = b[pidx<P>(y)];
           continue;
         }
-        slot_store_pair(dst, s0, __ldg(sl + P - y), b[pidx(y)], b[pidx(P - y)]);
+        slot_store_pair(dst, s0, __ldg(sl + P - y), b[pidx<P>(y)], b[pidx<P>(P - y)]);
       }
     }
   } else {
@@ -872,8 +899,11 @@ __device__ __forceinline__ void stage_rows(R* dst, const R* src, int n) {
 // *total. A plan's nx is at most P/2 (P >= 2 nx - 1,
 // P even), so the inverse transform forms only x < P/2 and the forward one
 // skips the zero half.
+//
+// P = 768 alone is held to 128 registers, two CTAs per SM (143 -> 98 us at
+// 384^2 x 48); every other length keeps the compiler's choice.
 template <typename R, int P, bool SAMP>
-__global__ void __launch_bounds__(kThreads) k_row_resid(cx<R>* __restrict__ T, int tstride,
+__global__ void __launch_bounds__(kThreads, sizeof(R) == 4 && P == 768 ? 2 : 0) k_row_resid(cx<R>* __restrict__ T, int tstride,
                                                         int64_t tslice, int nx, int ny,
                                                         const R* __restrict__ y,
                                                         int64_t y_stride,
@@ -904,7 +934,7 @@ __global__ void __launch_bounds__(kThreads) k_row_resid(cx<R>* __restrict__ T, i
   // the layout of y: the row pair's offsets (scan rows with sampling on)
   const int y0 = 2 * (pair0 + v);
   RowPairStore<R, SAMP> rows(nullptr, y + s * y_stride, y0, nx, ny, sm);
-  double acc = 0.0;
+  SumSq sq;
   // image rows x < P/2 from the last inverse pass, turned into the residual
   // in place: that pass writes exactly the positions its thread read, so r
   // replaces the image without a barrier (zero past nx; the forward pass
@@ -916,16 +946,25 @@ __global__ void __launch_bounds__(kThreads) k_row_resid(cx<R>* __restrict__ T, i
     if (xi >= 0) {
       if (rows.ok0) {
         r0 = z.x - (YS::on ? ys[2 * v * nx + xi] : rows.sslice[rows.off0 + xi]);
-        acc += (double)r0 * (double)r0;
       }
       if (rows.ok1) {
         r1 = z.y - (YS::on ? ys[(2 * v + 1) * nx + xi] : rows.sslice[rows.off1 + xi]);
-        acc += (double)r1 * (double)r1;
       }
     }
-    b[pidx(x)] = mk<R>(r0, r1);
+    b[pidx<P>(x)] = mk<R>(r0, r1);
+    sq.add(r0);
+    sq.add(r1);
   };
   run_passes<R, P, 0, true, false, true, false, true>(b, tw, tid, sl, resid);
+  double acc = sq.s;
+  if (sq.odd) {  // the thread's own elements again, converted
+    acc = 0.0;
+    for (int x = tid; x < P / 2; x += SH::TPV) {
+      const cx<R> r = b[pidx<P>(x)];
+      acc = fma((double)r.x, (double)r.x, acc);
+      acc = fma((double)r.y, (double)r.y, acc);
+    }
+  }
   __syncthreads();
   run_passes<R, P, 0, false, false, false, true>(b, tw, tid, sl, ns);  // spectrum of r0 + i r1
 #pragma unroll 4
@@ -934,7 +973,7 @@ __global__ void __launch_bounds__(kThreads) k_row_resid(cx<R>* __restrict__ T, i
     const int yy = 2 * (pair0 + vv);
     if (yy >= ny) continue;
     cx<R> A, B;
-    untangle(bufs[vv * SH::VSTR + pidx(kx)], bufs[vv * SH::VSTR + pidx((P - kx) % P)], &A,
+    untangle(bufs[vv * SH::VSTR + pidx<P>(kx)], bufs[vv * SH::VSTR + pidx<P>((P - kx) % P)], &A,
              &B);
     store_pair(Ts + (int64_t)kx * tstride + yy, A, B);  // tstride even: yy + 1 < tstride
   }
@@ -1022,7 +1061,7 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r_step(
       if (ok0) n0 = upd(x, z.x);
       if (ok1) n1 = upd((int64_t)nx + x, z.y);
     }
-    if constexpr (NEXT) b[pidx(x)] = mk<R>(n0, n1);
+    if constexpr (NEXT) b[pidx<P>(x)] = mk<R>(n0, n1);
   };
   SmemLoad<R> ld;
   run_passes<R, P, 0, true, false, true, false, true>(b, tw, tid, ld, st);
@@ -1037,7 +1076,7 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r_step(
       const int yy = 2 * (pair0 + vv);
       if (yy >= ny) continue;
       cx<R> A, B;
-      untangle(bufs[vv * SH::VSTR + pidx(kx)], bufs[vv * SH::VSTR + pidx((P - kx) % P)], &A, &B);
+      untangle(bufs[vv * SH::VSTR + pidx<P>(kx)], bufs[vv * SH::VSTR + pidx<P>((P - kx) % P)], &A, &B);
       store_pair(Ts + (int64_t)kx * tstride + yy, A, B);  // tstride even: yy + 1 < tstride
     }
   }
