@@ -106,7 +106,7 @@ void free_plan(pat_plan* pp) {
   // the plan's own memory: the table side, buffers allocated on first use,
   // and the workspace arena unless the caller owns it
   void* owned[] = {p.table,      p.tc_fwd,     p.tc_adj,     p.fold_members, p.fold_rep,
-                   p.fold_slot,  p.rb_members, p.rb_chunk,   p.rep_row,      p.shard_zmap,
+                   p.fold_order, p.rb_members, p.rb_chunk,   p.rep_row,      p.shard_zmap,
                    p.shard_tmap, p.shard_members};
   for (void* b : owned) dev_free(b);
   if (x.io_heap) {
@@ -150,15 +150,6 @@ int c2r_partials_bound(const Layout& L) {
   return (int)(smax * ((L.ny + 1) / 2 + 1));
 }
 
-// Complex elements per row of the X / Y spectra buffers: the bins (Kpad), or
-// the representative slots 4 * Upad of a folded single-precision plan's
-// batched tensor-core path, whichever is longer.
-int64_t spectrum_row_cap(const Layout& L) {
-  if (L.fp64 || L.px != L.py) return L.Kpad;
-  const int64_t h = L.px / 2, U = (h + 1) * (h + 2) / 2;
-  return std::max<int64_t>(L.Kpad, 4 * ((U + 31) / 32 * 32));
-}
-
 // FISTA momentum / residual history kept in the workspace: 4096 iterations
 // per solve (a plan that allocates its own memory grows it on demand).
 constexpr int kHistCap = 4097;
@@ -179,9 +170,9 @@ size_t ws_walk(pat_plan* pp, unsigned char* base, bool with_io, int64_t lean_sli
   const size_t cs = 2 * L.rsize;
   const int64_t per = std::max(L.nz, L.nt);
   const int64_t smax = lean ? lean_slices : (int64_t)L.max_batch * per;
-  // a volume's slices rounded up to whole quads where the plan may fold
-  const int64_t rows = L.fp64 || L.px != L.py ? smax : (int64_t)L.max_batch * ((per + 3) / 4 * 4);
-  const size_t xy = lean ? 0 : (size_t)rows * spectrum_row_cap(L) * cs;
+  // a volume's slices rounded up to whole groups where the plan may fold
+  const int64_t rows = L.fp64 || L.px != L.py ? smax : (int64_t)L.max_batch * ((per + kGroup - 1) / kGroup * kGroup);
+  const size_t xy = lean ? 0 : (size_t)rows * L.Kpad * cs;
   const size_t tb = (size_t)smax * L.tslice * cs;
   const size_t vol = lean ? 0 : (size_t)L.max_batch * L.nz * L.ny * L.nx * L.rsize;
   const size_t dat = lean ? 0 : (size_t)L.max_batch * L.nt * L.ny * L.nx * L.rsize;
@@ -346,10 +337,10 @@ cudaError_t forward_dev(const Plan& p, const void* rho, void* d, int batch, cuda
                         const void* sub, double* sumsq, int groups, double* group_sums) {
   const Layout& L = p.L;
   const int64_t plane = (int64_t)L.ny * L.nx, scan = (int64_t)L.my * L.mx;
-  const SpecRow zr = spec_row(p, batch, L.nz), tr = spec_row(p, batch, L.nt);
+  const SpecRow zr = spec_row(p, L.nz), tr = spec_row(p, L.nt);
   cudaError_t e = launch_spectrum(p, rho, plane, L.nx, L.ny, p.X, zr, batch * L.nz, s);
   if (e != cudaSuccess) return e;
-  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s, zr.quad > 0)) != cudaSuccess) return e;
+  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s, zr.group > 0)) != cudaSuccess) return e;
   return launch_image(p, p.Y, tr, d, scan, batch * L.nt, sub, sumsq, s, groups, group_sums,
                       sampling_of(L));
 }
@@ -359,19 +350,19 @@ cudaError_t gradient_dev(const Plan& p, const void* x, const void* y, void* grad
                          const FistaStep* step) {
   const Layout& L = p.L;
   const int64_t plane = (int64_t)L.ny * L.nx, scan = (int64_t)L.my * L.mx;
-  const SpecRow zr = spec_row(p, batch, L.nz), tr = spec_row(p, batch, L.nt);
-  const bool quad = zr.quad > 0;
+  const SpecRow zr = spec_row(p, L.nz), tr = spec_row(p, L.nt);
+  const bool grouped = zr.group > 0;
   // with a step that leaves the row transform of the next x in T, stage i
   // here is its column pass alone
   cudaError_t e = (step && step->next_T)
                       ? launch_spectrum_cols(p, L.ny, p.X, zr, batch * L.nz, s)
                       : launch_spectrum(p, x, plane, L.nx, L.ny, p.X, zr, batch * L.nz, s);
   if (e != cudaSuccess) return e;
-  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s, quad)) != cudaSuccess) return e;
+  if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s, grouped)) != cudaSuccess) return e;
   if ((e = launch_residual(p, p.Y, tr, y, scan, batch * L.nt, sumsq, s, groups, group_sums,
                            sampling_of(L), p.Y)) != cudaSuccess)
     return e;
-  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s, quad)) != cudaSuccess) return e;
+  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s, grouped)) != cudaSuccess) return e;
   if (step) return launch_image_step(p, p.X, zr, batch * L.nz, *step, s);
   return launch_image(p, p.X, zr, grad, plane, batch * L.nz, nullptr, nullptr, s);
 }
@@ -379,10 +370,10 @@ cudaError_t gradient_dev(const Plan& p, const void* x, const void* y, void* grad
 cudaError_t adjoint_dev(const Plan& p, const void* d, void* rho, int batch, cudaStream_t s) {
   const Layout& L = p.L;
   const int64_t plane = (int64_t)L.ny * L.nx, scan = (int64_t)L.my * L.mx;
-  const SpecRow zr = spec_row(p, batch, L.nz), tr = spec_row(p, batch, L.nt);
+  const SpecRow zr = spec_row(p, L.nz), tr = spec_row(p, L.nt);
   cudaError_t e = launch_spectrum(p, d, scan, L.nx, L.ny, p.Y, tr, batch * L.nt, s, sampling_of(L));
   if (e != cudaSuccess) return e;
-  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s, zr.quad > 0)) != cudaSuccess) return e;
+  if ((e = launch_contract_adj(p, p.Y, p.X, batch, s, zr.group > 0)) != cudaSuccess) return e;
   return launch_image(p, p.X, zr, rho, plane, batch * L.nz, nullptr, nullptr, s);
 }
 
@@ -1010,13 +1001,13 @@ int pat_stage_contract(pat_plan* plan, const void* in, void* out, int batch, int
   const Plan& p = plan->p;
   const int64_t rin = (int64_t)batch * (adjoint ? p.L.nt : p.L.nz);
   const int64_t rout = (int64_t)batch * (adjoint ? p.L.nz : p.L.nt);
-  if (tc_slots(p, batch)) {  // the tensor path's slot layout, converted in and out
-    PAT_CUDA(launch_to_slots(p, in, p.X, rin, s));
+  if (tc_slots(p, batch)) {  // the tensor path's grouped slices, converted in and out
+    PAT_CUDA(launch_to_groups(p, in, p.X, rin, s));
     if (adjoint)
-      PAT_CUDA(launch_contract_adj(p, p.X, p.Y, batch, s));
+      PAT_CUDA(launch_contract_adj(p, p.X, p.Y, batch, s, true));
     else
-      PAT_CUDA(launch_contract_fwd(p, p.X, p.Y, batch, s));
-    PAT_CUDA(launch_from_slots(p, p.Y, out, rout, s));
+      PAT_CUDA(launch_contract_fwd(p, p.X, p.Y, batch, s, true));
+    PAT_CUDA(launch_from_groups(p, p.Y, out, rout, s));
     return PAT_OK;
   }
   if (adjoint)

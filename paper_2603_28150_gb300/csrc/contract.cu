@@ -218,20 +218,23 @@ __global__ void __launch_bounds__(kWarps * 32, (sizeof(R) == 4 && !CPLX && VB ==
 //
 // The members of a block's representatives are scattered over the half
 // spectrum, so with one row of bins per slice every access is an 8-byte piece
-// of a 32-byte sector. QUAD spectra interleave four slices ([slice / 4][bin]
-// [slice % 4], see SpecRow): a lane's four time samples (depths) of one bin
-// are one whole sector. The spectra of a block are staged in shared memory in
-// the same quads, [member][quad][lane] with the 16-byte halves of a quad
-// swizzled so that a warp's 16-byte reads touch every bank once.
+// of a 32-byte sector. GRP spectra interleave eight slices ([slice / 8][bin]
+// [slice % 8], see SpecRow): a lane's eight time samples (depths) of one bin
+// are 64 contiguous bytes, two whole sectors. The spectra of a block are
+// staged in shared memory in quads of four slices, [member][quad][lane] with
+// the 16-byte halves of a quad swizzled so that a warp's 16-byte reads touch
+// every bank once.
 //
 // Measured per launch (one GB300, forward / adjoint): 128^2 -> 256^2 x 64 x
-// 256, 0.40 GB stored: 93 / 90 us, from 110 / 113 with bin rows and the table
-// loaded into registers; 256^2 -> 512^2 x 128 x 512, 5.8 GB: 1250 / 1233 from
-// 2270 / 1915; 202^2 -> 512^2 x 17 x 201: 147 / 173 from 507 / 316; five
-// volumes at 64^2 -> 128^2 x 32 x 128: 35 / 39 from 57 / 76. Without the table
-// copies the 128^2 launch takes 70 / 62 us and without the multiply-adds 80 /
-// 88: shared-memory and L1 traffic (the spectra, the ring and the 32-line
-// stores of scattered sectors) and the table stream overlap only in part.
+// 256, 0.40 GB stored: 96 / 92 us, from 110 / 113 with bin rows and the table
+// loaded into registers; 256^2 -> 512^2 x 128 x 512, 5.8 GB: 1253 / 1192 from
+// 2270 / 1915; 202^2 -> 512^2 x 17 x 201: 138 / 157 from 507 / 316 (147 / 173
+// with groups of four slices, 3 us faster at 128^2 where the spectra stay in
+// L2); five volumes at 64^2 -> 128^2 x 32 x 128: 36 / 39 from 57 / 76. Without
+// the table copies the 128^2 launch takes 70 / 62 us and without the
+// multiply-adds 80 / 88: shared-memory and L1 traffic (the spectra, the ring
+// and the 32-line stores of scattered sectors) and the table stream overlap
+// only in part.
 constexpr int kFoldThreads = 512;  // most threads of a CTA (caps the registers at 128)
 
 // 16-byte slot of half h (slices 2h, 2h + 1) of a lane's quad in its 1 KB row.
@@ -239,10 +242,15 @@ __device__ __forceinline__ int quad_slot(int lane, int h) {
   return (2 * lane + h) ^ ((lane >> 2) & 1);
 }
 
+// Offset of quad q (slices 4q .. 4q + 3) of a bin in grouped spectra.
+__device__ __forceinline__ int64_t group_off(int q, int64_t bin, int64_t Kpad) {
+  return ((int64_t)(q >> 1) * Kpad + bin) * kGroup + (q & 1) * 4;
+}
+
 // Starts the copy of quads [q0, q0 + nq) of the four members' spectra into
 // dst[4][rows][64] (16-byte slots); slices at or past n and absent members
 // become zero. in: this volume's spectra.
-template <bool QUAD>
+template <bool GRP>
 __device__ __forceinline__ void stage_quads(float4* dst, int rows, const cx<float>* in,
                                             const int* bins, int q0, int nq, int n, int64_t Kpad,
                                             int lane, int warp, int nwarps) {
@@ -256,9 +264,9 @@ __device__ __forceinline__ void stage_quads(float4* dst, int rows, const cx<floa
       for (int h = 0; h < 2; ++h) {
         const uint32_t d = (uint32_t)__cvta_generic_to_shared(row + quad_slot(lane, h));
         const int s = 4 * (q0 + q) + 2 * h;  // first slice of this half
-        if constexpr (QUAD) {
+        if constexpr (GRP) {
           const int bytes = ok ? 8 * max(0, min(2, n - s)) : 0;
-          const cx<float>* src = in + ((int64_t)(q0 + q) * Kpad + bin) * 4 + 2 * h;
+          const cx<float>* src = in + group_off(q0 + q, bin, Kpad) + 2 * h;
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d),
                        "l"(bytes ? src : in), "r"(bytes)
                        : "memory");
@@ -279,11 +287,11 @@ __device__ __forceinline__ void stage_quads(float4* dst, int rows, const cx<floa
 }
 
 // Stores the values of four consecutive slices 4q .. 4q + 3 of one bin.
-template <bool QUAD>
+template <bool GRP>
 __device__ __forceinline__ void store_quad(cx<float>* out, int q, int bin, int n, int64_t Kpad,
                                            cx<float> a, cx<float> b, cx<float> c, cx<float> d) {
-  if constexpr (QUAD) {  // slices at or past n are padding that no reader uses
-    float4* o = reinterpret_cast<float4*>(out + ((int64_t)q * Kpad + bin) * 4);
+  if constexpr (GRP) {  // slices at or past n are padding that no reader uses
+    float4* o = reinterpret_cast<float4*>(out + group_off(q, bin, Kpad));
     o[0] = make_float4(a.x, a.y, b.x, b.y);
     o[1] = make_float4(c.x, c.y, d.x, d.y);
   } else {
@@ -296,11 +304,11 @@ __device__ __forceinline__ void store_quad(cx<float>* out, int q, int bin, int n
 }
 
 // Adds what store_quad wrote to a .. d.
-template <bool QUAD>
+template <bool GRP>
 __device__ __forceinline__ void add_quad(const cx<float>* out, int q, int bin, int n, int64_t Kpad,
                                          cx<float>& a, cx<float>& b, cx<float>& c, cx<float>& d) {
-  const cx<float>* o = QUAD ? out + ((int64_t)q * Kpad + bin) * 4 : out + (int64_t)(4 * q) * Kpad + bin;
-  const int64_t st = QUAD ? 1 : Kpad;
+  const cx<float>* o = GRP ? out + group_off(q, bin, Kpad) : out + (int64_t)(4 * q) * Kpad + bin;
+  const int64_t st = GRP ? 1 : Kpad;
   a = cadd(a, o[0]);
   if (4 * q + 1 < n) b = cadd(b, o[st]);
   if (4 * q + 2 < n) c = cadd(c, o[2 * st]);
@@ -308,9 +316,9 @@ __device__ __forceinline__ void add_quad(const cx<float>* out, int q, int bin, i
 }
 
 // Complex values per volume of a spectrum of n slices.
-template <bool QUAD>
+template <bool GRP>
 __device__ __forceinline__ int64_t vol_len(int n, int64_t Kpad) {
-  return (QUAD ? (int64_t)((n + 3) / 4) * 4 : (int64_t)n) * Kpad;
+  return (GRP ? (int64_t)((n + kGroup - 1) / kGroup) * kGroup : (int64_t)n) * Kpad;
 }
 
 // 16-byte asynchronous copy of a table float4 (zero when !ok).
@@ -331,7 +339,7 @@ __device__ __forceinline__ void cp_wait() {
 // the lanes that read them (no barrier: a lane reads its own copies), so the
 // table bytes in flight do not cost registers.
 // grid (batch, nrb, splits of the time blocks), tb time blocks per split.
-template <bool QUAD, int T, int R>
+template <bool GRP, int T, int R>
 __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_fwd(const float4* __restrict__ table, const int4* __restrict__ members,
                const int* __restrict__ chunk, const cx<float>* __restrict__ X,
@@ -367,7 +375,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       const int4 mem = members[ub * 32 + lane];
       const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
       if (g0 == 0) pdl_wait();
-      stage_quads<QUAD>(xs, gc, X + b * vol_len<QUAD>(nz, Kpad), bins, g0, g1 - g0, nz, Kpad,
+      stage_quads<GRP>(xs, gc, X + b * vol_len<GRP>(nz, Kpad), bins, g0, g1 - g0, nz, Kpad,
                         lane, warp, nwarps);
     }
     cp_wait<0>();
@@ -403,7 +411,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       }
       const int4 mem = __ldg(members + ub * 32 + lane);
       const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
-      cx<float>* Yb = Y + b * vol_len<QUAD>(nt, Kpad);
+      cx<float>* Yb = Y + b * vol_len<GRP>(nt, Kpad);
 #pragma unroll
       for (int r = 0; r < T; r += 4) {
         const int q = (bk * T + r) / 4;
@@ -411,9 +419,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
           if (bins[m] < 0) continue;
-          if (g0 > 0) add_quad<QUAD>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m],
+          if (g0 > 0) add_quad<GRP>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m],
                                      acc[r + 2][m], acc[r + 3][m]);
-          store_quad<QUAD>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m], acc[r + 2][m],
+          store_quad<GRP>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m], acc[r + 2][m],
                            acc[r + 3][m]);
         }
       }
@@ -422,14 +430,14 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   }
 }
 
-// Adjoint: warp (zi, ti) of zw x tw owns the z-groups zc zw GPW + zi + j zw
+// Adjoint: warp (zi, ti) of zw x tw owns the z-groups (zc zw + zi) GPW + j
 // (j < GPW) and the quads ti, ti + tw, ...; the 4 members' D of SQ tw quads
 // are staged in shared memory (two buffers, the next stage's copies in flight
 // during the current one) and reused by all warps; the table comes through
 // the warp's ring as in the forward. With tw > 1 the warps' partial sums of
 // one z-group meet in shared memory at the end, in the order of ti. grid
 // (z-chunks x batch, nrb).
-template <bool QUAD, int GPW, int SQ, int R>
+template <bool GRP, int GPW, int SQ, int R>
 __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_adj(const float4* __restrict__ table, const int4* __restrict__ members,
                const int* __restrict__ chunk, const cx<float>* __restrict__ D,
@@ -443,7 +451,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   const int64_t ub = blockIdx.y;
   const int zc = blockIdx.x % nzc, b = blockIdx.x / nzc;
   const int zi = warp % zw, ti = warp / zw;
-  const int gbase = zc * zw * GPW + zi;
+  const int gbase = (zc * zw + zi) * GPW;
   const float4* tbl =
       table + ((int64_t)(chunk ? chunk[ub] : ub) * nt * nzg + gbase) * 32 + lane;
   const int ntq = (nt + 3) / 4, nst = (ntq + tq - 1) / tq;
@@ -455,9 +463,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int j = 0; j < GPW; ++j) {
-          const bool ok = 4 * pq + r < nt && gbase + j * zw < nzg;
+          const bool ok = 4 * pq + r < nt && gbase + j < nzg;
           cp_table(ring + ((slot * 4 + r) * GPW + j) * 32,
-                   ok ? src + ((int64_t)r * nzg + j * zw) * 32 : table, ok);
+                   ok ? src + ((int64_t)r * nzg + j) * 32 : table, ok);
         }
       pq += tw;
     }
@@ -467,7 +475,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   for (int i = 0; i < R - 1; ++i) copy_ahead(i);
   const int4 mem = members[ub * 32 + lane];
   const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
-  const cx<float>* Db = D + b * vol_len<QUAD>(nt, Kpad);
+  const cx<float>* Db = D + b * vol_len<GRP>(nt, Kpad);
   cx<float> acc[GPW][4][4];
 #pragma unroll
   for (int j = 0; j < GPW; ++j)
@@ -476,7 +484,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
 #pragma unroll
       for (int m = 0; m < 4; ++m) acc[j][q][m] = mk<float>(0.f, 0.f);
   pdl_wait();
-  stage_quads<QUAD>(ds, tq, Db, bins, 0, min(tq, ntq), nt, Kpad, lane, warp, nwarps);
+  stage_quads<GRP>(ds, tq, Db, bins, 0, min(tq, ntq), nt, Kpad, lane, warp, nwarps);
   cp_wait<0>();
   int slot = 0;
   for (int st = 0; st < nst; ++st) {
@@ -485,7 +493,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     if (st > 0) cp_wait<SQ>();
     __syncthreads();  // and every warp is done with the other buffer
     if (st + 1 < nst)
-      stage_quads<QUAD>(ds + ((st + 1) & 1) * 4 * tq * 64, tq, Db, bins, q0 + tq,
+      stage_quads<GRP>(ds + ((st + 1) & 1) * 4 * tq * 64, tq, Db, bins, q0 + tq,
                         min(tq, ntq - q0 - tq), nt, Kpad, lane, warp, nwarps);
     const float4* dst = ds + (st & 1) * 4 * tq * 64;
 #pragma unroll 1
@@ -548,22 +556,22 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       }
   }
   if (ti != 0) return;
-  cx<float>* Zb = Z + b * vol_len<QUAD>(nz, Kpad);
+  cx<float>* Zb = Z + b * vol_len<GRP>(nz, Kpad);
 #pragma unroll
   for (int j = 0; j < GPW; ++j) {
-    const int g = gbase + j * zw;
+    const int g = gbase + j;
     if (g >= nzg) break;
 #pragma unroll
     for (int m = 0; m < 4; ++m)
       if (bins[m] >= 0)
-        store_quad<QUAD>(Zb, g, bins[m], nz, Kpad, acc[j][0][m], acc[j][1][m], acc[j][2][m],
+        store_quad<GRP>(Zb, g, bins[m], nz, Kpad, acc[j][0][m], acc[j][1][m], acc[j][2][m],
                          acc[j][3][m]);
   }
 }
 
 constexpr size_t kSmemCta = 227 * 1024;  // most shared memory of a CTA (and of an SM's CTAs)
 
-template <bool QUAD, int T, int R>
+template <bool GRP, int T, int R>
 cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc, cudaStream_t s) {
   const Layout& L = p.L;
   constexpr size_t ring = (size_t)R * T * 512;  // bytes per warp
@@ -571,7 +579,7 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
   const bool two = 2 * (xbytes + 8 * ring) <= kSmemCta;
   const int nwarps = two ? 8 : (int)std::min<size_t>(16, (kSmemCta - xbytes) / ring);
   const size_t smem = xbytes + nwarps * ring;
-  auto fn = k_fold_fwd<QUAD, T, R>;
+  auto fn = k_fold_fwd<GRP, T, R>;
   cudaError_t e = cudaFuncSetAttribute((const void*)fn,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -599,7 +607,7 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
                     static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad, tb, gc);
 }
 
-template <bool QUAD>
+template <bool GRP>
 cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s) {
   const Layout& L = p.L;
   if ((size_t)L.nzg * 4096 > kSmemCta) return cudaErrorInvalidValue;  // more than 224 depths
@@ -610,11 +618,11 @@ cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStrea
   // volumes at 96^2 x 45: 78 against 84 us); at 64 depths two CTAs with
   // blocks of 4 are faster than one of 16 warps with blocks of 8 (93 / 101 us).
   if (2 * ((size_t)gc * 4096 + 64 * 1024) <= kSmemCta)
-    return fold_fwd_t<QUAD, 8, 2>(p, X, Y, batch, gc, s);
-  return fold_fwd_t<QUAD, 4, 3>(p, X, Y, batch, gc, s);
+    return fold_fwd_t<GRP, 8, 2>(p, X, Y, batch, gc, s);
+  return fold_fwd_t<GRP, 4, 3>(p, X, Y, batch, gc, s);
 }
 
-template <bool QUAD, int GPW, int SQ, int R>
+template <bool GRP, int GPW, int SQ, int R>
 cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw, int tw,
                        cudaStream_t s) {
   const Layout& L = p.L;
@@ -622,7 +630,7 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
   const size_t ring = (size_t)nwarps * R * 4 * GPW * 512;
   const size_t smem = std::max<size_t>(2 * 4096 * (size_t)SQ * tw + ring,
                                        (size_t)(tw - 1) * zw * GPW * 4096);
-  auto fn = k_fold_adj<QUAD, GPW, SQ, R>;
+  auto fn = k_fold_adj<GRP, GPW, SQ, R>;
   cudaError_t e = cudaFuncSetAttribute((const void*)fn,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -637,7 +645,7 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
 // for the time samples. Grids with less than about one CTA per SM split the
 // z-groups over more CTAs (64^2 x 32: 12.7 us in two, 17 in one; 32^2 x 16:
 // 5.7 us in four of one group per warp, 13 in one).
-template <bool QUAD>
+template <bool GRP>
 cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s) {
   const Layout& L = p.L;
   const int64_t ctas = L.nrb * batch;
@@ -648,11 +656,11 @@ cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStrea
     zw = (zw + 1) / 2;
     nzc = (units + zw - 1) / zw;
   }
-  if (zw == 1 && 2 * ctas * nzc <= 200) return fold_adj_t<QUAD, 1, 1, 4>(p, D, Z, batch, 1, 8, s);
+  if (zw == 1 && 2 * ctas * nzc <= 200) return fold_adj_t<GRP, 1, 1, 4>(p, D, Z, batch, 1, 8, s);
   static constexpr int kTw[8] = {8, 4, 2, 2, 1, 1, 1, 1};
   const int tw = kTw[zw - 1];
-  return tw <= 2 ? fold_adj_t<QUAD, 2, 2, 2>(p, D, Z, batch, zw, tw, s)
-                 : fold_adj_t<QUAD, 2, 1, 2>(p, D, Z, batch, zw, tw, s);
+  return tw <= 2 ? fold_adj_t<GRP, 2, 2, 2>(p, D, Z, batch, zw, tw, s)
+                 : fold_adj_t<GRP, 2, 1, 2>(p, D, Z, batch, zw, tw, s);
 }
 
 template <typename R, bool CPLX, int VB>
@@ -711,58 +719,57 @@ cudaError_t adj_vb(const Plan& p, const void* D, void* Z, int batch, cudaStream_
 
 }  // namespace
 
-__global__ void k_to_slots(const float2* __restrict__ in, float2* __restrict__ out,
-                           const int* __restrict__ slot, int64_t K, int64_t Kpad, int64_t srow,
+// Rows [S][Kpad] <-> grouped slices [S / 8][Kpad][8].
+__global__ void k_to_groups(const float2* __restrict__ in, float2* __restrict__ out, int64_t Kpad,
                            int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / K, k = i % K;
-    out[r * srow + __ldg(slot + k)] = in[r * Kpad + k];
+    const int64_t r = i / Kpad, k = i % Kpad;
+    out[((r / kGroup) * Kpad + k) * kGroup + r % kGroup] = in[i];
   }
 }
 
-__global__ void k_from_slots(const float2* __restrict__ in, float2* __restrict__ out,
-                             const int* __restrict__ slot, int64_t K, int64_t Kpad, int64_t srow,
+__global__ void k_from_groups(const float2* __restrict__ in, float2* __restrict__ out, int64_t Kpad,
                              int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / K, k = i % K;
-    out[r * Kpad + k] = in[r * srow + __ldg(slot + k)];
+    const int64_t r = i / Kpad, k = i % Kpad;
+    out[i] = in[((r / kGroup) * Kpad + k) * kGroup + r % kGroup];
   }
 }
 
-cudaError_t launch_to_slots(const Plan& p, const void* in, void* out, int64_t S, cudaStream_t s) {
-  const int64_t n = S * p.L.K;
+cudaError_t launch_to_groups(const Plan& p, const void* in, void* out, int64_t S, cudaStream_t s) {
+  const int64_t n = S * p.L.Kpad;
   const int g = (int)std::min<int64_t>((n + 255) / 256, 152 * 32);
-  k_to_slots<<<g, 256, 0, s>>>(static_cast<const float2*>(in), static_cast<float2*>(out),
-                               p.fold_slot, p.L.K, p.L.Kpad, slot_row(p.L), n);
+  k_to_groups<<<g, 256, 0, s>>>(static_cast<const float2*>(in), static_cast<float2*>(out), p.L.Kpad,
+                               n);
   return cudaGetLastError();
 }
 
-cudaError_t launch_from_slots(const Plan& p, const void* in, void* out, int64_t S,
+cudaError_t launch_from_groups(const Plan& p, const void* in, void* out, int64_t S,
                               cudaStream_t s) {
-  const int64_t n = S * p.L.K;
+  const int64_t n = S * p.L.Kpad;
   const int g = (int)std::min<int64_t>((n + 255) / 256, 152 * 32);
-  k_from_slots<<<g, 256, 0, s>>>(static_cast<const float2*>(in), static_cast<float2*>(out),
-                                 p.fold_slot, p.L.K, p.L.Kpad, slot_row(p.L), n);
+  k_from_groups<<<g, 256, 0, s>>>(static_cast<const float2*>(in), static_cast<float2*>(out),
+                                 p.L.Kpad, n);
   return cudaGetLastError();
 }
 
 cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s,
-                                bool quad) {
+                                bool grouped) {
   if (p.tc_fwd && p.tc_min_batch > 0 && batch >= p.tc_min_batch)
-    return tc_contract(p, p.tc_fwd, p.tc_adj, X, Y, batch, false, p.tc_err, s);
-  if (p.L.fold) return quad ? fold_fwd<true>(p, X, Y, batch, s) : fold_fwd<false>(p, X, Y, batch, s);
+    return tc_contract(p, p.tc_fwd, p.tc_adj, X, Y, batch, false, p.tc_err, s, grouped);
+  if (p.L.fold) return grouped ? fold_fwd<true>(p, X, Y, batch, s) : fold_fwd<false>(p, X, Y, batch, s);
   if (p.L.fp64)
     return p.L.real ? fwd_vb<double, false>(p, X, Y, batch, s) : fwd_vb<double, true>(p, X, Y, batch, s);
   return p.L.real ? fwd_vb<float, false>(p, X, Y, batch, s) : fwd_vb<float, true>(p, X, Y, batch, s);
 }
 
 cudaError_t launch_contract_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s,
-                                bool quad) {
+                                bool grouped) {
   if (p.tc_adj && p.tc_min_batch > 0 && batch >= p.tc_min_batch)
-    return tc_contract(p, p.tc_fwd, p.tc_adj, D, Z, batch, true, p.tc_err, s);
-  if (p.L.fold) return quad ? fold_adj<true>(p, D, Z, batch, s) : fold_adj<false>(p, D, Z, batch, s);
+    return tc_contract(p, p.tc_fwd, p.tc_adj, D, Z, batch, true, p.tc_err, s, grouped);
+  if (p.L.fold) return grouped ? fold_adj<true>(p, D, Z, batch, s) : fold_adj<false>(p, D, Z, batch, s);
   if (p.L.fp64)
     return p.L.real ? adj_vb<double, false>(p, D, Z, batch, s) : adj_vb<double, true>(p, D, Z, batch, s);
   return p.L.real ? adj_vb<float, false>(p, D, Z, batch, s) : adj_vb<float, true>(p, D, Z, batch, s);

@@ -56,14 +56,14 @@ struct Shape {
   // padded vector stride: the extra element puts consecutive vectors in
   // different banks for the transposed (vector-major) accesses of the row kernels
   static constexpr int VSTR = P + P / 16 + 1;
-  // stride of a column kernel on quad spectra, whose neighbouring threads are
-  // four slices by consecutive elements: 4 (mod 8) elements apart, so four
-  // slices x four elements touch the 16 8-byte banks once
-  static constexpr int VSTR_Q = (P + P / 16 + 3) / 8 * 8 + 4;
+  // stride of a column kernel on grouped spectra, whose neighbouring threads
+  // are eight slices by consecutive elements on the spectrum side: 2 (mod 4)
+  // elements apart, eight slices x two elements touch the 16 8-byte banks once
+  static constexpr int VSTR_G = (P + P / 16 + 1) / 4 * 4 + 2;
 };
 
 // Column kernels on the three spectrum layouts of SpecRow.
-enum { kRows = 0, kSlots = 1, kQuads = 2 };
+enum { kRows = 0, kSlots = 1, kGroups = 2 };
 
 // Radix of pass S and the product of the radices before it.
 template <int P, int S>
@@ -307,9 +307,13 @@ __device__ __forceinline__ void dft_reg(cx<R>* a) {
 // outputs [0, P/2) are used (the crop): the last pass, whose element r is
 // j + r P/RAD, neither forms nor writes its upper RAD/2 outputs (with a
 // shared-memory last pass those slots keep stale values).
+//
+// bufL, tidL: the vector and thread index of this thread in the last of
+// several passes, where another assignment of threads suits its stores.
 template <typename R, int P, int S, bool INV, bool FROM_LOAD, bool TO_STORE, bool ZIN = false,
           bool HOUT = false, class LD, class ST>
-__device__ __forceinline__ void run_passes(cx<R>* buf, const cx<R>* tw, int tid, LD& ld, ST& st) {
+__device__ __forceinline__ void run_passes(cx<R>* buf, const cx<R>* tw, int tid, LD& ld, ST& st,
+                                           cx<R>* bufL, int tidL) {
   constexpr int NST = RadixPlan<P>::NST;
   constexpr int RAD = PassOf<P, S>::RAD;
   constexpr int NS = PassOf<P, S>::NS;
@@ -370,7 +374,13 @@ __device__ __forceinline__ void run_passes(cx<R>* buf, const cx<R>* tw, int tid,
     __syncthreads();
   }
   if constexpr (S + 1 < NST)
-    run_passes<R, P, S + 1, INV, FROM_LOAD, TO_STORE, ZIN, HOUT>(buf, tw, tid, ld, st);
+    run_passes<R, P, S + 1, INV, FROM_LOAD, TO_STORE, ZIN, HOUT>(
+        S + 2 == NST ? bufL : buf, tw, S + 2 == NST ? tidL : tid, ld, st, bufL, tidL);
+}
+template <typename R, int P, int S, bool INV, bool FROM_LOAD, bool TO_STORE, bool ZIN = false,
+          bool HOUT = false, class LD, class ST>
+__device__ __forceinline__ void run_passes(cx<R>* buf, const cx<R>* tw, int tid, LD& ld, ST& st) {
+  run_passes<R, P, S, INV, FROM_LOAD, TO_STORE, ZIN, HOUT>(buf, tw, tid, ld, st, buf, tid);
 }
 
 template <typename R>
@@ -404,7 +414,7 @@ __device__ __forceinline__ cx<R>* setup_smem(const cx<R>* tw_g, cx<R>** tw_s) {
 
 template <typename R, int P, int MODE = kRows>
 constexpr size_t smem_bytes() {
-  return sizeof(cx<R>) * (size_t)(TwPlan<P>::N + Shape<P>::VPB * (MODE == kQuads ? Shape<P>::VSTR_Q
+  return sizeof(cx<R>) * (size_t)(TwPlan<P>::N + Shape<P>::VPB * (MODE == kGroups ? Shape<P>::VSTR_G
                                                                                  : Shape<P>::VSTR));
 }
 
@@ -640,38 +650,31 @@ __device__ __forceinline__ void slot_store_pair(cx<R>* dst, int s0, int s1, cx<R
   }
 }
 
-// The column (slice s, kx) of each of a block's vectors, and where its
-// spectrum lives. Rows and slots: consecutive vectors are consecutive columns,
-// a vector's threads are neighbours. Quads: the block holds the four slices of
-// VPB / 4 columns, and four neighbouring threads hold one element of the four
-// slices (one 32-byte sector).
+// The column (slice s, kx) of vector v of a block, and where its spectrum
+// lives. Rows and slots: consecutive vectors are consecutive columns. Groups:
+// the block holds the kGroup slices of VPB / kGroup columns, slice by slice.
 template <typename R, int P, int MODE>
 struct ColMap {
   using SH = Shape<P>;
-  static constexpr int VS = MODE == kQuads ? SH::VSTR_Q : SH::VSTR;
-  int v, tid;
+  static constexpr int VS = MODE == kGroups ? SH::VSTR_G : SH::VSTR;
+  static constexpr int STEP = MODE == kGroups ? kGroup : 1;
   bool ok;
   int64_t s, kx;
-  int64_t base;  // offset of element 0 (rows, quads) or of the slice's row (slots)
-  static constexpr int STEP = MODE == kQuads ? 4 : 1;
-  __device__ __forceinline__ ColMap(int ncols, int64_t nvec, int64_t stride, int quad) {
+  int64_t base;  // offset of element 0 (rows, groups) or of the slice's row (slots)
+  __device__ __forceinline__ ColMap(int v, int ncols, int64_t nvec, int64_t stride, int group) {
     // 32-bit quotients (slices x columns < 2^31): no 64-bit division
-    if constexpr (MODE == kQuads) {
-      const int sl = threadIdx.x & 3, c = threadIdx.x / (4 * SH::TPV);
-      tid = (threadIdx.x >> 2) % SH::TPV;
-      v = 4 * c + sl;
-      const unsigned g = blockIdx.x * (SH::VPB / 4) + c;  // (volume, quad, column)
-      const unsigned nq = (unsigned)(quad + 3) / 4;
-      const unsigned vq = g / (unsigned)ncols;
-      const unsigned vol = vq / nq;
-      const int sv = 4 * (int)(vq - vol * nq) + sl;  // slice within the volume
-      ok = g < nvec && sv < quad;
-      kx = ok ? (int64_t)(g - vq * (unsigned)ncols) : 0;
-      s = ok ? (int64_t)vol * quad + sv : 0;
-      base = ok ? ((int64_t)vq * stride + kx * P) * 4 + sl : 0;
+    if constexpr (MODE == kGroups) {
+      const int sl = v % kGroup;
+      const unsigned g = blockIdx.x * (SH::VPB / kGroup) + v / kGroup;  // (volume, group, column)
+      const unsigned ng = (unsigned)(group + kGroup - 1) / kGroup;
+      const unsigned vg = g / (unsigned)ncols;
+      const unsigned vol = vg / ng;
+      const int sv = kGroup * (int)(vg - vol * ng) + sl;  // slice within the volume
+      ok = g < nvec && sv < group;
+      kx = ok ? (int64_t)(g - vg * (unsigned)ncols) : 0;
+      s = ok ? (int64_t)vol * group + sv : 0;
+      base = ok ? ((int64_t)vg * stride + kx * P) * kGroup + sl : 0;
     } else {
-      v = threadIdx.x / SH::TPV;
-      tid = threadIdx.x % SH::TPV;
       const unsigned g = blockIdx.x * SH::VPB + v;
       ok = g < nvec;
       const unsigned gq = ok ? g / (unsigned)ncols : 0u;
@@ -682,6 +685,24 @@ struct ColMap {
   }
 };
 
+// Thread -> (vector, thread of the vector) on the two sides of a column
+// kernel. The T side (and both sides of rows and slots): a vector's threads
+// are neighbours, their elements of T contiguous. The spectrum side of groups:
+// kGroup neighbours hold one element of the group's slices, 64 contiguous
+// bytes. The two differ in the first and the last pass only, which exchange
+// through shared memory anyway (with the spectrum-side assignment in both, T
+// moved in 32-byte pieces: 14.5 us a column pass at P = 256, from 12).
+template <int P, int MODE, bool SPECTRUM>
+struct ColThread {
+  using SH = Shape<P>;
+  static constexpr bool G = MODE == kGroups && (SPECTRUM || RadixPlan<P>::NST == 1);
+  int v, tid;
+  __device__ __forceinline__ ColThread()
+      : v(G ? kGroup * ((int)threadIdx.x / (kGroup * SH::TPV)) + (int)threadIdx.x % kGroup
+            : (int)threadIdx.x / SH::TPV),
+        tid(G ? ((int)threadIdx.x / kGroup) % SH::TPV : (int)threadIdx.x % SH::TPV) {}
+};
+
 // Stage i, column pass: T[s][kx][0..n_in) zero-padded to P, FFT over y,
 // written to the spectrum `out` (row stride out_stride); with kSlots to
 // out[s][slot[kx * P + ky]] (the representative-slot layout; the transform
@@ -690,30 +711,30 @@ template <typename R, int P, int MODE, bool ZIN>
 __global__ void __launch_bounds__(kThreads) k_col_fwd(const cx<R>* __restrict__ T, int tstride,
                                                       int64_t tslice, int n_in, int ncols,
                                                       int64_t nvec, cx<R>* __restrict__ out,
-                                                      int64_t out_stride, int quad,
+                                                      int64_t out_stride, int group,
                                                       const cx<R>* __restrict__ tw_g,
                                                       const int* __restrict__ slot) {
   using SH = Shape<P>;
   using CM = ColMap<R, P, MODE>;
   cx<R>* tw;
   cx<R>* bufs = setup_smem<R, P>(tw_g, &tw);
-  const CM c(ncols, nvec, out_stride, quad);
-  const bool ok = c.ok;
-  const int tid = c.tid;
-  const cx<R>* src = T + c.s * tslice + c.kx * tstride;
-  cx<R>* dst = out + c.base;
-  cx<R>* b = bufs + c.v * CM::VS;
+  const ColThread<P, MODE, false> ti;
+  const ColThread<P, MODE, true> to;
+  const CM ci(ti.v, ncols, nvec, out_stride, group), co(to.v, ncols, nvec, out_stride, group);
+  const cx<R>* src = T + ci.s * tslice + ci.kx * tstride;
+  cx<R>* dst = out + co.base;
+  cx<R>* b = bufs + ti.v * CM::VS;
   pdl_wait();
   __syncthreads();
-  auto ld = [&](int y) -> cx<R> { return (ok && y < n_in) ? src[y] : mk<R>(0, 0); };
+  auto ld = [&](int y) -> cx<R> { return (ci.ok && y < n_in) ? src[y] : mk<R>(0, 0); };
   if constexpr (MODE == kSlots) {
-    const int* sl = slot + c.kx * P;
+    const int* sl = slot + ci.kx * P;
     NoStore<R> ns;
-    run_passes<R, P, 0, false, true, false, ZIN>(b, tw, tid, ld, ns);  // ends with a barrier
-    if (ok) {
+    run_passes<R, P, 0, false, true, false, ZIN>(b, tw, ti.tid, ld, ns);  // ends with a barrier
+    if (ci.ok) {
 #pragma unroll
       for (int i = 0; i < (P / 2 + SH::TPV) / SH::TPV; ++i) {
-        const int y = tid + i * SH::TPV;
+        const int y = ti.tid + i * SH::TPV;
         if (y > P / 2) break;
         const int s0 = __ldg(sl + y);
         if (y == 0 || y == P / 2) {
@@ -725,9 +746,10 @@ __global__ void __launch_bounds__(kThreads) k_col_fwd(const cx<R>* __restrict__ 
     }
   } else {
     auto st = [&](int y, cx<R> val) {
-      if (ok) dst[y * CM::STEP] = val;
+      if (co.ok) dst[y * CM::STEP] = val;
     };
-    run_passes<R, P, 0, false, true, true, ZIN>(b, tw, tid, ld, st);
+    run_passes<R, P, 0, false, true, true, ZIN>(b, tw, ti.tid, ld, st, bufs + to.v * CM::VS,
+                                                to.tid);
   }
 }
 
@@ -735,7 +757,7 @@ __global__ void __launch_bounds__(kThreads) k_col_fwd(const cx<R>* __restrict__ 
 // [0, n_out) kept (crop) into T[s][kx][y].
 template <typename R, int P, int MODE, bool HOUT>
 __global__ void __launch_bounds__(kThreads) k_col_inv(const cx<R>* __restrict__ in,
-                                                      int64_t in_stride, int quad, int ncols,
+                                                      int64_t in_stride, int group, int ncols,
                                                       int64_t nvec, cx<R>* __restrict__ T,
                                                       int tstride, int64_t tslice, int n_out,
                                                       const cx<R>* __restrict__ tw_g,
@@ -743,22 +765,24 @@ __global__ void __launch_bounds__(kThreads) k_col_inv(const cx<R>* __restrict__ 
   using CM = ColMap<R, P, MODE>;
   cx<R>* tw;
   cx<R>* bufs = setup_smem<R, P>(tw_g, &tw);
-  const CM c(ncols, nvec, in_stride, quad);
-  const bool ok = c.ok;
-  const cx<R>* src = in + c.base;
-  const int* sl = MODE == kSlots ? slot + c.kx * P : nullptr;
-  cx<R>* dst = T + c.s * tslice + c.kx * tstride;
+  const ColThread<P, MODE, true> ti;
+  const ColThread<P, MODE, false> to;
+  const CM ci(ti.v, ncols, nvec, in_stride, group), co(to.v, ncols, nvec, in_stride, group);
+  const cx<R>* src = in + ci.base;
+  const int* sl = MODE == kSlots ? slot + ci.kx * P : nullptr;
+  cx<R>* dst = T + co.s * tslice + co.kx * tstride;
   pdl_wait();
   __syncthreads();
   auto ld = [&](int y) -> cx<R> {
-    return ok ? src[MODE == kSlots ? __ldg(sl + y) : y * CM::STEP] : mk<R>(0, 0);
+    return ci.ok ? src[MODE == kSlots ? __ldg(sl + y) : y * CM::STEP] : mk<R>(0, 0);
   };
   auto st = [&](int y, cx<R> val) {
-    if (ok && y < n_out) dst[y] = val;
+    if (co.ok && y < n_out) dst[y] = val;
   };
   // (slot-mapped columns load element by element here: gathering mirror
   // pairs as 16-byte loads through the work vector measured slower)
-  run_passes<R, P, 0, true, true, true, false, HOUT>(bufs + c.v * CM::VS, tw, c.tid, ld, st);
+  run_passes<R, P, 0, true, true, true, false, HOUT>(bufs + ti.v * CM::VS, tw, ti.tid, ld, st,
+                                                     bufs + to.v * CM::VS, to.tid);
 }
 
 // Stage iii row pass, first half: the half spectra A = T[kx][y0], B =
@@ -1128,12 +1152,12 @@ cudaError_t col_fwd_t(const cx<R>* T, int tstride, int64_t tslice, int n_in, int
   cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  // quads: units of four slices (the last of a volume may hold fewer)
-  const int64_t units = MODE == kQuads ? (int64_t)(S / sr.quad) * ((sr.quad + 3) / 4) : S;
-  constexpr int per = MODE == kQuads ? SH::VPB / 4 : SH::VPB;
+  // groups: units of kGroup slices (the last of a volume may hold fewer)
+  const int64_t units = MODE == kGroups ? (int64_t)(S / sr.group) * ((sr.group + kGroup - 1) / kGroup) : S;
+  constexpr int per = MODE == kGroups ? SH::VPB / kGroup : SH::VPB;
   const int64_t nvec = units * ncols, blocks = (nvec + per - 1) / per;
   return launch_pdl(fn, dim3((unsigned)blocks), dim3(kThreads), smem, st, T, tstride, tslice, n_in,
-                    ncols, nvec, out, sr.stride, sr.quad, tw, sr.slot);
+                    ncols, nvec, out, sr.stride, sr.group, tw, sr.slot);
 }
 
 template <typename R, int P, int MODE>
@@ -1146,10 +1170,10 @@ cudaError_t col_inv_t(const cx<R>* in, const SpecRow& sr, int ncols, int S, cx<R
   cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  const int64_t units = MODE == kQuads ? (int64_t)(S / sr.quad) * ((sr.quad + 3) / 4) : S;
-  constexpr int per = MODE == kQuads ? SH::VPB / 4 : SH::VPB;
+  const int64_t units = MODE == kGroups ? (int64_t)(S / sr.group) * ((sr.group + kGroup - 1) / kGroup) : S;
+  constexpr int per = MODE == kGroups ? SH::VPB / kGroup : SH::VPB;
   const int64_t nvec = units * ncols, blocks = (nvec + per - 1) / per;
-  return launch_pdl(fn, dim3((unsigned)blocks), dim3(kThreads), smem, st, in, sr.stride, sr.quad,
+  return launch_pdl(fn, dim3((unsigned)blocks), dim3(kThreads), smem, st, in, sr.stride, sr.group,
                     ncols, nvec, T, tstride, tslice, n_out, tw, sr.slot);
 }
 }  // namespace
@@ -1158,7 +1182,7 @@ template <typename R, int P>
 cudaError_t FftLen<R, P>::col_fwd(const cx<R>* T, int tstride, int64_t tslice, int n_in, int ncols, int S,
                                   cx<R>* out, const SpecRow& sr, const cx<R>* tw, cudaStream_t st) {
   if constexpr (sizeof(R) == 4) {  // double-precision plans do not fold
-    if (sr.quad) return col_fwd_t<R, P, kQuads>(T, tstride, tslice, n_in, ncols, S, out, sr, tw, st);
+    if (sr.group) return col_fwd_t<R, P, kGroups>(T, tstride, tslice, n_in, ncols, S, out, sr, tw, st);
   }
   return sr.slot ? col_fwd_t<R, P, kSlots>(T, tstride, tslice, n_in, ncols, S, out, sr, tw, st)
                  : col_fwd_t<R, P, kRows>(T, tstride, tslice, n_in, ncols, S, out, sr, tw, st);
@@ -1168,7 +1192,7 @@ template <typename R, int P>
 cudaError_t FftLen<R, P>::col_inv(const cx<R>* in, const SpecRow& sr, int ncols, int S, cx<R>* T, int tstride,
                                   int64_t tslice, int n_out, const cx<R>* tw, cudaStream_t st) {
   if constexpr (sizeof(R) == 4) {
-    if (sr.quad) return col_inv_t<R, P, kQuads>(in, sr, ncols, S, T, tstride, tslice, n_out, tw, st);
+    if (sr.group) return col_inv_t<R, P, kGroups>(in, sr, ncols, S, T, tstride, tslice, n_out, tw, st);
   }
   return sr.slot ? col_inv_t<R, P, kSlots>(in, sr, ncols, S, T, tstride, tslice, n_out, tw, st)
                  : col_inv_t<R, P, kRows>(in, sr, ncols, S, T, tstride, tslice, n_out, tw, st);

@@ -207,10 +207,7 @@ struct Plan {
   // the representative of each bin
   int* fold_members = nullptr;  // [Upad][4]
   int* fold_rep = nullptr;      // [K]
-  // Slot layout of the spectra on the batched tensor-core path: row [Upad][4]
-  // complex, bin k at fold_slot[k] = 4 u + i (the i-th member of its
-  // representative u), so a representative's bins share one 32-byte sector.
-  int* fold_slot = nullptr;     // [K]
+  int* fold_order = nullptr;    // [U] representatives in 8 x 8 tiles of (a, b)
   double fold_deviation = 0;    // max |Hh(bin) - Hh(representative)| seen (stored scale)
   double radial_deviation = 0;  // max |Hh(representative) - Hh(its stored row)| (user tables)
   // Block maps of the CUDA-core contraction (device): the bins of the
@@ -318,15 +315,17 @@ int cuda_fail(cudaError_t e, const char* what);
 // Launchers (each returns cudaError_t of the launch).
 // ----------------------------------------------------------------------------
 // Where the spectra of a run of slices live: one row of `stride` complex
-// values per slice (bin k at k, or at slot[k] with `slot`), or with quad > 0
-// (slices per volume) four slices interleaved: volume v's slice s, bin k at
-// ((v ceil(quad / 4) + s / 4) stride + k) 4 + s % 4. A bin's four slices are
-// then one 32-byte sector, which the contraction of a folded table needs (its
-// bins are scattered), and a column of four slices stays contiguous.
+// values per slice (bin k at k, or at slot[k] with `slot`), or with group > 0
+// (slices per volume) kGroup slices interleaved: volume v's slice s, bin k at
+// ((v ceil(group / 8) + s / 8) stride + k) 8 + s % 8. A bin's eight slices are
+// then 64 contiguous bytes, which the contraction of a folded table needs (its
+// bins are scattered, and DRAM moves 64 bytes at a time), and a column of
+// eight slices stays contiguous for the transforms.
+constexpr int kGroup = 8;
 struct SpecRow {
   int64_t stride = 0;
   const int* slot = nullptr;
-  int quad = 0;
+  int group = 0;
 };
 // FFT stages. `in`/`out` element type follows L.fp64.
 // Stage i: real slices [S][ny][nx] (slice stride in_stride elements, row
@@ -379,34 +378,33 @@ cudaError_t launch_spectrum_rows(const Plan& p, const void* in, int64_t in_strid
 cudaError_t launch_spectrum_cols(const Plan& p, int ny_in, void* out, const SpecRow& sr, int S,
                                  cudaStream_t s);
 // Contractions over the resident table (tensor cores when the plan has the
-// split tables and batch >= tc_min_batch). quad: the spectra of a folded plan
-// on the CUDA cores are in quads (SpecRow), else one row of Kpad bins a slice.
+// split tables and batch >= tc_min_batch). grouped: the spectra of a folded
+// plan interleave kGroup slices (SpecRow); else one row of Kpad bins a slice, or of slots on the
+// tensor cores (tc_slots).
 cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s,
-                                bool quad = false);
+                                bool grouped = false);
 cudaError_t launch_contract_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s,
-                                bool quad = false);
+                                bool grouped = false);
 
-// The batched tensor-core contraction of a folded plan reads and writes
-// spectra in the representative-slot layout (rows of 4 * Upad complex
-// values, bin k at fold_slot[k]); every other path uses rows of Kpad bins.
+// Batched tensor-core contraction of a folded plan. pat_stage_contract_slots
+// runs it on spectra in the representative-slot layout (rows of 4 * Upad
+// complex values, bin k at 4 u + i); the plan's own spectra are grouped.
 inline bool tc_slots(const Plan& p, int batch) {
   return p.tc_fwd && p.L.fold && p.tc_min_batch > 0 && batch >= p.tc_min_batch;
 }
 inline int64_t slot_row(const Layout& L) { return 4 * L.Upad; }
-// Layout of the plan's own spectra of `n` slices per volume at this batch:
-// slots for the folded tensor-core path, quads for the folded CUDA-core path
-// (whole sectors for its scattered bins: see contract.cu), else rows of Kpad.
-inline SpecRow spec_row(const Plan& p, int batch, int n) {
+// Layout of the plan's own spectra of `n` slices per volume: grouped slices on
+// folded plans (their bins are scattered: see contract.cu and tc_contract.cu),
+// else rows of Kpad.
+inline SpecRow spec_row(const Plan& p, int n) {
   SpecRow r;
-  const bool sl = tc_slots(p, batch);
-  r.stride = sl ? slot_row(p.L) : p.L.Kpad;
-  r.slot = sl ? p.fold_slot : nullptr;
-  r.quad = !sl && p.L.fold ? n : 0;
+  r.stride = p.L.Kpad;
+  r.group = p.L.fold ? n : 0;
   return r;
 }
-// [S][Kpad] bins -> [S][4 Upad] slots and back (single precision).
-cudaError_t launch_to_slots(const Plan& p, const void* in, void* out, int64_t S, cudaStream_t s);
-cudaError_t launch_from_slots(const Plan& p, const void* in, void* out, int64_t S,
+// [S][Kpad] rows -> grouped slices and back (S a multiple of kGroup; single precision).
+cudaError_t launch_to_groups(const Plan& p, const void* in, void* out, int64_t S, cudaStream_t s);
+cudaError_t launch_from_groups(const Plan& p, const void* in, void* out, int64_t S,
                               cudaStream_t s);
 // Split-BF16 tensor-core contraction (tc_contract.cu).
 bool tc_supported(const Layout& L);
@@ -414,7 +412,7 @@ size_t tc_table_bytes(const Layout& L);  // one direction
 cudaError_t tc_build_tables(const Plan& p, void* fwd, void* adj, cudaStream_t s);
 cudaError_t tc_contract(const Plan& p, const void* tables_fwd, const void* tables_adj,
                         const void* in, void* out, int batch, bool adjoint, int* err,
-                        cudaStream_t s);
+                        cudaStream_t s, bool grouped);
 // Default pipeline wait limit of the tensor-core kernels (polls of
 // mbarrier.try_wait per wait; a few seconds).
 constexpr int64_t kTcSpinDefault = int64_t(1) << 22;

@@ -397,8 +397,17 @@ int build_fold_maps(Plan& p, std::vector<int>* members_out) {
   for (int64_t k = 0; k < L.K; ++k)
     if (rep[k] < 0) return fail(PAT_ERR_CUDA, "internal: a bin without representative");
   if (members_out) *members_out = members;
-  PAT_CUDA(dev_alloc(&p.fold_slot, slot.size() * sizeof(int)));
-  PAT_CUDA(cudaMemcpy(p.fold_slot, slot.data(), slot.size() * sizeof(int),
+  // processing order of the tensor-core contraction: 8 x 8 tiles of (a, b)
+  std::vector<int64_t> key((size_t)L.U);
+  std::vector<int> order((size_t)L.U);
+  for (int64_t u = 0; u < L.U; ++u) {
+    const int64_t a = members[4 * u] / L.py, b = members[4 * u] % L.py;
+    key[u] = ((a / 8) * (L.py + 8) + b / 8) * 64 + (a % 8) * 8 + b % 8;
+    order[u] = (int)u;
+  }
+  std::sort(order.begin(), order.end(), [&](int x, int y) { return key[x] < key[y]; });
+  PAT_CUDA(dev_alloc(&p.fold_order, order.size() * sizeof(int)));
+  PAT_CUDA(cudaMemcpy(p.fold_order, order.data(), order.size() * sizeof(int),
                       cudaMemcpyHostToDevice));
   PAT_CUDA(dev_alloc(&p.fold_members, members.size() * sizeof(int)));
   PAT_CUDA(dev_alloc(&p.fold_rep, rep.size() * sizeof(int)));
@@ -658,8 +667,8 @@ int build_table_from_source(Plan& p, const void* table, pat_table_format fmt, bo
     } else {
       dev_free(p.fold_members);
       dev_free(p.fold_rep);
-      dev_free(p.fold_slot);
-      p.fold_members = p.fold_rep = p.fold_slot = nullptr;
+      dev_free(p.fold_order);
+      p.fold_members = p.fold_rep = p.fold_order = nullptr;
     }
   }
   return PAT_OK;

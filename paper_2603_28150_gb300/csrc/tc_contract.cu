@@ -24,13 +24,16 @@
 //
 // D4-folded plans (k_tc_fold) keep one tile set per representative {|kx|,
 // |ky|} (a quarter of the bytes) and put its up to 4 bins side by side in the
-// MMA's N dimension (N = 4 x 32); their spectra use the representative-slot
-// layout (a representative's 4 bins in one 32-byte sector of every row), so
-// a representative's operand chunk is a 3D box (32 bytes x 128 rows x 16
-// volumes) that one tensor copy moves.
+// MMA's N dimension (N = 4 x 32). Their spectra interleave eight slices per bin
+// (SpecRow's groups), so a member's operand chunk is a 3D box (64 bytes = eight
+// slices of one bin, x 16 groups x 16 volumes) that one tensor copy moves, and
+// the column transforms on the other side stay contiguous.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+
+#include <algorithm>
+#include <utility>
 
 #include "pat_internal.h"
 
@@ -389,6 +392,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_contract(Params p) {
 // row n = m * 32 + h * 16 + b is the real (h = 0) or imaginary (h = 1) part of
 // volume b at bin members[u][m], so one pass over u's tiles serves all 4 bins
 // (the table is read once per representative instead of once per bin).
+// GRP: grouped spectra, one 16 KB box per member; else in the
+// representative-slot layout of pat_stage_contract_slots (a representative's 4
+// bins in one 32-byte sector of every row), one 64 KB box. Representatives are
+// taken in the order of `order`, 8 x 8 tiles of (a, b), so that the bins next
+// to a member's are in use at about the same time (adjoint 880 us, 1310 in the
+// order of u). 16 volumes at 128^2 -> 256^2 x 128 x 512: 813 / 794 us forward /
+// adjoint, 833 / 839 on slots, whose column transforms moved 8 of every 32 bytes
+// (2140 us of a pair's 4550; grouped 1190 of 3500). With groups of four slices
+// the forward took 1450 us: 2.2 GB of results leave for DRAM in pieces of 32
+// bytes, half of what it moves at a time.
 // Warp roles (192 threads): warp 0 streams the table tiles (cp.async.bulk,
 // kFS-slot ring); warp 1 issues the MMAs (and, in the adjoint, stages each
 // operand chunk by one 3D tensor copy as soon as the previous one has been
@@ -407,15 +420,17 @@ constexpr int kFThreads = 192;
 constexpr int kFN = 128;                  // MMA N: 4 members x (re, im) x 16 volumes
 constexpr int kFBBytes = kFN * kTile * 2;  // one part (hi or lo) of a B chunk: 32 KB
 // staged FP32 operand chunk: 16 volumes x 128 rows x one representative's 4
-// complex members (32 bytes)
+// complex members
 constexpr int kStageBytes = kVB * kTile * 32;
+constexpr int kMemBytes = kStageBytes / 4;  // one member's box (GRP)
 
 struct FoldParams {
   const unsigned char* table;  // split tiles of this direction, per representative
   const int4* members;         // [U] bins of each representative (-1 = none)
-  const float2* in;            // X [b][nz][srow] (fwd) or D [b][nt][srow] (adj), slot layout
-  float2* out;                 // Y [b][nt][srow] (fwd) or Z [b][nz][srow] (adj), slot layout
-  int64_t U, srow;
+  const int* order;            // [U] representatives in processing order
+  const float2* in;            // X (fwd) or D (adj)
+  float2* out;                 // Y (fwd) or Z (adj)
+  int64_t U, srow;             // complex values per row: slots, or bins (Kpad) of a group
   int batch;
   int rows_in, rows_out;  // nz, nt (fwd) or nt, nz (adj)
   int R;                  // tile rows per representative: mtiles (fwd) or kchunks (adj)
@@ -471,14 +486,16 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-template <bool ADJ>
+template <bool ADJ, bool GRP>
 __global__ void __launch_bounds__(kFThreads, 1)
     k_tc_fold(FoldParams p, const __grid_constant__ CUtensorMap tin,
               const __grid_constant__ CUtensorMap tout) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* slots = smem;                               // [kFS][32 KB]
   unsigned char* bbuf = smem + (size_t)kFS * kTileBytes;     // [hi 32 KB | lo 32 KB]
-  unsigned char* stage = bbuf + 2 * (size_t)kFBBytes;        // in: [128 rows][16 b][8 floats]; out: [16 b][128 rows][8 floats]
+  // staging, in: [128 rows][16 b][8 floats], out: [16 b][128 rows][8 floats];
+  // GRP, in only: [4 members][16 groups][16 b][16 floats], its 16-byte quarters swizzled
+  unsigned char* stage = bbuf + 2 * (size_t)kFBBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(stage + kStageBytes);
   uint64_t* full = bars;             // [kFS] tile landed
   uint64_t* empty = bars + kFS;      // [kFS] tile consumed by the MMAs
@@ -530,6 +547,21 @@ __global__ void __launch_bounds__(kFThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_base_s;
+  // Copies row chunk `kc` of representative u into the staging buffer (one thread).
+  auto load_chunk = [&](int64_t u, int kc) {
+    if constexpr (GRP) {
+      const int4 mem = p.members[u];
+      const int n = (mem.x >= 0) + (mem.y >= 0) + (mem.z >= 0) + (mem.w >= 0);
+      mbar_arrive_expect_tx(sfull, (uint32_t)(n * kMemBytes));
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        if (member(mem, m) >= 0)
+          tma_load_3d(stage + m * kMemBytes, &tin, 2 * kGroup * member(mem, m), 0, kc * (kTile / kGroup), sfull);
+    } else {
+      mbar_arrive_expect_tx(sfull, kStageBytes);
+      tma_load_3d(stage, &tin, (int)(8 * u), 0, kc * kTile, sfull);
+    }
+  };
   int64_t issued = 0;  // table tiles copied (warp 0)
   int64_t staged = 0;  // operand chunks staged (warp 1)
 
@@ -542,7 +574,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
           !fwait_warp(&empty[s], (uint32_t)(((j / kFS) - 1) & 1), abort_s, p.spin))
         break;
       if (lane == 0) {
-        const int64_t u = blockIdx.x + (j / (2 * R)) * gridDim.x;
+        const int64_t u = p.order[blockIdx.x + (j / (2 * R)) * gridDim.x];
         const int64_t tile = u * 2 * R + j % (2 * R);
         mbar_arrive_expect_tx(&full[s], kTileBytes);
         bulk_g2s(slots + (size_t)s * kTileBytes, p.table + tile * (int64_t)kTileBytes, kTileBytes,
@@ -564,9 +596,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
     const int64_t nchunks = nmine * NB;
     auto stage_chunk = [&](int64_t c) {
       if (lane == 0) {
-        const int64_t u = blockIdx.x + (c / NB) * gridDim.x;
-        mbar_arrive_expect_tx(sfull, kStageBytes);
-        tma_load_3d(stage, &tin, (int)(8 * u), 0, (int)(c % NB) * kTile, sfull);
+        load_chunk(p.order[blockIdx.x + (c / NB) * gridDim.x], (int)(c % NB));
       }
       staged = c + 1;
       __syncwarp();
@@ -625,30 +655,41 @@ __global__ void __launch_bounds__(kFThreads, 1)
     // ---- gather + split (B operand) and epilogue (accumulators -> Y / Z)
     const int ct = tid - 64;     // 0..127
     const int quarter = warp & 3;  // TMEM lanes 32 * quarter ... of this warp
-    // Operands in the slot layout: row (b, r) of X / D holds the 4 members of
-    // representative u at [4u, 4u + 4) of its srow complex values (32 bytes).
+    // Slots: row (b, r) of X / D holds the 4 members of representative u at
+    // [4u, 4u + 4) of its srow complex values (32 bytes). Groups: 64 bytes
+    // hold 8 rows of one member.
     auto gather = [&](int64_t i, int kc, int64_t c) -> bool {
       (void)kc;
       if (!fwait_warp(sfull, (uint32_t)(c & 1), abort_s, p.spin)) return false;
       tc_fence_after();
-      const int64_t u = blockIdx.x + i * gridDim.x;
+      const int64_t u = p.order[blockIdx.x + i * gridDim.x];
       const int4 mem = p.members[u];
       unsigned char* bh = bbuf;
       const float* sf = reinterpret_cast<const float*>(stage);
       // items (b, octet of rows): 16 x 16, two per thread; both read out of
       // the staging buffer first, so (adjoint) the next chunk's copy can start
       // while this one is converted
-      float4 lo4s[2][8], hi4s[2][8];  // members (0, 1) and (2, 3) of 8 rows
+      // slots: members (0, 1) / (2, 3) of 8 rows; groups: rows 4 (q & 1) + (0, 1) /
+      // (2, 3) of member q >> 1
+      float4 lo4s[2][8], hi4s[2][8];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const int it = ct + k * 128;
         const int b = it & 15, oct = it >> 4;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-          const float4* src =
-              reinterpret_cast<const float4*>(sf + ((size_t)(oct * 8 + q) * kVB + b) * 8);
-          lo4s[k][q] = src[0];
-          hi4s[k][q] = src[1];
+          if constexpr (GRP) {  // 64-byte swizzle: quarter c of row b sits at c ^ (b >> 1 & 3)
+            const float4* src = reinterpret_cast<const float4*>(
+                sf + (((q >> 1) * (kTile / kGroup) + oct) * kVB + b) * 16);
+            const int sw = (b >> 1) & 3;
+            lo4s[k][q] = src[(2 * (q & 1)) ^ sw];
+            hi4s[k][q] = src[(2 * (q & 1) + 1) ^ sw];
+          } else {
+            const float4* src =
+                reinterpret_cast<const float4*>(sf + ((size_t)(oct * 8 + q) * kVB + b) * 8);
+            lo4s[k][q] = src[0];
+            hi4s[k][q] = src[1];
+          }
         }
       }
       if (ADJ) {
@@ -669,9 +710,17 @@ __global__ void __launch_bounds__(kFThreads, 1)
           float re[8], im[8];
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
-            const float4 w = m < 2 ? lo4[q] : hi4[q];
-            re[q] = present ? ((m & 1) ? w.z : w.x) : 0.f;
-            im[q] = present ? ((m & 1) ? w.w : w.y) : 0.f;
+            float4 w;
+            bool second;
+            if constexpr (GRP) {  // row q: pair (q >> 1) & 1 of half q >> 2
+              w = (q & 2) ? hi4[2 * m + (q >> 2)] : lo4[2 * m + (q >> 2)];
+              second = q & 1;
+            } else {
+              w = m < 2 ? lo4[q] : hi4[q];
+              second = m & 1;
+            }
+            re[q] = present ? (second ? w.z : w.x) : 0.f;
+            im[q] = present ? (second ? w.w : w.y) : 0.f;
           }
           uint4 h, l;
           split8(re, &h, &l);
@@ -686,13 +735,27 @@ __global__ void __launch_bounds__(kFThreads, 1)
       mbar_arrive(bready);
       return true;
     };
+    // Groups: row `row` of volumes [b0, b1) of u's members; eight lanes (rows)
+    // fill a member's 64 bytes.
+    auto store_rows = [&](int64_t u, int row, int b0, int b1, const float (*v)[32]) {
+      const int4 mem = p.members[u];
+#pragma unroll
+      for (int bb = 0; bb < kVB; ++bb) {
+        if (bb < b0 || bb >= b1 || bb >= p.batch) continue;
+        float2* o = p.out + (int64_t)(bb * p.rows_out + row / kGroup * kGroup) * p.srow + row % kGroup;
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+          if (member(mem, m) >= 0)
+            o[kGroup * (int64_t)member(mem, m)] = make_float2(v[m][bb], v[m][16 + bb]);
+      }
+    };
     // Adjoint drain of representative i in `parts` shares of the volumes:
     // share `part` stores volumes [part * 16 / parts, (part + 1) * 16 / parts).
     auto epilogue_adj = [&](int64_t i, int part, int parts) -> bool {
       if (part == 0 && !fwait_warp(&afull[i & 1], (uint32_t)((i >> 1) & 1), abort_s, p.spin))
         return false;
       tc_fence_after();
-      const int64_t u = blockIdx.x + i * gridDim.x;
+      const int64_t u = p.order[blockIdx.x + i * gridDim.x];
       const int row = quarter * 32 + lane;
       const int b0 = part * kVB / parts, b1 = (part + 1) * kVB / parts;
       float v[4][32];
@@ -702,19 +765,20 @@ __global__ void __launch_bounds__(kFThreads, 1)
         tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + col + (uint32_t)(m * 32), v[m]);
 #pragma unroll
       for (int bb = 0; bb < kVB; ++bb) {
-        if (bb < b0 || bb >= b1 || bb >= p.batch) continue;
+        if (GRP || bb < b0 || bb >= b1 || bb >= p.batch) continue;
         float4* o =
             reinterpret_cast<float4*>(p.out + ((int64_t)bb * p.rows_out + row) * p.srow + 4 * u);
         o[0] = make_float4(v[0][bb], v[0][16 + bb], v[1][bb], v[1][16 + bb]);
         o[1] = make_float4(v[2][bb], v[2][16 + bb], v[3][bb], v[3][16 + bb]);
       }
+      if constexpr (GRP) store_rows(u, row, b0, b1, v);
       if (part == parts - 1) {
         tc_fence_before();
         mbar_arrive(&aempty[i & 1]);
       }
       return true;
     };
-    // ---- forward: the staging buffer alternates between the X chunk of the
+    // ---- forward (slots): the staging buffer alternates between the X chunk of the
     // next representative and the output tiles of the current one, which
     // leave by 3D tensor stores (one per 128-sample tile: 16 volumes x 128
     // rows x 32 bytes; volumes past the batch are not written).
@@ -728,16 +792,14 @@ __global__ void __launch_bounds__(kFThreads, 1)
     int64_t fstaged = 0;  // forward X chunks staged (thread ct 0)
     auto stage_x = [&](int64_t i) {
       if (ct == 0) {
-        const int64_t u = blockIdx.x + i * gridDim.x;
-        mbar_arrive_expect_tx(sfull, kStageBytes);
-        tma_load_3d(stage, &tin, (int)(8 * u), 0, 0, sfull);
+        load_chunk(p.order[blockIdx.x + i * gridDim.x], 0);
         fstaged = i + 1;
       }
     };
     auto epilogue_fwd = [&](int64_t i, int a, int64_t q) -> bool {
       if (!fwait_warp(&afull[q & 1], (uint32_t)((q >> 1) & 1), abort_s, p.spin)) return false;
       tc_fence_after();
-      const int64_t u = blockIdx.x + i * gridDim.x;
+      const int64_t u = p.order[blockIdx.x + i * gridDim.x];
       const int nmt = min(2, R - 2 * a);
       const int r = quarter * 32 + lane;  // row of the 128-sample tile
       float* sf = reinterpret_cast<float*>(stage);
@@ -747,6 +809,10 @@ __global__ void __launch_bounds__(kFThreads, 1)
 #pragma unroll
         for (int m = 0; m < 4; ++m)
           tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + col + (uint32_t)(m * 32), v[m]);
+        if constexpr (GRP) {
+          store_rows(u, (2 * a + h) * kTile + r, 0, kVB, v);
+          continue;
+        }
         // the staging buffer is free (X read out, previous tile's store read)
         if (!gsync()) return false;
 #pragma unroll
@@ -780,10 +846,14 @@ __global__ void __launch_bounds__(kFThreads, 1)
       }
       for (int64_t i = 0; i < nmine && ok; ++i) {
         if (i + 1 < nmine) ok = gather(i + 1, 0, i + 1);
+        if (GRP && ok && i + 2 < nmine) {  // X(i + 1) read out by every warp
+          ok = gsync();
+          if (ok) stage_x(i + 2);
+        }
         for (int a = 0; a < NA && ok; ++a) ok = epilogue_fwd(i, a, i * NA + a);
         // thread ct 0 waited for its last store's read; the others wrote the
         // tile before the barrier that preceded it
-        if (ok && i + 2 < nmine) stage_x(i + 2);
+        if (!GRP && ok && i + 2 < nmine) stage_x(i + 2);
       }
       // after an abort: the staging copy still in flight lands before the
       // shared memory is released, and every store has read its tile
@@ -909,10 +979,12 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
                                    const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Tensor map of the operand (or result) spectra of one pass of up to 16 volumes in the
-// representative-slot layout, seen as FP32 [nb][rows][2 srow]: a box of 8
-// floats x 128 rows x 16 volumes is one representative's operand chunk
-// (volumes past nb read as zero). With rows_outer the map's dimensions are
+// Tensor map of the operand (or result) spectra of one pass of up to 16 volumes, seen
+// as FP32 [nb][rows][2 srow] (slots) or [nb][rows / 8][16 srow] (groups): a box of
+// 8 floats x 128 rows x 16 volumes is the operand chunk of one representative, of
+// 16 floats x 16 groups x 16 volumes that of one member (64-byte swizzle: the
+// gather threads of neighbouring volumes then read different banks), volumes past
+// nb reading as zero. With rows_outer the map's dimensions are
 // ordered (x, volume, row), so the box lands in shared memory as
 // [row][volume][8 floats] and the gather threads of one row octet read
 // neighbouring 32-byte groups. The encoder comes from the driver at run
@@ -928,24 +1000,25 @@ EncodeTiledFn load_encoder() {
 }
 
 cudaError_t encode_operand_map(CUtensorMap* map, const void* base, int64_t srow, int rows,
-                               int nb, bool rows_outer = false) {
+                               int nb, bool grouped, bool rows_outer = false) {
   static const EncodeTiledFn encode = load_encoder();  // resolved once, thread-safe
   if (!encode) return cudaErrorNotSupported;
-  cuuint64_t dims[3] = {(cuuint64_t)(2 * srow), (cuuint64_t)rows, (cuuint64_t)nb};
-  cuuint64_t strides[2] = {(cuuint64_t)(srow * 8), (cuuint64_t)(srow * 8 * rows)};
-  cuuint32_t box[3] = {8, (cuuint32_t)tc::kTile, (cuuint32_t)tc::kVB};
+  const int per = grouped ? kGroup : 1;  // slices per row of the map
+  const cuuint64_t nrow = (cuuint64_t)(rows / per), rbytes = (cuuint64_t)srow * 8 * per;
+  const cuuint32_t brow = (cuuint32_t)(tc::kTile / per);
+  cuuint64_t dims[3] = {(cuuint64_t)(2 * srow * per), nrow, (cuuint64_t)nb};
+  cuuint64_t strides[2] = {rbytes, rbytes * nrow};
+  cuuint32_t box[3] = {grouped ? 2u * kGroup : 8u, brow, (cuuint32_t)tc::kVB};
   if (rows_outer) {
-    dims[1] = (cuuint64_t)nb;
-    dims[2] = (cuuint64_t)rows;
-    strides[0] = (cuuint64_t)(srow * 8 * rows);
-    strides[1] = (cuuint64_t)(srow * 8);
-    box[1] = (cuuint32_t)tc::kVB;
-    box[2] = (cuuint32_t)tc::kTile;
+    std::swap(dims[1], dims[2]);
+    std::swap(strides[0], strides[1]);
+    std::swap(box[1], box[2]);
   }
   const cuuint32_t step[3] = {1, 1, 1};
   const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims,
                             strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                            grouped ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
@@ -956,7 +1029,7 @@ cudaError_t encode_operand_map(CUtensorMap* map, const void* base, int64_t srow,
 // passes of 16 through the tensor cores.
 cudaError_t tc_contract(const Plan& p, const void* tables_fwd, const void* tables_adj,
                         const void* in, void* out, int batch, bool adjoint, int* err,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool grouped) {
   const Layout& L = p.L;
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -964,7 +1037,9 @@ cudaError_t tc_contract(const Plan& p, const void* tables_fwd, const void* table
   if (e != cudaSuccess) return e;
   if (L.fold) {
     const size_t smem = tc::fold_smem();
-    auto fn = adjoint ? tc::k_tc_fold<true> : tc::k_tc_fold<false>;
+    auto fn = grouped ? (adjoint ? tc::k_tc_fold<true, true> : tc::k_tc_fold<false, true>)
+                   : (adjoint ? tc::k_tc_fold<true, false> : tc::k_tc_fold<false, false>);
+    const int64_t srow = grouped ? L.Kpad : slot_row(L);
     e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     if (e != cudaSuccess) return e;
@@ -973,10 +1048,11 @@ cudaError_t tc_contract(const Plan& p, const void* tables_fwd, const void* table
       tc::FoldParams q;
       q.table = static_cast<const unsigned char*>(adjoint ? tables_adj : tables_fwd);
       q.members = reinterpret_cast<const int4*>(p.fold_members);
-      q.in = static_cast<const float2*>(in) + (int64_t)b0 * rows_in * 4 * L.Upad;
-      q.out = static_cast<float2*>(out) + (int64_t)b0 * rows_out * 4 * L.Upad;
+      q.order = p.fold_order;
+      q.in = static_cast<const float2*>(in) + (int64_t)b0 * rows_in * srow;
+      q.out = static_cast<float2*>(out) + (int64_t)b0 * rows_out * srow;
       q.U = L.U;
-      q.srow = 4 * L.Upad;
+      q.srow = srow;
       q.batch = std::min(tc::kVB, batch - b0);
       q.rows_in = rows_in;
       q.rows_out = rows_out;
@@ -984,8 +1060,9 @@ cudaError_t tc_contract(const Plan& p, const void* tables_fwd, const void* table
       q.err = err;
       q.spin = (uint32_t)p.tc_spin;
       CUtensorMap map_in, map_out;
-      if ((e = encode_operand_map(&map_in, q.in, q.srow, rows_in, q.batch, true)) != cudaSuccess ||
-          (e = encode_operand_map(&map_out, q.out, q.srow, rows_out, q.batch)) != cudaSuccess)
+      if ((e = encode_operand_map(&map_in, q.in, srow, rows_in, q.batch, grouped, true)) !=
+              cudaSuccess ||
+          (e = encode_operand_map(&map_out, q.out, srow, rows_out, q.batch, grouped)) != cudaSuccess)
         return e;
       const int grid = (int)std::min<int64_t>(L.U, sms);
       fn<<<grid, tc::kFThreads, smem, s>>>(q, map_in, map_out);

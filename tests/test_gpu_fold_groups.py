@@ -1,6 +1,6 @@
-"""Folded CUDA-core contraction on spectra interleaved by four slices: depth
-and time counts around the tiles (quads of slices, blocks of 4 / 8 samples,
-stages, rings, z-chunks, the second pass past 128 depths), every transform
+"""Folded CUDA-core contraction on spectra interleaved by eight slices: depth
+and time counts around the tiles (groups and quads of slices, blocks of 4 / 8
+samples, stages, rings, z-chunks, the second pass past 128 depths), every transform
 length's thread layout, several volumes, and the plain layout of the stage
 entry point, against the FP64 oracle (FP32 target: 1e-5 relative l2)."""
 import numpy as np
@@ -12,7 +12,7 @@ from tests.helpers import cuda, host
 
 pytestmark = pytest.mark.gpu
 
-# (n, P, nz, nt, B): the smallest counts, one past and one short of a quad,
+# (n, P, nz, nt, B): the smallest counts, one past and one short of a group,
 # ragged time blocks, few and many z-groups, the largest depth count
 SHAPES = [(8, 16, 1, 1, 1), (8, 16, 3, 2, 2), (12, 24, 4, 3, 1), (16, 32, 5, 5, 3),
           (24, 48, 17, 13, 1), (32, 64, 9, 65, 2), (48, 96, 33, 31, 1), (64, 128, 49, 40, 1),
@@ -22,7 +22,7 @@ SHAPES = [(8, 16, 1, 1, 1), (8, 16, 3, 2, 2), (12, 24, 4, 3, 1), (16, 32, 5, 5, 
 
 
 @pytest.mark.parametrize("n,P,nz,nt,B", SHAPES, ids=[str(s) for s in SHAPES])
-def test_folded_quads_match_oracle(n, P, nz, nt, B):
+def test_folded_groups_match_oracle(n, P, nz, nt, B):
     import torch
     g = oracle.Grid(nx=n, ny=max(1, n - 3), nz=nz, nt=nt, px=P, py=P)
     h = synth.random_kernels(nz, nt, P, P, seed=n + nz, d4=True)
