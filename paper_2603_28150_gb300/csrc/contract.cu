@@ -291,9 +291,10 @@ template <bool GRP>
 __device__ __forceinline__ void store_quad(cx<float>* out, int q, int bin, int n, int64_t Kpad,
                                            cx<float> a, cx<float> b, cx<float> c, cx<float> d) {
   if constexpr (GRP) {  // slices at or past n are padding that no reader uses
-    float4* o = reinterpret_cast<float4*>(out + group_off(q, bin, Kpad));
-    o[0] = make_float4(a.x, a.y, b.x, b.y);
-    o[1] = make_float4(c.x, c.y, d.x, d.y);
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                     out + group_off(q, bin, Kpad)),
+                 "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y), "f"(d.x), "f"(d.y)
+                 : "memory");
   } else {
     cx<float>* o = out + (int64_t)(4 * q) * Kpad + bin;
     if (4 * q < n) o[0] = a;
