@@ -285,7 +285,8 @@ int pat_plan_set_sensor_response(pat_plan* plan, const double* r, int nr, pat_st
 
 /* Synchronises the device and reports whether any bounded device-side wait of
  * the plan's kernels gave up since the last check (PAT_ERR_TIMEOUT; the flag
- * is cleared), else PAT_OK. */
+ * is cleared), else PAT_OK. The folded contraction's waits for its table
+ * copies have a fixed limit (2^22 tests). */
 int pat_plan_check(pat_plan* plan);
 
 /* Limit of the pipeline waits of the tensor-core contraction (the mbarrier

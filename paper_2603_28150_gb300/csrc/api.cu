@@ -740,7 +740,7 @@ int pat_plan_check(pat_plan* plan) {
   PAT_CUDA(cudaMemcpy(&h, plan->p.tc_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (h) {
     PAT_CUDA(cudaMemset(plan->p.tc_err, 0, sizeof(int)));
-    return fail(PAT_ERR_TIMEOUT, "a bounded wait of the tensor-core contraction gave up");
+    return fail(PAT_ERR_TIMEOUT, "a bounded wait of a contraction kernel gave up");
   }
   return PAT_OK;
   PAT_GUARD_END

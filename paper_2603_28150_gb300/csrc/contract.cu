@@ -15,6 +15,7 @@
 // imaginary parts of X are contracted by the same real coefficient.
 #include <algorithm>
 
+#include "async.cuh"
 #include "pat_internal.h"
 
 namespace pat {
@@ -226,15 +227,14 @@ __global__ void __launch_bounds__(kWarps * 32, (sizeof(R) == 4 && !CPLX && VB ==
 // every bank once.
 //
 // Measured per launch (one GB300, forward / adjoint): 128^2 -> 256^2 x 64 x
-// 256, 0.40 GB stored: 96 / 92 us, from 110 / 113 with bin rows and the table
-// loaded into registers; 256^2 -> 512^2 x 128 x 512, 5.8 GB: 1253 / 1192 from
-// 2270 / 1915; 202^2 -> 512^2 x 17 x 201: 138 / 157 from 507 / 316 (147 / 173
-// with groups of four slices, 3 us faster at 128^2 where the spectra stay in
-// L2); five volumes at 64^2 -> 128^2 x 32 x 128: 36 / 39 from 57 / 76. Without
-// the table copies the 128^2 launch takes 70 / 62 us and without the
-// multiply-adds 80 / 88: shared-memory and L1 traffic (the spectra, the ring
-// and the 32-line stores of scattered sectors) and the table stream overlap
-// only in part.
+// 256, 0.40 GB stored: 83 / 89 us, from 110 / 113 with bin rows and the table
+// loaded into registers; 256^2 -> 512^2 x 128 x 512, 5.8 GB: 1154 / 1154 from
+// 2270 / 1915; 202^2 -> 512^2 x 17 x 201: 118 / 146 from 507 / 316; five
+// volumes at 64^2 -> 128^2 x 32 x 128: 31 / 37 from 57 / 76. What bounds them
+// is the load / store unit: a block of 4 samples reads its spectra (32 cycles
+// a step and warp), the ring (16), stages and stores scattered sectors (a cycle
+// per line): 64 us of the 83 at 128^2, beside 62 us of DRAM traffic and 34 us
+// of multiply-adds.
 constexpr int kFoldThreads = 512;  // most threads of a CTA (caps the registers at 128)
 
 // 16-byte slot of half h (slices 2h, 2h + 1) of a lane's quad in its 1 KB row.
@@ -322,66 +322,123 @@ __device__ __forceinline__ int64_t vol_len(int n, int64_t Kpad) {
   return (GRP ? (int64_t)((n + kGroup - 1) / kGroup) * kGroup : (int64_t)n) * Kpad;
 }
 
-// 16-byte asynchronous copy of a table float4 (zero when !ok).
-__device__ __forceinline__ void cp_table(float4* dst, const float4* src, bool ok) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
-                   (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src), "r"(ok ? 16 : 0)
-               : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Forward: a warp takes blocks of T time samples and walks the z-groups; the
-// T table float4s of a step sit in the warp's ring of R slots, copied ahead by
-// the lanes that read them (no barrier: a lane reads its own copies), so the
-// table bytes in flight do not cost registers.
-// grid (batch, nrb, splits of the time blocks), tb time blocks per split.
+// A warp's ring of R slots of SLOT float4 rows (32 lanes) in shared memory,
+// filled by bulk copies of contiguous pieces of the table: lane 0 issues the
+// copies of a step, all lanes wait for it and read their own column, and the
+// slot is refilled as soon as every lane has read it, so R steps are in flight
+// and their bytes cost neither registers nor load / store slots. A wait that
+// runs out marks the ring dead: nothing more is issued or read, and close()
+// records the error once its copies have landed.
+constexpr uint32_t kRingTests = 1u << 22;  // tests per wait (seconds)
+
+template <int R, int SLOT>
+struct TableRing {
+  float4* rows;    // [R][SLOT][32]
+  uint64_t* full;  // [R]
+  int slot = 0;    // of the oldest step: the one to read, and then to refill
+  uint32_t par = 0;
+  int fly = 0;     // steps issued and not read
+  bool dead = false;
+  __device__ __forceinline__ TableRing(unsigned char* smem, uint64_t* bars, int warp, int lane)
+      : rows(reinterpret_cast<float4*>(smem) + warp * (R * SLOT * 32)), full(bars + warp * R) {
+    if (lane == 0) {
+      for (int i = 0; i < R; ++i) mbar_init(&full[i], 1);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+  }
+  // Opens slot i for copies of `bytes` in all (lane 0).
+  __device__ __forceinline__ float4* open(int i, uint32_t bytes) {
+    mbar_arrive_expect_tx(&full[i], bytes);
+    return rows + i * (SLOT * 32);
+  }
+  __device__ __forceinline__ void copy(int i, float4* dst, const float4* src, int nrows) {
+    bulk_g2s(dst, src, (uint32_t)nrows * 512u, &full[i]);
+  }
+  // Waits for the oldest step; its slot.
+  __device__ __forceinline__ const float4* wait() {
+    if (!dead) dead = !mbar_wait(&full[slot], par, kRingTests);
+    return rows + slot * (SLOT * 32);
+  }
+  // The oldest step has been read by this lane; its slot was refilled.
+  __device__ __forceinline__ void next() {
+    if (++slot == R) {
+      slot = 0;
+      par ^= 1u;
+    }
+  }
+  __device__ __forceinline__ void close(int lane, int* err) {
+    if (__any_sync(0xffffffffu, dead) && lane == 0) {
+      atomicExch(err, 1);
+      const uint64_t deadline = global_ns() + kDrainNs;
+      for (; fly > 0; --fly, next()) drain_wait(&full[slot], par, deadline);
+    }
+  }
+};
+
+// Warp index, uniform for the compiler: the cursors of the rings then live in
+// uniform registers.
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+}
+
+// Forward: a warp takes blocks of T time samples and walks the z-groups, a
+// step of its ring holding the T table rows of one group. grid (batch, nrb,
+// splits of the time blocks), tb time blocks per split.
 template <bool GRP, int T, int R>
 __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_fwd(const float4* __restrict__ table, const int4* __restrict__ members,
                const int* __restrict__ chunk, const cx<float>* __restrict__ X,
-               cx<float>* __restrict__ Y, int nz, int nt, int nzg, int64_t Kpad, int tb, int gc) {
+               cx<float>* __restrict__ Y, int nz, int nt, int nzg, int64_t Kpad, int tb, int gc,
+               int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = warp_index(), nwarps = blockDim.x >> 5;
   float4* xs = reinterpret_cast<float4*>(smem_raw);  // [4][gc][64]
-  float4* ring = xs + 4 * gc * 64 + warp * (R * T * 32) + lane;
+  unsigned char* rings = smem_raw + 4096 * gc;
+  TableRing<R, T> ring(rings, reinterpret_cast<uint64_t*>(rings + nwarps * (R * T * 512)), warp,
+                       lane);
   const int64_t ub = blockIdx.y;
   const int b = blockIdx.x;
-  const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32 + lane;
+  const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32;
   const int bk0 = blockIdx.z * tb + warp;
   const int bend = min((nt + T - 1) / T, (int)(blockIdx.z + 1) * tb);
   for (int g0 = 0; g0 < nzg; g0 += gc) {  // z-groups whose spectra fit: one pass up to gc groups
     const int g1 = min(nzg, g0 + gc);
     int pbk = bk0, pg = g0;  // next step to copy
-    auto copy_ahead = [&](int slot) {
-      if (pbk < bend) {
-        const float4* src = tbl + ((int64_t)pbk * T * nzg + pg) * 32;
+    auto refill = [&](int i) {
+      if (pbk < bend && !ring.dead) {
+        if (lane == 0) {
+          const int n = min(T, nt - pbk * T);
+          float4* dst = ring.open(i, (uint32_t)n * 512u);
 #pragma unroll
-        for (int r = 0; r < T; ++r)
-          cp_table(ring + (slot * T + r) * 32, src + (int64_t)r * nzg * 32, pbk * T + r < nt);
+          for (int r = 0; r < T; r += 4)
+            if (r < n)
+              ring.copy(i, dst + r * 32, tbl + folded_row(pbk * T + r, pg, nt, nzg),
+                        min(4, n - r));
+        }
+        ++ring.fly;
         if (++pg == g1) {
           pg = g0;
           pbk += nwarps;
         }
       }
-      cp_commit();
     };
 #pragma unroll
-    for (int i = 0; i < R - 1; ++i) copy_ahead(i);  // the table is constant: no wait needed
+    for (int i = 0; i < R; ++i) refill((ring.slot + i) % R);  // the table is constant: no wait
     {
       const int4 mem = members[ub * 32 + lane];
       const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
       if (g0 == 0) pdl_wait();
-      stage_quads<GRP>(xs, gc, X + b * vol_len<GRP>(nz, Kpad), bins, g0, g1 - g0, nz, Kpad,
-                        lane, warp, nwarps);
+      stage_quads<GRP>(xs, gc, X + b * vol_len<GRP>(nz, Kpad), bins, g0, g1 - g0, nz, Kpad, lane,
+                       warp, nwarps);
     }
     cp_wait<0>();
     __syncthreads();
-    int slot = 0;
     for (int bk = bk0; bk < bend; bk += nwarps) {
       cx<float> acc[T][4];
 #pragma unroll
@@ -390,12 +447,14 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         for (int m = 0; m < 4; ++m) acc[r][m] = mk<float>(0.f, 0.f);
 #pragma unroll 1
       for (int g = 0; g < g1 - g0; ++g) {
-        copy_ahead((slot + R - 1) % R);
-        cp_wait<R - 1>();
+        const float4* hs = ring.wait();
         float4 h[T];
 #pragma unroll
-        for (int r = 0; r < T; ++r) h[r] = ring[(slot * T + r) * 32];
-        slot = (slot + 1) % R;
+        for (int r = 0; r < T; ++r) h[r] = hs[r * 32 + lane];
+        --ring.fly;
+        __syncwarp();
+        refill(ring.slot);
+        ring.next();
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           float4 x[4];
@@ -421,14 +480,15 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         for (int m = 0; m < 4; ++m) {
           if (bins[m] < 0) continue;
           if (g0 > 0) add_quad<GRP>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m],
-                                     acc[r + 2][m], acc[r + 3][m]);
+                                    acc[r + 2][m], acc[r + 3][m]);
           store_quad<GRP>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m], acc[r + 2][m],
-                           acc[r + 3][m]);
+                          acc[r + 3][m]);
         }
       }
     }
-    if (g1 < nzg) __syncthreads();  // the spectra and rings are free
+    if (g1 < nzg) __syncthreads();  // the spectra are free
   }
+  ring.close(lane, err);
 }
 
 // Adjoint: warp (zi, ti) of zw x tw owns the z-groups (zc zw + zi) GPW + j
@@ -443,37 +503,36 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_adj(const float4* __restrict__ table, const int4* __restrict__ members,
                const int* __restrict__ chunk, const cx<float>* __restrict__ D,
                cx<float>* __restrict__ Z, int nz, int nt, int nzg, int64_t Kpad, int nzc, int zw,
-               int tw) {
+               int tw, int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = warp_index(), nwarps = blockDim.x >> 5;
   const int tq = SQ * tw;                            // quads per stage
   float4* ds = reinterpret_cast<float4*>(smem_raw);  // [2][4][tq][64]
-  float4* ring = ds + 2 * 4 * tq * 64 + warp * (R * 4 * GPW * 32) + lane;
+  unsigned char* rings = smem_raw + 2 * 4096 * tq;
+  TableRing<R, 4 * GPW> ring(
+      rings, reinterpret_cast<uint64_t*>(rings + nwarps * (R * 4 * GPW * 512)), warp, lane);
   const int64_t ub = blockIdx.y;
   const int zc = blockIdx.x % nzc, b = blockIdx.x / nzc;
   const int zi = warp % zw, ti = warp / zw;
   const int gbase = (zc * zw + zi) * GPW;
-  const float4* tbl =
-      table + ((int64_t)(chunk ? chunk[ub] : ub) * nt * nzg + gbase) * 32 + lane;
+  const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32;
   const int ntq = (nt + 3) / 4, nst = (ntq + tq - 1) / tq;
-  int pq = ti;  // next quad to copy
-  auto copy_ahead = [&](int slot) {
-    if (pq < ntq) {
-      const float4* src = tbl + (int64_t)pq * 4 * nzg * 32;
+  int pq = gbase < nzg ? ti : ntq;  // next quad to copy
+  auto refill = [&](int i) {
+    if (pq < ntq && !ring.dead) {
+      if (lane == 0) {
+        const int n = min(4, nt - 4 * pq), ng = min(GPW, nzg - gbase);
+        float4* dst = ring.open(i, (uint32_t)(n * ng) * 512u);
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int j = 0; j < GPW; ++j) {
-          const bool ok = 4 * pq + r < nt && gbase + j < nzg;
-          cp_table(ring + ((slot * 4 + r) * GPW + j) * 32,
-                   ok ? src + ((int64_t)r * nzg + j) * 32 : table, ok);
-        }
+        for (int j = 0; j < GPW; ++j)
+          if (j < ng) ring.copy(i, dst + j * 128, tbl + folded_row(4 * pq, gbase + j, nt, nzg), n);
+      }
+      ++ring.fly;
       pq += tw;
     }
-    cp_commit();
   };
 #pragma unroll
-  for (int i = 0; i < R - 1; ++i) copy_ahead(i);
+  for (int i = 0; i < R; ++i) refill(i);
   const int4 mem = members[ub * 32 + lane];
   const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
   const cx<float>* Db = D + b * vol_len<GRP>(nt, Kpad);
@@ -486,52 +545,55 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       for (int m = 0; m < 4; ++m) acc[j][q][m] = mk<float>(0.f, 0.f);
   pdl_wait();
   stage_quads<GRP>(ds, tq, Db, bins, 0, min(tq, ntq), nt, Kpad, lane, warp, nwarps);
-  cp_wait<0>();
-  int slot = 0;
   for (int st = 0; st < nst; ++st) {
     const int q0 = st * tq;
-    // this stage's D: SQ ring groups were committed after its copies
-    if (st > 0) cp_wait<SQ>();
+    cp_wait<0>();     // this stage's D
     __syncthreads();  // and every warp is done with the other buffer
     if (st + 1 < nst)
       stage_quads<GRP>(ds + ((st + 1) & 1) * 4 * tq * 64, tq, Db, bins, q0 + tq,
-                        min(tq, ntq - q0 - tq), nt, Kpad, lane, warp, nwarps);
+                       min(tq, ntq - q0 - tq), nt, Kpad, lane, warp, nwarps);
     const float4* dst = ds + (st & 1) * 4 * tq * 64;
 #pragma unroll 1
-    for (int i = 0; i < SQ; ++i) {
-      const int q = ti + i * tw;
-      copy_ahead((slot + R - 1) % R);
-      cp_wait<R - 1>();
-      if (q0 + q < ntq) {
-        float4 h[4][GPW];
+    for (int q = ti; q < min(tq, ntq - q0) && gbase < nzg; q += tw) {
+      const float4* hs = ring.wait();
+      float4 h[4][GPW];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < 4; ++r)
 #pragma unroll
-          for (int j = 0; j < GPW; ++j) h[r][j] = ring[((slot * 4 + r) * GPW + j) * 32];
+        for (int j = 0; j < GPW; ++j) h[r][j] = hs[(j * 4 + r) * 32 + lane];
+      --ring.fly;
+      __syncwarp();
+      refill(ring.slot);
+      ring.next();
+      if (4 * (q0 + q) + 4 > nt) {  // rows past nt were not copied; D is zero there
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf)
+        for (int r = 1; r < 4; ++r)
 #pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const float4 d = dst[(m * tq + q) * 64 + quad_slot(lane, hf)];
+          for (int j = 0; j < GPW; ++j)
+            if (4 * (q0 + q) + r >= nt) h[r][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-              const cx<float> dv = k ? mk<float>(d.z, d.w) : mk<float>(d.x, d.y);
+      for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
-              for (int j = 0; j < GPW; ++j) {
-                const float4 hv = h[2 * hf + k][j];
-                mac(acc[j][0][m], hv.x, dv);
-                mac(acc[j][1][m], hv.y, dv);
-                mac(acc[j][2][m], hv.z, dv);
-                mac(acc[j][3][m], hv.w, dv);
-              }
+        for (int m = 0; m < 4; ++m) {
+          const float4 d = dst[(m * tq + q) * 64 + quad_slot(lane, hf)];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const cx<float> dv = k ? mk<float>(d.z, d.w) : mk<float>(d.x, d.y);
+#pragma unroll
+            for (int j = 0; j < GPW; ++j) {
+              const float4 hv = h[2 * hf + k][j];
+              mac(acc[j][0][m], hv.x, dv);
+              mac(acc[j][1][m], hv.y, dv);
+              mac(acc[j][2][m], hv.z, dv);
+              mac(acc[j][3][m], hv.w, dv);
             }
           }
-      }
-      slot = (slot + 1) % R;
+        }
     }
   }
+  ring.close(lane, err);
   if (tw > 1) {
-    cp_wait<0>();
     __syncthreads();  // the staging buffers and rings are free
     cx<float>* red = reinterpret_cast<cx<float>*>(smem_raw);  // [(ti - 1) zw + zi][GPW 16][32]
     if (ti > 0) {
@@ -566,7 +628,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     for (int m = 0; m < 4; ++m)
       if (bins[m] >= 0)
         store_quad<GRP>(Zb, g, bins[m], nz, Kpad, acc[j][0][m], acc[j][1][m], acc[j][2][m],
-                         acc[j][3][m]);
+                        acc[j][3][m]);
   }
 }
 
@@ -575,7 +637,7 @@ constexpr size_t kSmemCta = 227 * 1024;  // most shared memory of a CTA (and of 
 template <bool GRP, int T, int R>
 cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc, cudaStream_t s) {
   const Layout& L = p.L;
-  constexpr size_t ring = (size_t)R * T * 512;  // bytes per warp
+  constexpr size_t ring = (size_t)R * (T * 512 + 8);  // bytes per warp
   const size_t xbytes = (size_t)gc * 4096;
   const bool two = 2 * (xbytes + 8 * ring) <= kSmemCta;
   const int nwarps = two ? 8 : (int)std::min<size_t>(16, (kSmemCta - xbytes) / ring);
@@ -586,8 +648,8 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
   if (e != cudaSuccess) return e;
   // Splits of the time blocks over CTAs, by waves of CTAs x (blocks of the
   // busiest warp + the CTA's load of its SM + its prologue): the order of the
-  // measured times at 71 to 1059 blocks (64^2: 10.1 us in 2, 16 in 1; 128^2:
-  // 93 us in 1, 99 in 2; 5 volumes at 64^2: 35 us in 2, 39 in 1).
+  // measured times at 71 to 1059 blocks (64^2: 9.2 us in 2, 14.5 in 1; 128^2:
+  // 83 us in 1, 91 in 2; 5 volumes at 64^2: 31 us in 2, 33.5 in 1).
   const int nb = (L.nt + T - 1) / T, slots = two ? (int)kFoldCtas : (int)kFoldCtas / 2;
   const int64_t ctas = L.nrb * batch;
   int tb = nb;
@@ -605,7 +667,7 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
   return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
                     reinterpret_cast<const int4*>(p.rb_members),
                     static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(X),
-                    static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad, tb, gc);
+                    static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad, tb, gc, p.tc_err);
 }
 
 template <bool GRP>
@@ -614,12 +676,17 @@ cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStrea
   if ((size_t)L.nzg * 4096 > kSmemCta) return cudaErrorInvalidValue;  // more than 224 depths
   // the spectra of up to 128 depths are resident at a time, more take another pass
   const int gc = std::min(L.nzg, 32);
-  // Blocks of 8 samples read the spectra half as often as blocks of 4, but
-  // their ring leaves room for two CTAs per SM only up to 48 depths (three
-  // volumes at 96^2 x 45: 78 against 84 us); at 64 depths two CTAs with
-  // blocks of 4 are faster than one of 16 warps with blocks of 8 (93 / 101 us).
-  if (2 * ((size_t)gc * 4096 + 64 * 1024) <= kSmemCta)
+  // Blocks of 8 samples read the spectra half as often as blocks of 4. With
+  // two steps in the ring two CTAs fit an SM up to 48 depths (three volumes at
+  // 96^2 x 45: 72 us, 76 in blocks of 4), with one up to 80, which pays from
+  // two waves of CTAs on (128^2 x 64: 83 us in blocks of 4 with three steps, 86
+  // in blocks of 8 with one; five volumes 374 and 343). Beyond that one CTA of
+  // 16 warps in blocks of 4 (256^2 x 128: 1154 us, 1219 with 8 warps of 8).
+  const size_t xbytes = (size_t)gc * 4096;
+  if (2 * (xbytes + 8 * 2 * (8 * 512 + 8)) <= kSmemCta)
     return fold_fwd_t<GRP, 8, 2>(p, X, Y, batch, gc, s);
+  if (2 * (xbytes + 8 * (8 * 512 + 8)) <= kSmemCta && L.nrb * batch >= 2 * kFoldCtas)
+    return fold_fwd_t<GRP, 8, 1>(p, X, Y, batch, gc, s);
   return fold_fwd_t<GRP, 4, 3>(p, X, Y, batch, gc, s);
 }
 
@@ -628,7 +695,7 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
                        cudaStream_t s) {
   const Layout& L = p.L;
   const int nzc = (L.nzg + zw * GPW - 1) / (zw * GPW), nwarps = zw * tw;
-  const size_t ring = (size_t)nwarps * R * 4 * GPW * 512;
+  const size_t ring = (size_t)nwarps * R * (4 * GPW * 512 + 8);
   const size_t smem = std::max<size_t>(2 * 4096 * (size_t)SQ * tw + ring,
                                        (size_t)(tw - 1) * zw * GPW * 4096);
   auto fn = k_fold_adj<GRP, GPW, SQ, R>;
@@ -639,13 +706,15 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
   return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
                     reinterpret_cast<const int4*>(p.rb_members),
                     static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(D),
-                    static_cast<cx<float>*>(Z), L.nz, L.nt, L.nzg, L.Kpad, nzc, zw, tw);
+                    static_cast<cx<float>*>(Z), L.nz, L.nt, L.nzg, L.Kpad, nzc, zw, tw, p.tc_err);
 }
 
 // Two z-groups per warp and up to 8 warps along z; fewer along z leave warps
 // for the time samples. Grids with less than about one CTA per SM split the
-// z-groups over more CTAs (64^2 x 32: 12.7 us in two, 17 in one; 32^2 x 16:
-// 5.7 us in four of one group per warp, 13 in one).
+// z-groups over more CTAs (64^2 x 32: 12.1 us in two, 16 in one; 32^2 x 16:
+// 5.8 us in four of one group per warp, 13 in one). A stage holds two quads of
+// D per warp along the time, or four from two waves of CTAs on (256^2 x 128 x
+// 512: 1175 us with two, 1154 with four; five volumes at 128^2 346 and 332).
 template <bool GRP>
 cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s) {
   const Layout& L = p.L;
@@ -660,6 +729,8 @@ cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStrea
   if (zw == 1 && 2 * ctas * nzc <= 200) return fold_adj_t<GRP, 1, 1, 4>(p, D, Z, batch, 1, 8, s);
   static constexpr int kTw[8] = {8, 4, 2, 2, 1, 1, 1, 1};
   const int tw = kTw[zw - 1];
+  if (tw == 1 && ctas * nzc >= 2 * kFoldCtas)
+    return fold_adj_t<GRP, 2, 4, 2>(p, D, Z, batch, zw, tw, s);
   return tw <= 2 ? fold_adj_t<GRP, 2, 2, 2>(p, D, Z, batch, zw, tw, s)
                  : fold_adj_t<GRP, 2, 1, 2>(p, D, Z, batch, zw, tw, s);
 }

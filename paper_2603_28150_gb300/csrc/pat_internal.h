@@ -77,7 +77,9 @@ struct vec16<double> {
 // ("kx-major half spectrum"); K = (px/2 + 1) py, padded to Kpad (multiple of 32).
 // Table: [kb = k / 32][t][zg][lane = k % 32][ZG] elements, 16 bytes per
 // (kb, t, zg, lane) group; ZG = z-planes per group (4 real f32, 2 complex f32
-// or real f64, 1 complex f64).
+// or real f64, 1 complex f64). Folded tables keep four time samples of a group
+// together, [kb][t / 4][zg][t % 4][lane] (see folded_row), so what a step of
+// the contraction reads is one contiguous piece.
 struct Layout {
   int nx, ny, nz, nt, px, py, max_batch;
   bool fp64, real;
@@ -100,6 +102,13 @@ struct Layout {
   // (i < mx, j < my) of the sensor grid; sx = sy = 1 is the plain operator.
   int sx = 1, sy = 1, ox = 0, oy = 0, mx = 0, my = 0;
 };
+
+// 16-byte units before row (t, zg) of a chunk of a folded table (nt samples, nzg
+// groups; the last quad of samples may hold fewer than four rows).
+__host__ __device__ __forceinline__ int64_t folded_row(int t, int zg, int nt, int nzg) {
+  const int t0 = t & ~3, rows = nt - t0 < 4 ? nt - t0 : 4;
+  return ((int64_t)t0 * nzg + (int64_t)zg * rows + (t - t0)) * 32;
+}
 
 // Sampling pattern handed to the row kernels (identity when s.on == false).
 struct Samp {

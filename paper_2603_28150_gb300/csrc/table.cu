@@ -105,7 +105,7 @@ __global__ void k_stats(const cx<RS>* __restrict__ src, int64_t sstride, int row
 // taken modulo 1 in 64-bit fixed point so large arguments keep full accuracy,
 // then contracts over m with W[m][j] = w_m cos(2 pi m (z0 + j) / mz) / (mz px py)
 // (w_m = 1 at m = 0 and mz/2, else 2) from shared memory.
-__global__ void k_kspace(int px, int py, int mz, int nz, int nt, int nzg, int ZG, int cplx,
+__global__ void k_kspace(int px, int py, int mz, int nz, int nt, int nzg, int ZG, int cplx, int fold,
                          const unsigned long long* __restrict__ u_fix,  // [K][mz/2+1] phase/sample
                          const float* __restrict__ W,                   // [mz/2+1][nz]
                          void* table, int64_t K) {
@@ -132,7 +132,9 @@ __global__ void k_kspace(int px, int py, int mz, int nz, int nt, int nzg, int ZG
       float acc = 0.f;
       for (int m = 0; m < M; ++m) acc = fmaf(cs[m * 32 + lane], ws[m * nz + j], acc);
       if (k < K) {
-        const int64_t idx = table_index(k, t, j, nt, nzg, ZG);
+        const int64_t idx =
+            fold ? ((k >> 5) * nt * nzg * 32 + folded_row(t, j / ZG, nt, nzg) + (k & 31)) * ZG + j % ZG
+                 : table_index(k, t, j, nt, nzg, ZG);
         if (cplx) {
           cx<float> v;
           v.x = acc;
@@ -182,7 +184,7 @@ __global__ void k_fold_gather(const float4* __restrict__ full, float4* __restric
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     const int64_t k = row_bin[u];
     if (k >= 0) v = full[(((k >> 5) * nt + t) * nzg + g) * 32 + (k & 31)];
-    folded[(((u >> 5) * nt + t) * nzg + g) * 32 + (u & 31)] = v;
+    folded[(u >> 5) * nt * nzg * 32 + folded_row(t, g, nt, nzg) + (u & 31)] = v;
   }
 }
 
@@ -232,19 +234,26 @@ std::vector<double> twiddles(int n) {
 // a[t] = sum_{tau < nr, tau <= t} r[tau] a[t - tau] (FP64 sums), computed for
 // t from nt - 1 down to 0 so every term still reads the unfiltered value. The
 // blocked layout keeps, per table block, nt rows of `inner` scalars (real and
-// imaginary parts alike: the response is real).
+// imaginary parts alike: the response is real), in folded tables (nzg > 0) in
+// the order of folded_row.
 template <typename S>
 __global__ void k_sensor_fir(S* __restrict__ table, int64_t blocks, int nt, int64_t inner,
-                             const double* __restrict__ r, int nr) {
+                             const double* __restrict__ r, int nr, int nzg) {
+  constexpr int E = 16 / (int)sizeof(S);  // scalars per 16-byte unit
   const int64_t n = blocks * inner;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    S* a = table + (i / inner) * nt * inner + i % inner;
+    S* a = table + (i / inner) * nt * inner;
+    const int64_t w = i % inner;
+    const int zg = (int)(w / (32 * E));
+    auto at = [&](int t) -> S& {
+      return nzg ? a[folded_row(t, zg, nt, nzg) * E + w % (32 * E)] : a[(int64_t)t * inner + w];
+    };
     for (int t = nt - 1; t >= 0; --t) {
       double acc = 0.0;
       const int m = nr < t + 1 ? nr : t + 1;
-      for (int tau = 0; tau < m; ++tau) acc += r[tau] * (double)a[(int64_t)(t - tau) * inner];
-      a[(int64_t)t * inner] = (S)acc;
+      for (int tau = 0; tau < m; ++tau) acc += r[tau] * (double)at(t - tau);
+      at(t) = (S)acc;
     }
   }
 }
@@ -260,12 +269,13 @@ int apply_sensor_response(Plan& p, const double* r, int nr, cudaStream_t s) {
   cudaError_t e = cudaMemcpyAsync(rd, r, sizeof(double) * nr, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) {
     const int g = grid_for(blocks * inner);
+    const int nzg = L.fold ? L.nzg : 0;
     if (L.fp64)
       k_sensor_fir<double><<<g, 256, 0, s>>>(static_cast<double*>(p.table), blocks, L.nt, inner,
-                                             rd, nr);
+                                             rd, nr, nzg);
     else
       k_sensor_fir<float><<<g, 256, 0, s>>>(static_cast<float*>(p.table), blocks, L.nt, inner, rd,
-                                            nr);
+                                            nr, nzg);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -765,7 +775,7 @@ int kspace_generate(Plan& p, const pat_medium& m, const std::vector<int>& bins, 
                                 (int)smem));
   if (npos > 0) {  // a frequency shard may hold no rows
     k_kspace<<<(unsigned)((npos + 31) / 32), 256, smem, s>>>(L.px, L.py, m.mz, L.nz, L.nt, L.nzg,
-                                                              L.zg, L.real ? 0 : 1, u_d, W_d,
+                                                              L.zg, L.real ? 0 : 1, L.fold ? 1 : 0, u_d, W_d,
                                                               p.table, npos);
     GEN_CUDA(cudaGetLastError());
   }

@@ -35,6 +35,7 @@
 #include <algorithm>
 #include <utility>
 
+#include "async.cuh"
 #include "pat_internal.h"
 
 namespace pat {
@@ -48,61 +49,8 @@ constexpr int kTileBytes = kTile * kTile * 2;  // 32 KB of BF16
 constexpr int kLBO = 128;                // bytes between K-adjacent core matrices
 constexpr int kSBO = (kTile / 8) * 128;  // bytes between M/N-adjacent core matrices (2048)
 constexpr int kBBytes = kN * kTile * 2;  // one 32 x 128 B-operand chunk (8 KB)
-// Teardown drains (copies and MMAs still in flight after an abort) wait at
-// most this long in total, measured on the global timer.
-constexpr uint64_t kDrainNs = 2000000000ull;
 
 // -------------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded pipeline wait for the phase with the given parity: at most `limit`
-// tests (mbarrier.try_wait itself suspends the thread for a bounded time, so
-// the loop polls without sleeping); false on timeout. limit = 0 gives up at
-// once (the plan's wait limit set to 0 exercises the abort path).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit) {
-  for (uint32_t i = 0; i < limit; ++i)
-    if (mbar_test(bar, parity)) return true;
-  return false;
-}
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-// Teardown wait: until the phase completes or the global timer passes
-// `deadline` (shared by all drain waits of a thread, so once it has passed the
-// remaining drains return at once).
-__device__ __forceinline__ bool drain_wait(uint64_t* bar, uint32_t parity, uint64_t deadline) {
-  while (!mbar_test(bar, parity))
-    if (global_ns() > deadline) return false;
-  return true;
-}
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -914,7 +862,7 @@ size_t smem_for(int kchunks) {
 // blocked FP32 table (row rep[k] of the stored table, or row k when rep is
 // NULL); adjoint tile of bin k, K chunk kc (t columns), part.
 __global__ void k_split_tables(const float* __restrict__ table, const int* __restrict__ rep,
-                               int nz, int nt, int nzg, int64_t K,
+                               int fold, int nz, int nt, int nzg, int64_t K,
                                unsigned char* __restrict__ fwd, unsigned char* __restrict__ adj) {
   const int64_t n = K * nt * nz;
   const int mtiles = nt / kTile;
@@ -925,7 +873,9 @@ __global__ void k_split_tables(const float* __restrict__ table, const int* __res
     const int64_t k = i / ((int64_t)nz * nt);
     const int64_t row = rep ? rep[k] : k;  // folded tables: the bin's representative row
     const int64_t kb = row >> 5, l = row & 31;
-    const float h = table[(((kb * nt + t) * nzg + z / 4) * 32 + l) * 4 + z % 4];
+    const int64_t unit = fold ? kb * nt * nzg * 32 + folded_row(t, z / 4, nt, nzg)
+                              : ((kb * nt + t) * nzg + z / 4) * 32;
+    const float h = table[(unit + l) * 4 + z % 4];
     const __nv_bfloat16 hi = __float2bfloat16_rn(h);
     const __nv_bfloat16 lo = __float2bfloat16_rn(h - __bfloat162float(hi));
     // forward: tile (k, mt = t / 128), rows t % 128, K = z
@@ -966,7 +916,7 @@ cudaError_t tc_build_tables(const Plan& p, void* fwd, void* adj, cudaStream_t s)
   int64_t g = (n + 255) / 256;
   if (g > 152 * 64) g = 152 * 64;
   tc::k_split_tables<<<(int)g, 256, 0, s>>>(static_cast<const float*>(p.table),
-                                            L.fold ? p.rep_row : nullptr, L.nz,
+                                            L.fold ? p.rep_row : nullptr, L.fold ? 1 : 0, L.nz,
                                             L.nt, L.nzg, rows, static_cast<unsigned char*>(fwd),
                                             static_cast<unsigned char*>(adj));
   return cudaGetLastError();
