@@ -407,23 +407,18 @@ int check_call(pat_plan* plan, int batch) {
 
 // Host-or-device argument: a device pointer is used as is; a host pointer is
 // staged (copied in for inputs) through `stage`.
+// Where an argument lives is looked up once.
 struct Arg {
   const void* user;
-  void* dev;
+  void* dev = nullptr;
   bool host;
+  explicit Arg(const void* u) : user(u), host(!is_device_ptr(u)) {}
 };
 
 int stage_in(Arg& a, void* stage, size_t bytes, cudaStream_t s) {
-  a.host = !is_device_ptr(a.user);
   a.dev = a.host ? stage : const_cast<void*>(a.user);
   if (a.host && bytes) PAT_CUDA(cudaMemcpyAsync(stage, a.user, bytes, cudaMemcpyHostToDevice, s));
   return PAT_OK;
-}
-
-int any_host(std::initializer_list<const void*> ptrs) {
-  for (const void* q : ptrs)
-    if (q && !is_device_ptr(q)) return 1;
-  return 0;
 }
 
 // Seeded start vector of the power iteration (splitmix64 of Steele, Lea &
@@ -755,10 +750,10 @@ int pat_forward(pat_plan* plan, const void* rho, void* d, int batch, pat_stream 
   Plan& p = plan->p;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t ob = obj_elems(p.L, batch) * p.L.rsize, db = dat_elems(p.L, batch) * p.L.rsize;
-  if (any_host({rho, d}) && (rc = ensure_io(plan)) != PAT_OK) return rc;
-  Arg a{rho, nullptr, false};
+  Arg a(rho), o(d);
+  if ((a.host || o.host) && (rc = ensure_io(plan)) != PAT_OK) return rc;
   if ((rc = stage_in(a, plan->x.io_obj[0], ob, s)) != PAT_OK) return rc;
-  const bool hout = !is_device_ptr(d);
+  const bool hout = o.host;
   void* dst = hout ? plan->x.io_dat : d;
   PAT_CUDA(forward_dev(p, a.dev, dst, batch, s));
   if (hout) {
@@ -780,10 +775,10 @@ int pat_adjoint(pat_plan* plan, const void* d, void* rho, int batch, pat_stream 
   Plan& p = plan->p;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t ob = obj_elems(p.L, batch) * p.L.rsize, db = dat_elems(p.L, batch) * p.L.rsize;
-  if (any_host({rho, d}) && (rc = ensure_io(plan)) != PAT_OK) return rc;
-  Arg a{d, nullptr, false};
+  Arg a(d), o(rho);
+  if ((a.host || o.host) && (rc = ensure_io(plan)) != PAT_OK) return rc;
   if ((rc = stage_in(a, plan->x.io_dat, db, s)) != PAT_OK) return rc;
-  const bool hout = !is_device_ptr(rho);
+  const bool hout = o.host;
   void* dst = hout ? plan->x.io_obj[0] : rho;
   PAT_CUDA(adjoint_dev(p, a.dev, dst, batch, s));
   if (hout) {
@@ -810,11 +805,11 @@ int pat_gradient(pat_plan* plan, const void* xin, const void* y, void* grad, int
   PlanExt& px = plan->x;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t ob = obj_elems(p.L, batch) * p.L.rsize, db = dat_elems(p.L, batch) * p.L.rsize;
-  if (any_host({xin, y, grad}) && (rc = ensure_io(plan)) != PAT_OK) return rc;
-  Arg ax{xin, nullptr, false}, ay{y, nullptr, false};
+  Arg ax(xin), ay(y), ag(grad);
+  if ((ax.host || ay.host || ag.host) && (rc = ensure_io(plan)) != PAT_OK) return rc;
   if ((rc = stage_in(ax, px.io_obj[0], ob, s)) != PAT_OK) return rc;
   if ((rc = stage_in(ay, px.io_dat, db, s)) != PAT_OK) return rc;
-  const bool hout = !is_device_ptr(grad);
+  const bool hout = ag.host;
   void* dst = hout ? px.io_obj[1] : grad;
   PAT_CUDA(gradient_dev(p, ax.dev, ay.dev, dst, batch, s, px.res + 1));
   if (hout) PAT_CUDA(cudaMemcpyAsync(grad, dst, ob, cudaMemcpyDeviceToHost, s));

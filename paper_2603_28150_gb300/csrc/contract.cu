@@ -643,8 +643,7 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
   const int nwarps = two ? 8 : (int)std::min<size_t>(16, (kSmemCta - xbytes) / ring);
   const size_t smem = xbytes + nwarps * ring;
   auto fn = k_fold_fwd<GRP, T, R>;
-  cudaError_t e = cudaFuncSetAttribute((const void*)fn,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   // Splits of the time blocks over CTAs, by waves of CTAs x (blocks of the
   // busiest warp + the CTA's load of its SM + its prologue): the order of the
@@ -699,8 +698,7 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
   const size_t smem = std::max<size_t>(2 * 4096 * (size_t)SQ * tw + ring,
                                        (size_t)(tw - 1) * zw * GPW * 4096);
   auto fn = k_fold_adj<GRP, GPW, SQ, R>;
-  cudaError_t e = cudaFuncSetAttribute((const void*)fn,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((unsigned)(nzc * batch), (unsigned)L.nrb);
   return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
@@ -741,11 +739,8 @@ cudaError_t fwd_t(const Plan& p, const void* X, void* Y, int batch, cudaStream_t
   constexpr int ZG = Elem<R, CPLX>::ZG;
   const size_t smem = sizeof(cx<R>) * (size_t)VB * L.nzg * ZG * 32;
   auto fn = k_contract_fwd<R, CPLX, VB>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute((const void*)fn,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_smem(fn, smem);
+  if (e != cudaSuccess) return e;
   dim3 grid((unsigned)L.nkb, (unsigned)((batch + VB - 1) / VB));
   return launch_pdl(fn, grid, dim3(kWarps * 32), smem, s,
                     static_cast<const typename vec16<R>::type*>(p.table),

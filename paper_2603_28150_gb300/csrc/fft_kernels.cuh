@@ -1118,11 +1118,6 @@ __global__ void __launch_bounds__(kThreads) k_row_c2r_step(
   }
 }
 
-template <typename R, int P>
-cudaError_t set_smem_attr(const void* fn) {
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem_bytes<R, P>());
-}
 }  // namespace
 
 // ---- launchers, one per stage and length ---------------------------------------
@@ -1133,7 +1128,7 @@ cudaError_t FftLen<R, P>::row_r2c(const R* in, int64_t in_stride, int nx_in, int
   const bool zin = 2 * nx_in <= P;  // the zero padding covers [P/2, P)
   auto fn = sm.on ? (zin ? k_row_r2c<R, P, true, true> : k_row_r2c<R, P, true, false>)
                   : (zin ? k_row_r2c<R, P, false, true> : k_row_r2c<R, P, false, false>);
-  cudaError_t e = set_smem_attr<R, P>((const void*)fn);
+  cudaError_t e = allow_smem(fn, smem_bytes<R, P>());
   if (e != cudaSuccess) return e;
   const int pairs = (ny_in + 1) / 2;
   dim3 grid((pairs + SH::VPB - 1) / SH::VPB, S);
@@ -1149,8 +1144,7 @@ cudaError_t col_fwd_t(const cx<R>* T, int tstride, int64_t tslice, int n_in, int
   const bool zin = 2 * n_in <= P;
   auto fn = zin ? k_col_fwd<R, P, MODE, true> : k_col_fwd<R, P, MODE, false>;
   constexpr size_t smem = smem_bytes<R, P, MODE>();
-  cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   // groups: units of kGroup slices (the last of a volume may hold fewer)
   const int64_t units = MODE == kGroups ? (int64_t)(S / sr.group) * ((sr.group + kGroup - 1) / kGroup) : S;
@@ -1167,8 +1161,7 @@ cudaError_t col_inv_t(const cx<R>* in, const SpecRow& sr, int ncols, int S, cx<R
   const bool hout = 2 * n_out <= P;  // rows [P/2, P) are cropped away
   auto fn = hout ? k_col_inv<R, P, MODE, true> : k_col_inv<R, P, MODE, false>;
   constexpr size_t smem = smem_bytes<R, P, MODE>();
-  cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   const int64_t units = MODE == kGroups ? (int64_t)(S / sr.group) * ((sr.group + kGroup - 1) / kGroup) : S;
   constexpr int per = MODE == kGroups ? SH::VPB / kGroup : SH::VPB;
@@ -1206,7 +1199,7 @@ cudaError_t FftLen<R, P>::row_c2r(const cx<R>* T, int tstride, int64_t tslice, i
   const bool hout = 2 * nx_out <= P;
   auto fn = sm.on ? (hout ? k_row_c2r<R, P, true, true> : k_row_c2r<R, P, true, false>)
                   : (hout ? k_row_c2r<R, P, false, true> : k_row_c2r<R, P, false, false>);
-  cudaError_t e = set_smem_attr<R, P>((const void*)fn);
+  cudaError_t e = allow_smem(fn, smem_bytes<R, P>());
   if (e != cudaSuccess) return e;
   const int pairs = (ny_out + 1) / 2;
   dim3 grid((pairs + SH::VPB - 1) / SH::VPB, S);
@@ -1224,8 +1217,7 @@ cudaError_t FftLen<R, P>::row_resid(cx<R>* T, int tstride, int64_t tslice, int n
   auto fn = sm.on ? k_row_resid<R, P, true> : k_row_resid<R, P, false>;
   const size_t smem =
       smem_bytes<R, P>() + (sm.on ? ResidStage<R, P, true>::bytes : ResidStage<R, P, false>::bytes);
-  cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   const int pairs = (ny + 1) / 2;
   dim3 grid((pairs + SH::VPB - 1) / SH::VPB, S);
@@ -1241,8 +1233,7 @@ cudaError_t FftLen<R, P>::row_c2r_step(const cx<R>* T, int tstride, int64_t tsli
   using SH = Shape<P>;
   auto fn = f.next_T ? k_row_c2r_step<R, P, true> : k_row_c2r_step<R, P, false>;
   const size_t smem = smem_bytes<R, P>() + StepStage<R, P>::bytes;
-  cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
   const int pairs = (ny + 1) / 2;
   dim3 grid((pairs + SH::VPB - 1) / SH::VPB, S);

@@ -158,6 +158,16 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Lets a kernel be launched with `smem` bytes of dynamic shared memory (up to
+// 48 KB every kernel may be).
+template <typename F>
+cudaError_t allow_smem(F fn, size_t smem) {
+  return smem <= 48 * 1024 ? cudaSuccess
+                           : cudaFuncSetAttribute((const void*)fn,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  (int)smem);
+}
+
 // ---- device allocations --------------------------------------------------------
 // Every device allocation of a plan (its table, maps, workspace and the
 // temporaries of table preparation) goes through dev_alloc / dev_free, which

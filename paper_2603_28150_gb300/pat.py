@@ -12,6 +12,7 @@ stages through the device (synchronous). Shapes, x fastest:
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from dataclasses import dataclass
 
@@ -195,8 +196,13 @@ def _stream(stream=None) -> int:
     torch = _torch()
     if stream is not None:
         return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
-    if torch.cuda.is_available():
-        return int(torch.cuda.current_stream().cuda_stream)
+    if torch.cuda.is_initialized() or torch.cuda.is_available():
+        # the current stream's handle without a Stream object where torch offers
+        # it (13 us of a 43 us forward at 32^2 went into building one)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return raw(torch.cuda.current_device())
+        return torch.cuda.current_stream().cuda_stream
     return 0
 
 
@@ -204,11 +210,15 @@ def _need(a, n: int, dtype, what: str) -> None:
     """Raises ValueError unless `a` holds exactly n elements of numpy dtype
     `dtype`: the C ABI takes raw pointers and sizes, so a short or wrongly
     typed buffer would be read or written past its end."""
-    m = int(np.prod(a.shape))
+    m = _numel(a)
     dt = a.dtype if isinstance(a, np.ndarray) else _np_dtype(a.dtype)
-    if m != n or dt != np.dtype(dtype):
+    if m != n or dt != dtype:
         raise ValueError(f"{what}: expected {n} elements of {np.dtype(dtype).name}, "
                          f"got {m} of {dt}")
+
+
+def _numel(a) -> int:
+    return a.size if isinstance(a, np.ndarray) else a.numel()
 
 
 def _ptr(a) -> int:
@@ -356,7 +366,7 @@ class Plan:
         return (batch, self.nt, self.my, self.mx)
 
     def _batch_of(self, a, per) -> int:
-        n = int(np.prod(a.shape))
+        n = _numel(a)
         if n % per:
             raise ValueError(f"array of {n} elements is not a whole number of {per}-element volumes")
         return n // per
@@ -707,10 +717,15 @@ def _pow2_at_least(n: int) -> int:
     return p
 
 
-def _np_dtype(tdt):
+@functools.lru_cache(maxsize=None)
+def _dtype_map() -> dict:
     torch = _torch()
     return {torch.float32: np.float32, torch.float64: np.float64,
-            torch.complex64: np.complex64, torch.complex128: np.complex128}.get(tdt, None)
+            torch.complex64: np.complex64, torch.complex128: np.complex128}
+
+
+def _np_dtype(tdt):
+    return _dtype_map().get(tdt, None)
 
 
 def _table_format(table, plan: Plan):
@@ -731,7 +746,10 @@ def _table_format(table, plan: Plan):
                      f"spectral {spectral} complex")
 
 
+@functools.lru_cache(maxsize=None)
 def _autograd_fn():
+    """The autograd function, created once: a class per call cost most of a
+    small gradient's time."""
     torch = _torch()
 
     class PatOp(torch.autograd.Function):
