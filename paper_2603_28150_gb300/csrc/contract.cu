@@ -95,7 +95,8 @@ __device__ __forceinline__ void mac_conj(cx<R>& acc, cx<R> h, cx<R> x) {
   acc.y = fma(-h.y, x.x, acc.y);
 }
 
-// grid (nkb, ceil(batch / VB)); block kWarps * 32; dynamic smem VB * nzg*ZG * 32 complex.
+// grid (ceil(batch / VB), nkb): the volume groups of a block of bins are
+// neighbours and share its table rows through L2. Block kWarps * 32; dynamic smem VB * nzg*ZG * 32 complex.
 template <typename R, bool CPLX, int VB>
 __global__ void __launch_bounds__(kWarps * 32)
     k_contract_fwd(const typename vec16<R>::type* __restrict__ table,
@@ -107,9 +108,9 @@ __global__ void __launch_bounds__(kWarps * 32)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<R>* xs = reinterpret_cast<cx<R>*>(smem_raw);  // [VB][nzg*ZG][32]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t kb = blockIdx.x;
+  const int64_t kb = blockIdx.y;
   const int64_t k = kb * 32 + lane;
-  const int b0 = blockIdx.y * VB;
+  const int b0 = blockIdx.x * VB;
   const int nzp = nzg * ZG;
   pdl_wait();
   for (int i = threadIdx.x; i < VB * nzp * 32; i += blockDim.x) {
@@ -126,7 +127,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 #pragma unroll
     for (int v = 0; v < VB; ++v) acc[v] = mk<R>(0, 0);
     const V* hp = tb + (int64_t)t * nzg * 32;
-#pragma unroll 4
+#pragma unroll(CPLX && VB == 1 && sizeof(R) == 4 ? 4 : 4)
     for (int g = 0; g < nzg; ++g) {
       E e[ZG];
       unpack<R, CPLX>(ld_stream(hp + g * 32), e);
@@ -144,10 +145,23 @@ __global__ void __launch_bounds__(kWarps * 32)
   }
 }
 
-// grid (nkb, ceil(batch / VB), z-chunks); block kWarps * 32. Warp w of z-chunk c
+// grid (ceil(batch / VB), nkb, z-chunks); block kWarps * 32. Warp w of z-chunk c
 // owns the z-groups g = c * kWarps * GPW + w + j * kWarps, j < GPW. Single-
 // volume float variants are held to 32 registers so 8 CTAs (all 64 warp slots)
 // stay resident: the stream needs the warps more than the registers.
+//
+// Samples walked at a time, their loads in flight together. Complex float
+// tables: eight for one volume (128^2 x 64 x 256, 4.3 GB: 716 -> 622 us, 650
+// with two; 384 x 326 x 12 x 40: 217 -> 204), four for two (833 -> 675). Four for real tables with four volumes
+// (128 x 96 on 256 x 192: 536 -> 422) and in FP64 with one (64^2 x 32 x 128:
+// 143 -> 134); one elsewhere (single real volumes live on occupancy).
+template <typename R, bool CPLX, int VB, int GPW>
+__host__ __device__ constexpr int adj_unroll() {
+  if (sizeof(R) == 4 && CPLX) return VB == 1 ? 8 : 4;
+  if (!CPLX && GPW <= 2 && VB == (sizeof(R) == 4 ? 4 : 1)) return 4;
+  return 1;
+}
+
 template <typename R, bool CPLX, int VB, int GPW>
 __global__ void __launch_bounds__(kWarps * 32, (sizeof(R) == 4 && !CPLX && VB == 1 && GPW <= 2) ? 8 : 1)
     k_contract_adj(const typename vec16<R>::type* __restrict__ table,
@@ -157,9 +171,9 @@ __global__ void __launch_bounds__(kWarps * 32, (sizeof(R) == 4 && !CPLX && VB ==
   typedef typename Elem<R, CPLX>::T E;
   constexpr int ZG = Elem<R, CPLX>::ZG;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t kb = blockIdx.x;
+  const int64_t kb = blockIdx.y;
   const int64_t k = kb * 32 + lane;
-  const int b0 = blockIdx.y * VB;
+  const int b0 = blockIdx.x * VB;
   const int gbase = blockIdx.z * kWarps * GPW + warp;
   cx<R> acc[GPW][ZG][VB];
 #pragma unroll
@@ -170,8 +184,9 @@ __global__ void __launch_bounds__(kWarps * 32, (sizeof(R) == 4 && !CPLX && VB ==
       for (int v = 0; v < VB; ++v) acc[j][q][v] = mk<R>(0, 0);
   const bool kok = k < K;
   const V* tb = table + (kb * nt) * (int64_t)nzg * 32 + lane;
+  constexpr int kUnroll = adj_unroll<R, CPLX, VB, GPW>();
   pdl_wait();
-#pragma unroll 1
+#pragma unroll(kUnroll)
   for (int t = 0; t < nt; ++t) {
     cx<R> d[VB];
 #pragma unroll
@@ -741,7 +756,7 @@ cudaError_t fwd_t(const Plan& p, const void* X, void* Y, int batch, cudaStream_t
   auto fn = k_contract_fwd<R, CPLX, VB>;
   const cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)L.nkb, (unsigned)((batch + VB - 1) / VB));
+  dim3 grid((unsigned)((batch + VB - 1) / VB), (unsigned)L.nkb);
   return launch_pdl(fn, grid, dim3(kWarps * 32), smem, s,
                     static_cast<const typename vec16<R>::type*>(p.table),
                     static_cast<const cx<R>*>(X), static_cast<cx<R>*>(Y), L.nz, L.nt, L.nzg, L.K,
@@ -752,7 +767,7 @@ template <typename R, bool CPLX, int VB, int GPW>
 cudaError_t adj_launch(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s) {
   const Layout& L = p.L;
   const int per_chunk = kWarps * GPW;
-  dim3 grid((unsigned)L.nkb, (unsigned)((batch + VB - 1) / VB),
+  dim3 grid((unsigned)((batch + VB - 1) / VB), (unsigned)L.nkb,
             (unsigned)((L.nzg + per_chunk - 1) / per_chunk));
   return launch_pdl(k_contract_adj<R, CPLX, VB, GPW>, grid, dim3(kWarps * 32), 0, s,
                     static_cast<const typename vec16<R>::type*>(p.table),
@@ -770,7 +785,8 @@ cudaError_t adj_t(const Plan& p, const void* D, void* Z, int batch, cudaStream_t
   return adj_launch<R, CPLX, VB, 4>(p, D, Z, batch, s);
 }
 
-// Volumes per table pass: the table is read once per ceil(batch / VB) group.
+// Volumes per table pass: a group of VB volumes reads the table once; the
+// groups of a block of bins are neighbouring CTAs, which share it through L2.
 template <typename R, bool CPLX>
 cudaError_t fwd_vb(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s) {
   if (batch >= 4) return fwd_t<R, CPLX, 4>(p, X, Y, batch, s);
@@ -779,7 +795,11 @@ cudaError_t fwd_vb(const Plan& p, const void* X, void* Y, int batch, cudaStream_
 }
 template <typename R, bool CPLX>
 cudaError_t adj_vb(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s) {
-  if (batch >= 4) return adj_t<R, CPLX, 4>(p, D, Z, batch, s);
+  // complex float tables in pairs: four volumes' D in one CTA push the table
+  // out of L1 (2085 us a launch at 128^2 x 64 x 256), two groups of two read
+  // the same rows through L2 (1049 us)
+  if constexpr (!(CPLX && sizeof(R) == 4))
+    if (batch >= 4) return adj_t<R, CPLX, 4>(p, D, Z, batch, s);
   if (batch >= 2) return adj_t<R, CPLX, 2>(p, D, Z, batch, s);
   return adj_t<R, CPLX, 1>(p, D, Z, batch, s);
 }
