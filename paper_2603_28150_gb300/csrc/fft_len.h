@@ -22,9 +22,10 @@ struct FftLen {
                              int64_t out_stride, int S, const R* sub, double* partials, const cx<R>* tw,
                              cudaStream_t st, int* nblocks, Samp sm);
   // fused residual pass between H and H* (inverse row, r = S H x - y, forward row);
-  // with `total` its last block also sums the FP64 partials (block counter `count`)
+  // with `total` its last block also sums the FP64 partials (block counter `count`), per group of
+  // S / groups slices into total[groups] when groups > 0
   static cudaError_t row_resid(cx<R>* T, int tstride, int64_t tslice, int nx, int ny, const R* y,
-                               int64_t y_stride, int S, double* partials, double* total,
+                               int64_t y_stride, int S, double* partials, double* total, int groups,
                                unsigned* count, const cx<R>* tw, cudaStream_t st, int* nblocks,
                                Samp sm);
   // stage iii row pass with the FISTA step in place of the gradient store

@@ -385,6 +385,11 @@ struct FistaStep {
   unsigned* done;
   bool next_T;  // also write the row transform of y_{k+1} over the rows of T
                 // (the next iteration's stage i then runs its column pass only)
+  // Slot step (slots != nullptr): slot s = volume s has its own coefficients
+  // (Slots), which the last block advances for the `nslots` active slots; scal,
+  // betas, iter, r2_cur and r2_hist are not used.
+  const Slots* slots = nullptr;
+  int nslots = 0;
 };
 // Stage iii over the depth slices of `S` = batch * nz spectra with the FISTA
 // step in place of the gradient store.

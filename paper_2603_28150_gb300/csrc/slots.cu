@@ -7,9 +7,8 @@
 // different iterations; one step advances slots [0, n) together:
 //   r = H y - d for all n volumes in one batched forward (the table is read
 //       once per group of volumes, not once per request), per-slot ||r||^2;
-//   g = H* r, batched;
-//   per-slot prox + momentum update with that slot's own coefficients;
-//   per-slot t_{k+1}, beta_{k+1} (FP64).
+//   g = H* r, batched, its last pass applying each slot's prox + momentum
+//       update with that slot's own coefficients, and t_{k+1}, beta_{k+1} (FP64).
 // The host keeps the active requests packed in [0, n) (pat_slot_move), and
 // each step runs as a CUDA graph captured once per n.
 #include <cmath>
@@ -19,35 +18,6 @@
 
 namespace pat {
 namespace {
-
-template <typename R>
-__global__ void __launch_bounds__(256) k_slot_update(R* __restrict__ y, R* __restrict__ xprev,
-                                                     const R* __restrict__ grad, int64_t vol,
-                                                     int64_t n, const double* __restrict__ invL,
-                                                     const double* __restrict__ lamL,
-                                                     const double* __restrict__ beta) {
-  pdl_wait();
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = i / vol;
-    const R yv = y[i], g = grad[i], xp = xprev[i];
-    R x = yv - g * (R)invL[s] - (R)lamL[s];  // prox of Eq. 14 after the step of Eq. 15
-    x = x > (R)0 ? x : (R)0;
-    y[i] = x + (R)beta[s] * (x - xp);
-    xprev[i] = x;
-  }
-}
-
-// t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2 and the next beta, per active slot.
-__global__ void k_slot_tick(double* t, double* beta, int* k, int n) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const double t1 = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t[s] * t[s]));
-  const double t2 = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t1 * t1));
-  t[s] = t1;
-  beta[s] = (t1 - 1.0) / t2;
-  k[s] += 1;
-}
 
 __global__ void k_slot_init(Slots sl, int slot, double invL, double lamL) {
   sl.t[slot] = 1.0;
@@ -73,23 +43,14 @@ size_t dat_bytes(const Layout& L) { return (size_t)L.nt * L.my * L.mx * L.rsize;
 cudaError_t slot_step(pat_plan* pp, int n, cudaStream_t s) {
   Plan& p = pp->p;
   Slots& sl = pp->x.slots;
-  const Layout& L = p.L;
-  cudaError_t e = gradient_dev(p, p.vol_a, p.dat_b, p.vol_c, n, s, nullptr, n, sl.r2);
-  if (e != cudaSuccess) return e;
-  const int64_t vol = (int64_t)L.nz * L.ny * L.nx, tot = vol * n;
-  int64_t g = (tot + 255) / 256;
-  if (g > 152 * 16) g = 152 * 16;
-  if (L.fp64)
-    e = launch_pdl(k_slot_update<double>, dim3((unsigned)g), dim3(256), 0, s,
-                   static_cast<double*>(p.vol_a), static_cast<double*>(p.vol_b),
-                   static_cast<const double*>(p.vol_c), vol, tot, sl.invL, sl.lamL, sl.beta);
-  else
-    e = launch_pdl(k_slot_update<float>, dim3((unsigned)g), dim3(256), 0, s,
-                   static_cast<float*>(p.vol_a), static_cast<float*>(p.vol_b),
-                   static_cast<const float*>(p.vol_c), vol, tot, sl.invL, sl.lamL, sl.beta);
-  if (e != cudaSuccess) return e;
-  k_slot_tick<<<(n + 127) / 128, 128, 0, s>>>(sl.t, sl.beta, sl.k, n);
-  return cudaGetLastError();
+  // the gradient's last stage applies the update and advances the slots
+  FistaStep step{};
+  step.y = p.vol_a;
+  step.xprev = p.vol_b;
+  step.done = reinterpret_cast<unsigned*>(p.iter_dev + 1);
+  step.slots = &sl;
+  step.nslots = n;
+  return gradient_dev(p, p.vol_a, p.dat_b, nullptr, n, s, nullptr, n, sl.r2, &step);
 }
 
 Graph* step_graph(pat_plan* pp, int n, int* rc) {
