@@ -39,7 +39,11 @@ template <> struct RadixPlan<32>   { static constexpr int NST = 2, RMAX = 8;  st
 template <> struct RadixPlan<64>   { static constexpr int NST = 2, RMAX = 8;  static constexpr int R[3] = {8, 8, 1}; };
 template <> struct RadixPlan<128>  { static constexpr int NST = 2, RMAX = 16; static constexpr int R[3] = {16, 8, 1}; };
 template <> struct RadixPlan<256>  { static constexpr int NST = 2, RMAX = 16; static constexpr int R[3] = {16, 16, 1}; };
-template <> struct RadixPlan<512>  { static constexpr int NST = 2, RMAX = 32; static constexpr int R[3] = {32, 16, 1}; };
+// 512 in three passes: two of radix 32 and 16 hold 32 elements a thread, 80 to 122
+// registers and two or three CTAs per SM (residual pass of 512 slices of 256^2
+// 278 us, FISTA step of 17 slices 22); 16 x 2 x 16 holds 16 (222 and 14; 16 x 4 x 8
+// 232 and 13, 8 x 4 x 16 252, 4 x 8 x 16 295).
+template <> struct RadixPlan<512>  { static constexpr int NST = 3, RMAX = 16; static constexpr int R[3] = {16, 2, 16}; };
 template <> struct RadixPlan<1024> { static constexpr int NST = 2, RMAX = 32; static constexpr int R[3] = {32, 32, 1}; };
 // three times a power of two: a 24-point first pass (every later radix divides 24)
 template <> struct RadixPlan<24>   { static constexpr int NST = 1, RMAX = 24; static constexpr int R[3] = {24, 1, 1}; };
@@ -91,9 +95,8 @@ struct TwPlan {
 
 // One padding slot per 16 elements, or per 32 where the first pass has radix
 // 32, keeps the scatter of the first pass (stride 16 or 32) free of
-// shared-memory bank conflicts (with one per 16 the radix-32 scatter met
-// two-way conflicts, 30 % of all wavefronts of the column passes at P = 512;
-// column inverse of 201 slices 69.8 -> 59.6 us).
+// shared-memory bank conflicts (with one per 16 a radix-32 scatter met two-way
+// conflicts).
 template <int P>
 __device__ __forceinline__ int pidx(int i) {
   return i + (i >> (RadixPlan<P>::RMAX == 32 ? 5 : 4));
@@ -350,7 +353,7 @@ __device__ __forceinline__ void run_passes(cx<R>* buf, const cx<R>* tw, int tid,
       }
     }
     // paired FP32 adds in the radix-2 butterflies of the plans with radices up
-    // to 16 (P <= 256: measured faster; the radix-32 and 3 * 2^k plans were
+    // to 16 (2^k up to 512: measured faster; the radix-32 and 3 * 2^k plans were
     // slower with them and keep scalar adds)
     dft_reg<R, RAD, INV, zin, hout, (RadixPlan<P>::RMAX <= 16)>(v[q]);
   }
