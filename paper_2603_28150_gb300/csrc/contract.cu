@@ -735,7 +735,6 @@ cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStrea
   const int units = (L.nzg + 1) / 2;
   int nzc = (units + 7) / 8;
   int zw = (units + nzc - 1) / nzc;
-  if (zw == 3) zw = 4;  // eight warps, one pair of them staging only: 143 us at 202^2 x 17, 146 with six
   while (zw > 1 && 2 * ctas * nzc <= 200) {
     zw = (zw + 1) / 2;
     nzc = (units + zw - 1) / zw;
