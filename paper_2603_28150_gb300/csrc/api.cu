@@ -994,15 +994,21 @@ int pat_stage_contract(pat_plan* plan, const void* in, void* out, int batch, int
   if (!in || !out) return fail(PAT_ERR_ARG, "in or out is NULL");
   cudaStream_t s = (cudaStream_t)stream;
   const Plan& p = plan->p;
-  const int64_t rin = (int64_t)batch * (adjoint ? p.L.nt : p.L.nz);
-  const int64_t rout = (int64_t)batch * (adjoint ? p.L.nz : p.L.nt);
-  if (tc_slots(p, batch)) {  // the tensor path's grouped slices, converted in and out
-    PAT_CUDA(launch_to_groups(p, in, p.X, rin, s));
+  const int nin = adjoint ? p.L.nt : p.L.nz, nout = adjoint ? p.L.nz : p.L.nt;
+  // A folded plan contracts grouped slices; converting rows in and out pays
+  // once the time side's spectra outgrow the caches. Forward / adjoint in rows
+  // and converted: 64^2 x 32 x 128 (8.5 MB) 13 / 15 and 21 / 23 us, 100^2 x 33 x
+  // 201 (53 MB) 90 / 72 and 69 / 78, 128^2 x 64 x 256 (68 MB) 113 / 106 and 116 /
+  // 121, 256^2 x 128 x 512 (540 MB) 2275 / 1778 and 1353 / 1373.
+  const int64_t tbytes = 8 * p.L.Kpad * p.L.nt * batch;
+  const bool conv = p.L.fold && tbytes > ((int64_t)(adjoint ? 128 : 32) << 20);
+  if (conv || tc_slots(p, batch)) {
+    PAT_CUDA(launch_to_groups(p, in, p.X, batch, nin, s));
     if (adjoint)
       PAT_CUDA(launch_contract_adj(p, p.X, p.Y, batch, s, true));
     else
       PAT_CUDA(launch_contract_fwd(p, p.X, p.Y, batch, s, true));
-    PAT_CUDA(launch_from_groups(p, p.Y, out, rout, s));
+    PAT_CUDA(launch_from_groups(p, p.Y, out, batch, nout, s));
     return PAT_OK;
   }
   if (adjoint)

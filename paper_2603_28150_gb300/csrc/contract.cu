@@ -319,6 +319,35 @@ __device__ __forceinline__ void store_quad(cx<float>* out, int q, int bin, int n
   }
 }
 
+// Stores quad q of the four members, v[slice of the quad][member]. In rows
+// (GRP false) a frequency shard's members are four consecutive aligned slots:
+// one 32-byte store per slice then takes the place of four scattered 8-byte
+// ones.
+template <bool GRP>
+__device__ __forceinline__ void store_members(cx<float>* out, int q, const int* bins, int n,
+                                              int64_t Kpad, const cx<float> (*v)[4]) {
+  if constexpr (!GRP) {
+    cx<float>* o = out + (int64_t)(4 * q) * Kpad + bins[0];
+    const bool run = bins[0] >= 0 && bins[1] == bins[0] + 1 && bins[2] == bins[0] + 2 &&
+                     bins[3] == bins[0] + 3;
+    if (run && ((reinterpret_cast<uintptr_t>(o) | (uintptr_t)(Kpad * 8)) & 31) == 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (4 * q + i < n)
+          asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
+                           o + i * Kpad),
+                       "f"(v[i][0].x), "f"(v[i][0].y), "f"(v[i][1].x), "f"(v[i][1].y),
+                       "f"(v[i][2].x), "f"(v[i][2].y), "f"(v[i][3].x), "f"(v[i][3].y)
+                       : "memory");
+      return;
+    }
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+    if (bins[m] >= 0)
+      store_quad<GRP>(out, q, bins[m], n, Kpad, v[0][m], v[1][m], v[2][m], v[3][m]);
+}
+
 // Adds what store_quad wrote to a .. d.
 template <bool GRP>
 __device__ __forceinline__ void add_quad(const cx<float>* out, int q, int bin, int n, int64_t Kpad,
@@ -491,14 +520,14 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       for (int r = 0; r < T; r += 4) {
         const int q = (bk * T + r) / 4;
         if (4 * q >= nt) break;
+        if (g0 > 0) {
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          if (bins[m] < 0) continue;
-          if (g0 > 0) add_quad<GRP>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m],
-                                    acc[r + 2][m], acc[r + 3][m]);
-          store_quad<GRP>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m], acc[r + 2][m],
-                          acc[r + 3][m]);
+          for (int m = 0; m < 4; ++m)
+            if (bins[m] >= 0)
+              add_quad<GRP>(Yb, q, bins[m], nt, Kpad, acc[r][m], acc[r + 1][m], acc[r + 2][m],
+                            acc[r + 3][m]);
         }
+        store_members<GRP>(Yb, q, bins, nt, Kpad, &acc[r]);
       }
     }
     if (g1 < nzg) __syncthreads();  // the spectra are free
@@ -694,12 +723,14 @@ cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStrea
   // two steps in the ring two CTAs fit an SM up to 48 depths (three volumes at
   // 96^2 x 45: 72 us, 76 in blocks of 4), with one up to 80, which pays from
   // two waves of CTAs on (128^2 x 64: 83 us in blocks of 4 with three steps, 86
-  // in blocks of 8 with one; five volumes 374 and 343). Beyond that one CTA of
+  // in blocks of 8 with one; five volumes 374 and 343) and in rows at any
+  // size (one shard of 128^2 x 64: 110 in blocks of 4, 95 of 8; one of four
+  // 44 and 35; bin rows 129 and 113). Beyond that one CTA of
   // 16 warps in blocks of 4 (256^2 x 128: 1154 us, 1219 with 8 warps of 8).
   const size_t xbytes = (size_t)gc * 4096;
   if (2 * (xbytes + 8 * 2 * (8 * 512 + 8)) <= kSmemCta)
     return fold_fwd_t<GRP, 8, 2>(p, X, Y, batch, gc, s);
-  if (2 * (xbytes + 8 * (8 * 512 + 8)) <= kSmemCta && L.nrb * batch >= 2 * kFoldCtas)
+  if (2 * (xbytes + 8 * (8 * 512 + 8)) <= kSmemCta && (!GRP || L.nrb * batch >= 2 * kFoldCtas))
     return fold_fwd_t<GRP, 8, 1>(p, X, Y, batch, gc, s);
   return fold_fwd_t<GRP, 4, 3>(p, X, Y, batch, gc, s);
 }
@@ -806,40 +837,60 @@ cudaError_t adj_vb(const Plan& p, const void* D, void* Z, int batch, cudaStream_
 
 }  // namespace
 
-// Rows [S][Kpad] <-> grouped slices [S / 8][Kpad][8].
-__global__ void k_to_groups(const float2* __restrict__ in, float2* __restrict__ out, int64_t Kpad,
-                           int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / Kpad, k = i % Kpad;
-    out[((r / kGroup) * Kpad + k) * kGroup + r % kGroup] = in[i];
+// Rows [volumes][n][Kpad] <-> grouped slices: a thread holds the eight slices
+// of one bin, a warp reads or writes 256 bytes of a row at a time. Bound by the
+// bytes.
+template <bool TO>
+__global__ void __launch_bounds__(256) k_regroup(const float2* __restrict__ in,
+                                                 float2* __restrict__ out, int n, int G,
+                                                 int64_t Kpad, int kblocks) {
+  const int vg = blockIdx.x / kblocks, v = vg / G, g = vg - v * G;
+  const int64_t k = (int64_t)(blockIdx.x - vg * kblocks) * 256 + threadIdx.x;
+  if (k >= Kpad) return;
+  const int left = n - g * kGroup;  // slices of this group, eight or more but in the last
+  const int64_t row = ((int64_t)v * n + g * kGroup) * Kpad + k;
+  const int64_t grp = ((int64_t)vg * Kpad + k) * kGroup;
+  float2 x[kGroup];
+  if constexpr (TO) {
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j)
+      x[j] = j < left ? in[row + j * Kpad] : make_float2(0.f, 0.f);
+    float4* o = reinterpret_cast<float4*>(out + grp);
+#pragma unroll
+    for (int j = 0; j < kGroup / 2; ++j)
+      o[j] = make_float4(x[2 * j].x, x[2 * j].y, x[2 * j + 1].x, x[2 * j + 1].y);
+  } else {
+    const float4* src = reinterpret_cast<const float4*>(in + grp);
+#pragma unroll
+    for (int j = 0; j < kGroup / 2; ++j) {
+      const float4 q = src[j];
+      x[2 * j] = make_float2(q.x, q.y);
+      x[2 * j + 1] = make_float2(q.z, q.w);
+    }
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j)
+      if (j < left) out[row + j * Kpad] = x[j];
   }
 }
 
-__global__ void k_from_groups(const float2* __restrict__ in, float2* __restrict__ out, int64_t Kpad,
-                             int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = i / Kpad, k = i % Kpad;
-    out[i] = in[((r / kGroup) * Kpad + k) * kGroup + r % kGroup];
-  }
-}
-
-cudaError_t launch_to_groups(const Plan& p, const void* in, void* out, int64_t S, cudaStream_t s) {
-  const int64_t n = S * p.L.Kpad;
-  const int g = (int)std::min<int64_t>((n + 255) / 256, 152 * 32);
-  k_to_groups<<<g, 256, 0, s>>>(static_cast<const float2*>(in), static_cast<float2*>(out), p.L.Kpad,
-                               n);
+template <bool TO>
+cudaError_t regroup(const Plan& p, const void* in, void* out, int volumes, int n, cudaStream_t s) {
+  const int G = (n + kGroup - 1) / kGroup, kblocks = (int)((p.L.Kpad + 255) / 256);
+  const int64_t blocks = (int64_t)volumes * G * kblocks;
+  if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
+  k_regroup<TO><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const float2*>(in),
+                                                static_cast<float2*>(out), n, G, p.L.Kpad, kblocks);
   return cudaGetLastError();
 }
 
-cudaError_t launch_from_groups(const Plan& p, const void* in, void* out, int64_t S,
-                              cudaStream_t s) {
-  const int64_t n = S * p.L.Kpad;
-  const int g = (int)std::min<int64_t>((n + 255) / 256, 152 * 32);
-  k_from_groups<<<g, 256, 0, s>>>(static_cast<const float2*>(in), static_cast<float2*>(out),
-                                 p.L.Kpad, n);
-  return cudaGetLastError();
+cudaError_t launch_to_groups(const Plan& p, const void* in, void* out, int volumes, int n,
+                             cudaStream_t s) {
+  return regroup<true>(p, in, out, volumes, n, s);
+}
+
+cudaError_t launch_from_groups(const Plan& p, const void* in, void* out, int volumes, int n,
+                               cudaStream_t s) {
+  return regroup<false>(p, in, out, volumes, n, s);
 }
 
 cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s,

@@ -426,10 +426,11 @@ inline SpecRow spec_row(const Plan& p, int n) {
   r.group = p.L.fold ? n : 0;
   return r;
 }
-// [S][Kpad] rows -> grouped slices and back (S a multiple of kGroup; single precision).
-cudaError_t launch_to_groups(const Plan& p, const void* in, void* out, int64_t S, cudaStream_t s);
-cudaError_t launch_from_groups(const Plan& p, const void* in, void* out, int64_t S,
-                              cudaStream_t s);
+// Rows [volumes][n][Kpad] -> grouped slices and back (single precision).
+cudaError_t launch_to_groups(const Plan& p, const void* in, void* out, int volumes, int n,
+                             cudaStream_t s);
+cudaError_t launch_from_groups(const Plan& p, const void* in, void* out, int volumes, int n,
+                               cudaStream_t s);
 // Split-BF16 tensor-core contraction (tc_contract.cu).
 bool tc_supported(const Layout& L);
 size_t tc_table_bytes(const Layout& L);  // one direction
