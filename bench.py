@@ -287,7 +287,9 @@ def run_ours(args, world, rank, local):
     g = torch.empty_like(x)
     pair_ms = events_ms(lambda: plan.gradient(p0_d, y, out=g, resid=False), 20)
 
-    # dominant kernel: the depth contraction, timed alone with CUDA events
+    # dominant kernel: the depth contraction, timed alone with CUDA events. The
+    # stage entry works on bin rows; inside the operator the spectra are grouped
+    # and the same kernel takes about 83 / 89 us (its iteration fraction shows it)
     Kp = info["bins_padded"]
     Xb = torch.zeros((NZ, Kp), dtype=torch.complex64, device=dev)
     Yb = torch.zeros((NT, Kp), dtype=torch.complex64, device=dev)
@@ -452,8 +454,9 @@ def run_batched(dev):
         graph_ms(lambda: plan.stage_image(Sz, out=sz), 2)
     del sz, st, Sz, St
     hbm = measured_peaks().get("hbm_gbs") or 6800.0
-    # the tensor-core contraction alone, live, on spectra already in its
-    # representative-slot layout (as the operator runs it)
+    # the tensor-core contraction alone, live, on spectra in representative
+    # slots (the operator's own instance works on grouped spectra and is a few
+    # percent faster)
     srow = 4 * ((info["table_rows"] + 31) // 32 * 32)
     Xs = torch.zeros((B, nz, srow), dtype=torch.complex64, device=dev)
     Ys = torch.zeros((B, nt, srow), dtype=torch.complex64, device=dev)
@@ -479,8 +482,9 @@ def run_batched(dev):
                 "contract_adj_frac_hbm": algo / (ca_ms / 1e3) / 1e9 / hbm,
                 "contract_fwd_frac_hbm_incl_spectra": algo_spectra / (cf_ms / 1e3) / 1e9 / hbm,
                 "contract_adj_frac_hbm_incl_spectra": algo_spectra / (ca_ms / 1e3) / 1e9 / hbm,
-                # the FFT stages in the slot layout: operator minus its contraction;
-                # beside them the same stages in the bin layout, timed alone
+                # the rest of the operator (its FFT stages, on grouped spectra):
+                # operator minus the contraction above; beside it the same stages
+                # on bin rows, timed alone
                 "fft_slot_layout_ms_per_direction": [a_ms - cf_ms, at_ms - ca_ms],
                 "fft_bin_layout_ms_per_direction": [fft_fwd, fft_adj]})
     plan.check()

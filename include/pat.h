@@ -526,8 +526,9 @@ int pat_fista_step(float* y, float* xprev, const float* grad, int64_t n, double 
  * data synthesis. */
 int pat_axpby(float* y, const float* x, int64_t n, double a, double b, pat_stream stream);
 
-/* Stage ii of the folded split-BF16 path as the operator runs it, on spectra
- * already in its representative-slot layout (no conversion): rows of
+/* Stage ii of the folded split-BF16 path on spectra in representative slots
+ * (no conversion; the operator itself keeps its spectra grouped by eight
+ * slices): rows of
  * 4 * ceil(U / 32) * 32 complex float, bin k at slot 4 u + i (member i of its
  * D4 representative u), in[b][nz or nt][row], out likewise. Only for plans
  * built with PAT_FLAG_BF16_SPLIT, folded, and batch >= the tensor batch

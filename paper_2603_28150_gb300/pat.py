@@ -584,8 +584,8 @@ class Plan:
         return out
 
     def stage_contract_slots(self, X, out, batch: int, adjoint: bool = False, stream=None):
-        """Stage ii of the folded split-BF16 path on spectra already in its
-        representative-slot layout (rows of 4 * ceil(U/32) * 32 complex)."""
+        """Stage ii of the folded split-BF16 path on spectra in
+        representative slots (rows of 4 * ceil(U/32) * 32 complex)."""
         _check(lib().pat_stage_contract_slots(self._h, _ptr(X), _ptr(out), batch,
                                               1 if adjoint else 0, _stream(stream)))
         return out
