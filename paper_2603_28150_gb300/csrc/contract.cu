@@ -811,6 +811,16 @@ cudaError_t adj_t(const Plan& p, const void* D, void* Z, int batch, cudaStream_t
   // z-groups per warp: enough to cover nzg in one chunk up to 4 per warp,
   // beyond that several z-chunks each re-read D (small) but not the table.
   const int nzg = p.L.nzg;
+  if constexpr (sizeof(R) == 8) {
+    // The FP64 rate bounds these, and their time follows the slots for groups,
+    // those at or past nzg included: the fewest slots, then the fewest chunks.
+    // 17 groups (34 depths, 128 samples) in 32 slots and in 24: 128^2 1026 and
+    // 711 us, 64^2 303 and 210; complex, 34 groups in 64 and in 40: 574 and 337.
+    auto slots = [&](int gpw) { return (nzg + kWarps * gpw - 1) / (kWarps * gpw) * gpw; };
+    if (slots(1) < std::min(slots(2), slots(4))) return adj_launch<R, CPLX, VB, 1>(p, D, Z, batch, s);
+    if (slots(2) < slots(4)) return adj_launch<R, CPLX, VB, 2>(p, D, Z, batch, s);
+    return adj_launch<R, CPLX, VB, 4>(p, D, Z, batch, s);
+  }
   if (nzg <= kWarps) return adj_launch<R, CPLX, VB, 1>(p, D, Z, batch, s);
   if (nzg <= 2 * kWarps) return adj_launch<R, CPLX, VB, 2>(p, D, Z, batch, s);
   return adj_launch<R, CPLX, VB, 4>(p, D, Z, batch, s);
