@@ -53,6 +53,11 @@ __device__ __forceinline__ bool drain_wait(uint64_t* bar, uint32_t parity, uint6
     if (global_ns() > deadline) return false;
   return true;
 }
+// Orders this thread's (and, after a barrier, its peers') ordinary shared-memory
+// accesses before the asynchronous copies and MMAs it issues next.
+__device__ __forceinline__ void fence_proxy_async() {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::

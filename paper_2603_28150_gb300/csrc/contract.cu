@@ -396,8 +396,13 @@ struct TableRing {
     }
     __syncwarp();
   }
-  // Opens slot i for copies of `bytes` in all (lane 0).
+  // Opens slot i for copies of `bytes` in all (lane 0). The lanes' reads of the
+  // slot, ordinary loads before a __syncwarp, come before the copies that
+  // overwrite it: different proxies, so a fence. It costs what the loads still
+  // in flight take (forward / adjoint 83 / 89 us without, 87 / 88 with it at
+  // 128^2 x 64 x 256; 1154 / 1154 and 1225 / 1165 at 256^2 x 128 x 512).
   __device__ __forceinline__ float4* open(int i, uint32_t bytes) {
+    fence_proxy_async();
     mbar_arrive_expect_tx(&full[i], bytes);
     return rows + i * (SLOT * 32);
   }

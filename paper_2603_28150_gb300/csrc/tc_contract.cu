@@ -51,9 +51,6 @@ constexpr int kSBO = (kTile / 8) * 128;  // bytes between M/N-adjacent core matr
 constexpr int kBBytes = kN * kTile * 2;  // one 32 x 128 B-operand chunk (8 KB)
 
 // -------------------------------------------------------------------- PTX helpers
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
