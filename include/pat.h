@@ -285,12 +285,12 @@ int pat_plan_set_sensor_response(pat_plan* plan, const double* r, int nr, pat_st
 
 /* Synchronises the device and reports whether any bounded device-side wait of
  * the plan's kernels gave up since the last check (PAT_ERR_TIMEOUT; the flag
- * is cleared), else PAT_OK. The folded contraction's waits for its table
- * copies have a fixed limit (2^22 tests). */
+ * is cleared), else PAT_OK. */
 int pat_plan_check(pat_plan* plan);
 
-/* Limit of the pipeline waits of the tensor-core contraction (the mbarrier
- * waits between its table stream, operand staging, MMAs and accumulator
+/* Limit of the pipeline waits of the contraction kernels (the mbarrier waits of
+ * the folded contraction for its table copies, and those of the tensor-core
+ * contraction between its table stream, operand staging, MMAs and accumulator
  * drain): each tests its barrier at most `polls` times (< 2^32; each test may
  * suspend the thread for a short, hardware-defined time) before the kernel
  * gives up: it then records the timeout for pat_plan_check, lets every copy

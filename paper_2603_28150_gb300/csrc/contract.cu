@@ -375,21 +375,25 @@ __device__ __forceinline__ void cp_wait() {
 // filled by bulk copies of contiguous pieces of the table: lane 0 issues the
 // copies of a step, all lanes wait for it and read their own column, and the
 // slot is refilled as soon as every lane has read it, so R steps are in flight
-// and their bytes cost neither registers nor load / store slots. A wait that
-// runs out marks the ring dead: nothing more is issued or read, and close()
-// records the error once its copies have landed.
-constexpr uint32_t kRingTests = 1u << 22;  // tests per wait (seconds)
-
+// and their bytes cost neither registers nor load / store slots. A wait tests
+// its barrier `limit` times at most. Once one runs out on any lane the ring is
+// dead for the whole warp: nothing more is issued, read or passed, so slot, par
+// and fly go on naming every copy in flight (the step waited for among them),
+// and close() waits for these before the warp leaves its shared memory.
 template <int R, int SLOT>
 struct TableRing {
   float4* rows;    // [R][SLOT][32]
   uint64_t* full;  // [R]
+  uint32_t limit;
   int slot = 0;    // of the oldest step: the one to read, and then to refill
   uint32_t par = 0;
   int fly = 0;     // steps issued and not read
   bool dead = false;
-  __device__ __forceinline__ TableRing(unsigned char* smem, uint64_t* bars, int warp, int lane)
-      : rows(reinterpret_cast<float4*>(smem) + warp * (R * SLOT * 32)), full(bars + warp * R) {
+  __device__ __forceinline__ TableRing(unsigned char* smem, uint64_t* bars, int warp, int lane,
+                                       uint32_t lim)
+      : rows(reinterpret_cast<float4*>(smem) + warp * (R * SLOT * 32)),
+        full(bars + warp * R),
+        limit(lim) {
     if (lane == 0) {
       for (int i = 0; i < R; ++i) mbar_init(&full[i], 1);
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -409,24 +413,30 @@ struct TableRing {
   __device__ __forceinline__ void copy(int i, float4* dst, const float4* src, int nrows) {
     bulk_g2s(dst, src, (uint32_t)nrows * 512u, &full[i]);
   }
-  // Waits for the oldest step; its slot.
-  __device__ __forceinline__ const float4* wait() {
-    if (!dead) dead = !mbar_wait(&full[slot], par, kRingTests);
-    return rows + slot * (SLOT * 32);
+  // Waits for the oldest step, its slot in `src`; false, on every lane, once the
+  // ring is dead.
+  __device__ __forceinline__ bool wait(const float4** src) {
+    dead = !__all_sync(0xffffffffu, mbar_wait(&full[slot], par, limit));
+    *src = rows + slot * (SLOT * 32);
+    return !dead;
   }
-  // The oldest step has been read by this lane; its slot was refilled.
+  // The oldest step has been read by this warp and its slot refilled.
   __device__ __forceinline__ void next() {
     if (++slot == R) {
       slot = 0;
       par ^= 1u;
     }
   }
+  // Every lane of a dead ring's warp leaves once lane 0 has seen the copies land
+  // (kDrainNs at most).
   __device__ __forceinline__ void close(int lane, int* err) {
-    if (__any_sync(0xffffffffu, dead) && lane == 0) {
+    if (!dead) return;
+    if (lane == 0) {
       atomicExch(err, 1);
       const uint64_t deadline = global_ns() + kDrainNs;
       for (; fly > 0; --fly, next()) drain_wait(&full[slot], par, deadline);
     }
+    __syncwarp();
   }
 };
 
@@ -444,13 +454,13 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_fwd(const float4* __restrict__ table, const int4* __restrict__ members,
                const int* __restrict__ chunk, const cx<float>* __restrict__ X,
                cx<float>* __restrict__ Y, int nz, int nt, int nzg, int64_t Kpad, int tb, int gc,
-               int* __restrict__ err) {
+               uint32_t limit, int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = warp_index(), nwarps = blockDim.x >> 5;
   float4* xs = reinterpret_cast<float4*>(smem_raw);  // [4][gc][64]
   unsigned char* rings = smem_raw + 4096 * gc;
   TableRing<R, T> ring(rings, reinterpret_cast<uint64_t*>(rings + nwarps * (R * T * 512)), warp,
-                       lane);
+                       lane, limit);
   const int64_t ub = blockIdx.y;
   const int b = blockIdx.x;
   const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32;
@@ -488,7 +498,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     }
     cp_wait<0>();
     __syncthreads();
-    for (int bk = bk0; bk < bend; bk += nwarps) {
+    for (int bk = bk0; bk < bend && !ring.dead; bk += nwarps) {
       cx<float> acc[T][4];
 #pragma unroll
       for (int r = 0; r < T; ++r)
@@ -496,7 +506,8 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         for (int m = 0; m < 4; ++m) acc[r][m] = mk<float>(0.f, 0.f);
 #pragma unroll 1
       for (int g = 0; g < g1 - g0; ++g) {
-        const float4* hs = ring.wait();
+        const float4* hs;
+        if (!ring.wait(&hs)) break;
         float4 h[T];
 #pragma unroll
         for (int r = 0; r < T; ++r) h[r] = hs[r * 32 + lane];
@@ -518,6 +529,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
             }
         }
       }
+      if (ring.dead) break;
       const int4 mem = __ldg(members + ub * 32 + lane);
       const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
       cx<float>* Yb = Y + b * vol_len<GRP>(nt, Kpad);
@@ -552,14 +564,15 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_adj(const float4* __restrict__ table, const int4* __restrict__ members,
                const int* __restrict__ chunk, const cx<float>* __restrict__ D,
                cx<float>* __restrict__ Z, int nz, int nt, int nzg, int64_t Kpad, int nzc, int zw,
-               int tw, int* __restrict__ err) {
+               int tw, uint32_t limit, int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = warp_index(), nwarps = blockDim.x >> 5;
   const int tq = SQ * tw;                            // quads per stage
   float4* ds = reinterpret_cast<float4*>(smem_raw);  // [2][4][tq][64]
   unsigned char* rings = smem_raw + 2 * 4096 * tq;
   TableRing<R, 4 * GPW> ring(
-      rings, reinterpret_cast<uint64_t*>(rings + nwarps * (R * 4 * GPW * 512)), warp, lane);
+      rings, reinterpret_cast<uint64_t*>(rings + nwarps * (R * 4 * GPW * 512)), warp, lane,
+      limit);
   const int64_t ub = blockIdx.y;
   const int zc = blockIdx.x % nzc, b = blockIdx.x / nzc;
   const int zi = warp % zw, ti = warp / zw;
@@ -603,8 +616,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
                        min(tq, ntq - q0 - tq), nt, Kpad, lane, warp, nwarps);
     const float4* dst = ds + (st & 1) * 4 * tq * 64;
 #pragma unroll 1
-    for (int q = ti; q < min(tq, ntq - q0) && gbase < nzg; q += tw) {
-      const float4* hs = ring.wait();
+    for (int q = ti; q < min(tq, ntq - q0) && gbase < nzg && !ring.dead; q += tw) {
+      const float4* hs;
+      if (!ring.wait(&hs)) break;
       float4 h[4][GPW];
 #pragma unroll
       for (int r = 0; r < 4; ++r)
@@ -715,7 +729,8 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
   return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
                     reinterpret_cast<const int4*>(p.rb_members),
                     static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(X),
-                    static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad, tb, gc, p.tc_err);
+                    static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad, tb, gc,
+                    (uint32_t)p.tc_spin, p.tc_err);
 }
 
 template <bool GRP>
@@ -755,7 +770,8 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
   return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
                     reinterpret_cast<const int4*>(p.rb_members),
                     static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(D),
-                    static_cast<cx<float>*>(Z), L.nz, L.nt, L.nzg, L.Kpad, nzc, zw, tw, p.tc_err);
+                    static_cast<cx<float>*>(Z), L.nz, L.nt, L.nzg, L.Kpad, nzc, zw, tw,
+                    (uint32_t)p.tc_spin, p.tc_err);
 }
 
 // Two z-groups per warp and up to 8 warps along z; fewer along z leave warps

@@ -220,7 +220,7 @@ struct Plan {
   unsigned char* ws_base = nullptr;
   size_t ws_cap = 0, ws_used = 0;
   bool ws_external = false;
-  // Pipeline wait limit of the tensor-core kernels (polls per wait).
+  // Pipeline wait limit of the contraction kernels (polls per wait).
   int64_t tc_spin = 0;
   // D4 folding maps (device): bins of each representative (-1 = none), and
   // the representative of each bin
@@ -438,7 +438,7 @@ cudaError_t tc_build_tables(const Plan& p, void* fwd, void* adj, cudaStream_t s)
 cudaError_t tc_contract(const Plan& p, const void* tables_fwd, const void* tables_adj,
                         const void* in, void* out, int batch, bool adjoint, int* err,
                         cudaStream_t s, bool grouped);
-// Default pipeline wait limit of the tensor-core kernels (polls of
+// Default pipeline wait limit of the contraction kernels (polls of
 // mbarrier.try_wait per wait; a few seconds).
 constexpr int64_t kTcSpinDefault = int64_t(1) << 22;
 

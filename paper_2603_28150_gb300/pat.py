@@ -339,7 +339,7 @@ class Plan:
         _check(lib().pat_plan_check(self._h))
 
     def set_wait_limit(self, polls: int) -> None:
-        """Pipeline wait limit of the tensor-core kernels (tests per wait;
+        """Pipeline wait limit of the contraction kernels (tests per wait;
         < 0 restores the default, 0 makes every such wait give up)."""
         _check(lib().pat_plan_set_wait_limit(self._h, int(polls)))
 
