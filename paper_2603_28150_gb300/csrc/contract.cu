@@ -870,14 +870,14 @@ cudaError_t adj_vb(const Plan& p, const void* D, void* Z, int batch, cudaStream_
 
 // Rows [volumes][n][Kpad] <-> grouped slices: a thread holds the eight slices
 // of one bin, a warp reads or writes 256 bytes of a row at a time. Bound by the
-// bytes.
+// bytes. The padding bins K .. Kpad of either side are left alone.
 template <bool TO>
 __global__ void __launch_bounds__(256) k_regroup(const float2* __restrict__ in,
                                                  float2* __restrict__ out, int n, int G,
-                                                 int64_t Kpad, int kblocks) {
+                                                 int64_t K, int64_t Kpad, int kblocks) {
   const int vg = blockIdx.x / kblocks, v = vg / G, g = vg - v * G;
   const int64_t k = (int64_t)(blockIdx.x - vg * kblocks) * 256 + threadIdx.x;
-  if (k >= Kpad) return;
+  if (k >= K) return;
   const int left = n - g * kGroup;  // slices of this group, eight or more but in the last
   const int64_t row = ((int64_t)v * n + g * kGroup) * Kpad + k;
   const int64_t grp = ((int64_t)vg * Kpad + k) * kGroup;
@@ -906,11 +906,12 @@ __global__ void __launch_bounds__(256) k_regroup(const float2* __restrict__ in,
 
 template <bool TO>
 cudaError_t regroup(const Plan& p, const void* in, void* out, int volumes, int n, cudaStream_t s) {
-  const int G = (n + kGroup - 1) / kGroup, kblocks = (int)((p.L.Kpad + 255) / 256);
+  const int G = (n + kGroup - 1) / kGroup, kblocks = (int)((p.L.K + 255) / 256);
   const int64_t blocks = (int64_t)volumes * G * kblocks;
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
   k_regroup<TO><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const float2*>(in),
-                                                static_cast<float2*>(out), n, G, p.L.Kpad, kblocks);
+                                                static_cast<float2*>(out), n, G, p.L.K, p.L.Kpad,
+                                                kblocks);
   return cudaGetLastError();
 }
 
