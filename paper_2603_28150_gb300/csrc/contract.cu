@@ -624,6 +624,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int j = 0; j < GPW; ++j) h[r][j] = hs[(j * 4 + r) * 32 + lane];
+      float4 d0[4];  // read before the fence of the refill holds lane 0 up
+#pragma unroll
+      for (int m = 0; m < 4; ++m) d0[m] = dst[(m * tq + q) * 64 + quad_slot(lane, 0)];
       --ring.fly;
       __syncwarp();
       refill(ring.slot);
@@ -639,7 +642,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-          const float4 d = dst[(m * tq + q) * 64 + quad_slot(lane, hf)];
+          const float4 d = hf ? dst[(m * tq + q) * 64 + quad_slot(lane, 1)] : d0[m];
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
             const cx<float> dv = k ? mk<float>(d.z, d.w) : mk<float>(d.x, d.y);
@@ -739,19 +742,21 @@ cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStrea
   if ((size_t)L.nzg * 4096 > kSmemCta) return cudaErrorInvalidValue;  // more than 224 depths
   // the spectra of up to 128 depths are resident at a time, more take another pass
   const int gc = std::min(L.nzg, 32);
-  // Blocks of 8 samples read the spectra half as often as blocks of 4. With
-  // two steps in the ring two CTAs fit an SM up to 48 depths (three volumes at
-  // 96^2 x 45: 72 us, 76 in blocks of 4), with one up to 80, which pays from
-  // two waves of CTAs on (128^2 x 64: 83 us in blocks of 4 with three steps, 86
-  // in blocks of 8 with one; five volumes 374 and 343) and in rows at any
-  // size (one shard of 128^2 x 64: 110 in blocks of 4, 95 of 8; one of four
-  // 44 and 35; bin rows 129 and 113). Beyond that one CTA of
-  // 16 warps in blocks of 4 (256^2 x 128: 1154 us, 1219 with 8 warps of 8).
+  // Blocks of 8 samples read the spectra half as often as blocks of 4 and take
+  // half as many fences (TableRing::open). With two steps in the ring two CTAs
+  // fit an SM up to 48 depths (three volumes at 96^2 x 45: 75 us, 81 in blocks
+  // of 4). Beyond, blocks of 8 have one step in the ring, which pays from two
+  // waves of CTAs on: two CTAs an SM up to 80 depths (128^2 x 64: 89 us in
+  // blocks of 4 with three steps, 91 in blocks of 8; five volumes 402 and 351),
+  // then one of 16 warps (256^2 x 128 x 512: 1212 and 1165; 71 CTAs at
+  // 64^2 x 128 x 256: 47 and 50). In rows up to 80 depths at any size (one
+  // shard of 128^2 x 64: 110 in blocks of 4, 95 of 8; one of four 44 and 35;
+  // bin rows 129 and 113).
   const size_t xbytes = (size_t)gc * 4096;
   if (2 * (xbytes + 8 * 2 * (8 * 512 + 8)) <= kSmemCta)
     return fold_fwd_t<GRP, 8, 2>(p, X, Y, batch, gc, s);
-  if (2 * (xbytes + 8 * (8 * 512 + 8)) <= kSmemCta && (!GRP || L.nrb * batch >= 2 * kFoldCtas))
-    return fold_fwd_t<GRP, 8, 1>(p, X, Y, batch, gc, s);
+  const bool fits = 2 * (xbytes + 8 * (8 * 512 + 8)) <= kSmemCta;
+  if (GRP ? L.nrb * batch >= 2 * kFoldCtas : fits) return fold_fwd_t<GRP, 8, 1>(p, X, Y, batch, gc, s);
   return fold_fwd_t<GRP, 4, 3>(p, X, Y, batch, gc, s);
 }
 
