@@ -995,13 +995,19 @@ int pat_stage_contract(pat_plan* plan, const void* in, void* out, int batch, int
   cudaStream_t s = (cudaStream_t)stream;
   const Plan& p = plan->p;
   const int nin = adjoint ? p.L.nt : p.L.nz, nout = adjoint ? p.L.nz : p.L.nt;
-  // A folded plan contracts grouped slices; converting rows in and out pays
-  // once the time side's spectra outgrow the caches. Forward / adjoint in rows
-  // and converted: 64^2 x 32 x 128 (8.5 MB) 13 / 15 and 21 / 23 us, 100^2 x 33 x
-  // 201 (53 MB) 90 / 72 and 69 / 78, 128^2 x 64 x 256 (68 MB) 113 / 106 and 116 /
-  // 121, 256^2 x 128 x 512 (540 MB) 2275 / 1778 and 1353 / 1373.
-  const int64_t tbytes = 8 * p.L.Kpad * p.L.nt * batch;
-  const bool conv = p.L.fold && tbytes > ((int64_t)(adjoint ? 128 : 32) << 20);
+  // A folded plan contracts grouped slices best; converting rows in and out (and
+  // through X and Y) pays once the scattered rows outgrow the 129 MB of L2. The
+  // forward scatters its larger side: all volumes' input and output count. Rows /
+  // converted, us: 128^2 x 64 x 256, 85 MB, 100 / 118, two volumes 215 / 221, five
+  // 639 / 484; 100^2 x 33 x 201, 62 MB, 59 / 69, three 209 / 178; five of
+  // 128^2 x 5 x 101, 140 MB, 120 / 93; 256^2 x 64 x 128, 202 MB, 385 / 270;
+  // 256^2 x 128 x 512, 674 MB, 2141 / 1412. The adjoint reads that side, one
+  // volume at a time, and scatters the depths: 105 / 119, 201 / 217, 494 / 488;
+  // 64 / 80, 161 / 199; 100 / 148; 317 / 255; 1653 / 1395; 202^2 x 17 x 201,
+  // 229 MB, 212 / 226.
+  const int64_t bytes = 8 * p.L.Kpad * (p.L.nz + p.L.nt);  // of one volume
+  const int64_t l2 = (int64_t)128 << 20;
+  const bool conv = p.L.fold && (adjoint ? bytes > l2 && p.L.nz > 32 : bytes * batch > l2);
   if (conv || tc_slots(p, batch)) {
     PAT_CUDA(launch_to_groups(p, in, p.X, batch, nin, s));
     if (adjoint)

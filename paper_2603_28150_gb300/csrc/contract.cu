@@ -447,8 +447,11 @@ __device__ __forceinline__ int warp_index() {
 }
 
 // Forward: a warp takes blocks of T time samples and walks the z-groups, a
-// step of its ring holding the T table rows of one group. grid (batch, nrb,
-// splits of the time blocks), tb time blocks per split.
+// step of its ring holding the T table rows of one group; tb time blocks per
+// split. grid (batch, nrb, splits of the time blocks): the volumes of a block
+// share its table rows through L2. Rows: (splits, nrb, batch), since their
+// scattered 8-byte pieces are gathered into lines in L2 while one volume is
+// worked on (three volumes at 100^2 x 33 x 201: 329 us interleaved, 209 in turn).
 template <bool GRP, int T, int R>
 __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_fwd(const float4* __restrict__ table, const int4* __restrict__ members,
@@ -462,10 +465,10 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   TableRing<R, T> ring(rings, reinterpret_cast<uint64_t*>(rings + nwarps * (R * T * 512)), warp,
                        lane, limit);
   const int64_t ub = blockIdx.y;
-  const int b = blockIdx.x;
+  const int b = GRP ? blockIdx.x : blockIdx.z, split = GRP ? blockIdx.z : blockIdx.x;
   const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32;
-  const int bk0 = blockIdx.z * tb + warp;
-  const int bend = min((nt + T - 1) / T, (int)(blockIdx.z + 1) * tb);
+  const int bk0 = split * tb + warp;
+  const int bend = min((nt + T - 1) / T, (split + 1) * tb);
   for (int g0 = 0; g0 < nzg; g0 += gc) {  // z-groups whose spectra fit: one pass up to gc groups
     const int g1 = min(nzg, g0 + gc);
     int pbk = bk0, pg = g0;  // next step to copy
@@ -552,13 +555,70 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   ring.close(lane, err);
 }
 
+// Forward on rows, table rows through registers. What bounds it is the scattered
+// 8-byte accesses to the spectra; without rings two CTAs an SM leave the L1 that
+// gathers them 100 KB. Blocks of 4 samples, every depth resident. 128^2 x 64 x
+// 256: 100 us, 114 through rings; 100^2 x 33 x 201: 59 and 90; on one frequency
+// shard 89 and 96, 48 and 58. grid (1, nrb, batch).
+__global__ void __launch_bounds__(kWarps * 32, 2)
+    k_fold_fwd_rows(const float4* __restrict__ table, const int4* __restrict__ members,
+                    const int* __restrict__ chunk, const cx<float>* __restrict__ X,
+                    cx<float>* __restrict__ Y, int nz, int nt, int nzg, int64_t Kpad) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<float>* xs = reinterpret_cast<cx<float>*>(smem_raw);  // [4][nzp][32]
+  const int lane = threadIdx.x & 31, warp = warp_index(), nzp = nzg * 4;
+  const int64_t ub = blockIdx.y;
+  const int4 mem = members[ub * 32 + lane];
+  const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
+  const cx<float>* Xb = X + (int64_t)blockIdx.z * nz * Kpad;
+  cx<float>* Yb = Y + (int64_t)blockIdx.z * nt * Kpad;
+  pdl_wait();
+  for (int z = warp; z < nzp; z += kWarps) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      xs[(m * nzp + z) * 32 + lane] =
+          bins[m] >= 0 && z < nz ? Xb[(int64_t)z * Kpad + bins[m]] : mk<float>(0.f, 0.f);
+  }
+  __syncthreads();
+  const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32 + lane;
+  for (int t0 = 4 * warp; t0 < nt; t0 += 4 * kWarps) {
+    cx<float> acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[r][m] = mk<float>(0.f, 0.f);
+    const int n = min(4, nt - t0);
+    const float4* hp = tbl + folded_row(t0, 0, nt, nzg);
+#pragma unroll 4
+    for (int g = 0; g < nzg; ++g) {
+      float4 h[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        h[r] = r < n ? ld_stream(hp + (g * n + r) * 32) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        cx<float> x[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) x[m] = xs[(m * nzp + g * 4 + q) * 32 + lane];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const float hq = q == 0 ? h[r].x : q == 1 ? h[r].y : q == 2 ? h[r].z : h[r].w;
+#pragma unroll
+          for (int m = 0; m < 4; ++m) mac(acc[r][m], hq, x[m]);
+        }
+      }
+    }
+    store_members<false>(Yb, t0 / 4, bins, nt, Kpad, acc);
+  }
+}
+
 // Adjoint: warp (zi, ti) of zw x tw owns the z-groups (zc zw + zi) GPW + j
 // (j < GPW) and the quads ti, ti + tw, ...; the 4 members' D of SQ tw quads
 // are staged in shared memory (two buffers, the next stage's copies in flight
 // during the current one) and reused by all warps; the table comes through
 // the warp's ring as in the forward. With tw > 1 the warps' partial sums of
 // one z-group meet in shared memory at the end, in the order of ti. grid
-// (z-chunks x batch, nrb).
+// (z-chunks x batch, nrb), rows (z-chunks, nrb, batch) as in the forward.
 template <bool GRP, int GPW, int SQ, int R>
 __global__ void __launch_bounds__(kFoldThreads, 1)
     k_fold_adj(const float4* __restrict__ table, const int4* __restrict__ members,
@@ -574,7 +634,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       rings, reinterpret_cast<uint64_t*>(rings + nwarps * (R * 4 * GPW * 512)), warp, lane,
       limit);
   const int64_t ub = blockIdx.y;
-  const int zc = blockIdx.x % nzc, b = blockIdx.x / nzc;
+  const int zc = GRP ? blockIdx.x % nzc : blockIdx.x, b = GRP ? blockIdx.x / nzc : blockIdx.z;
   const int zi = warp % zw, ti = warp / zw;
   const int gbase = (zc * zw + zi) * GPW;
   const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32;
@@ -698,14 +758,86 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   }
 }
 
+// Adjoint on rows, table rows through registers: warp w of a z-chunk owns the
+// z-groups w and w + 8 of 16; the members' D of 32 samples at a time in shared
+// memory, the loads of 8 samples in flight together. Bound as k_fold_fwd_rows.
+// 128^2 x 128 x 128: 111 us, 134 through rings; 128^2 x 112 x 64 60 and 72, on one
+// frequency shard 50 and 68. grid (z-chunks, nrb, batch).
+__global__ void __launch_bounds__(kWarps * 32, 2)
+    k_fold_adj_rows(const float4* __restrict__ table, const int4* __restrict__ members,
+                    const int* __restrict__ chunk, const cx<float>* __restrict__ D,
+                    cx<float>* __restrict__ Z, int nz, int nt, int nzg, int64_t Kpad) {
+  constexpr int GPW = 2, TC = 32;
+  __shared__ cx<float> ds[TC][4][32];
+  const int lane = threadIdx.x & 31, warp = warp_index();
+  const int64_t ub = blockIdx.y;
+  const int4 mem = members[ub * 32 + lane];
+  const int bins[4] = {mem.x, mem.y, mem.z, mem.w};
+  const int gbase = blockIdx.x * kWarps * GPW + warp;
+  const cx<float>* Db = D + (int64_t)blockIdx.z * nt * Kpad;
+  const float4* tbl = table + (int64_t)(chunk ? chunk[ub] : ub) * nt * nzg * 32 + lane;
+  cx<float> acc[GPW][4][4];
+#pragma unroll
+  for (int j = 0; j < GPW; ++j)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[j][q][m] = mk<float>(0.f, 0.f);
+  pdl_wait();
+  for (int t0 = 0; t0 < nt; t0 += TC) {
+    __syncthreads();
+    for (int tt = warp; tt < TC; tt += kWarps) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m)
+        ds[tt][m][lane] = bins[m] >= 0 && t0 + tt < nt ? Db[(int64_t)(t0 + tt) * Kpad + bins[m]]
+                                                       : mk<float>(0.f, 0.f);
+    }
+    __syncthreads();
+    const int tn = min(TC, nt - t0);
+    for (int tt = 0; tt < tn; tt += 8) {
+      float4 h[8][GPW];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int j = 0; j < GPW; ++j) {
+          const int g = gbase + j * kWarps;
+          h[r][j] = g < nzg && tt + r < tn ? ld_stream(tbl + folded_row(t0 + tt + r, g, nt, nzg))
+                                           : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        cx<float> d[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) d[m] = ds[(tt + r) & (TC - 1)][m][lane];
+#pragma unroll
+        for (int j = 0; j < GPW; ++j) {
+          const float hq[4] = {h[r][j].x, h[r][j].y, h[r][j].z, h[r][j].w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) mac(acc[j][q][m], hq[q], d[m]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < GPW; ++j) {
+    const int g = gbase + j * kWarps;
+    if (g >= nzg) break;
+    store_members<false>(Z + (int64_t)blockIdx.z * nz * Kpad, g, bins, nz, Kpad, acc[j]);
+  }
+}
+
 constexpr size_t kSmemCta = 227 * 1024;  // most shared memory of a CTA (and of an SM's CTAs)
 
+// one: one CTA of up to 16 warps per SM even where two would fit.
 template <bool GRP, int T, int R>
-cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc, cudaStream_t s) {
+cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc, bool one,
+                       cudaStream_t s) {
   const Layout& L = p.L;
   constexpr size_t ring = (size_t)R * (T * 512 + 8);  // bytes per warp
   const size_t xbytes = (size_t)gc * 4096;
-  const bool two = 2 * (xbytes + 8 * ring) <= kSmemCta;
+  const bool two = !one && 2 * (xbytes + 8 * ring) <= kSmemCta;
   const int nwarps = two ? 8 : (int)std::min<size_t>(16, (kSmemCta - xbytes) / ring);
   const size_t smem = xbytes + nwarps * ring;
   auto fn = k_fold_fwd<GRP, T, R>;
@@ -728,7 +860,8 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
       tb = n;
     }
   }
-  dim3 grid((unsigned)batch, (unsigned)L.nrb, (unsigned)((nb + tb - 1) / tb));
+  const unsigned splits = (unsigned)((nb + tb - 1) / tb);
+  const dim3 grid(GRP ? (unsigned)batch : splits, (unsigned)L.nrb, GRP ? splits : (unsigned)batch);
   return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
                     reinterpret_cast<const int4*>(p.rb_members),
                     static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(X),
@@ -736,12 +869,33 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
                     (uint32_t)p.tc_spin, p.tc_err);
 }
 
-template <bool GRP>
-cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s) {
+cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, bool grouped,
+                     cudaStream_t s) {
   const Layout& L = p.L;
   if ((size_t)L.nzg * 4096 > kSmemCta) return cudaErrorInvalidValue;  // more than 224 depths
   // the spectra of up to 128 depths are resident at a time, more take another pass
   const int gc = std::min(L.nzg, 32);
+  const int64_t ctas = L.nrb * batch;
+  if (!grouped) {
+    // Rows, in bins or in a shard's slots. Up to a CTA per SM: rings of 16 warps,
+    // the time samples split (64^2 x 32 x 128: 12.1 us, 13.0 in CTAs of 8 warps,
+    // 18.7 without rings; one shard of four of 128^2 x 64 x 256: 31, 36, 58).
+    // More CTAs hide the table's latency themselves: no rings (see
+    // k_fold_fwd_rows). Slots are stored in 32-byte runs, which leaves the rings
+    // ahead at few depths (17 on 404^2: 140 us and 155) and past 112, where the
+    // spectra leave room for one CTA (128^2 x 128 x 128: 107 and 120).
+    if (ctas <= kFoldCtas / 2) return fold_fwd_t<false, 4, 2>(p, X, Y, batch, gc, true, s);
+    if (p.shard_world && L.nzg > 28) return fold_fwd_t<false, 8, 1>(p, X, Y, batch, gc, false, s);
+    if (p.shard_world && L.nzg <= 5) return fold_fwd_t<false, 4, 2>(p, X, Y, batch, gc, false, s);
+    const size_t smem = (size_t)L.nzg * 4096;
+    const cudaError_t e = allow_smem(k_fold_fwd_rows, smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(k_fold_fwd_rows, dim3(1, (unsigned)L.nrb, (unsigned)batch), dim3(kWarps * 32),
+                      smem, s, static_cast<const float4*>(p.table),
+                      reinterpret_cast<const int4*>(p.rb_members),
+                      static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(X),
+                      static_cast<cx<float>*>(Y), L.nz, L.nt, L.nzg, L.Kpad);
+  }
   // Blocks of 8 samples read the spectra half as often as blocks of 4 and take
   // half as many fences (TableRing::open). With two steps in the ring two CTAs
   // fit an SM up to 48 depths (three volumes at 96^2 x 45: 75 us, 81 in blocks
@@ -749,15 +903,12 @@ cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, cudaStrea
   // waves of CTAs on: two CTAs an SM up to 80 depths (128^2 x 64: 89 us in
   // blocks of 4 with three steps, 91 in blocks of 8; five volumes 402 and 351),
   // then one of 16 warps (256^2 x 128 x 512: 1212 and 1165; 71 CTAs at
-  // 64^2 x 128 x 256: 47 and 50). In rows up to 80 depths at any size (one
-  // shard of 128^2 x 64: 110 in blocks of 4, 95 of 8; one of four 44 and 35;
-  // bin rows 129 and 113).
+  // 64^2 x 128 x 256: 47 and 50).
   const size_t xbytes = (size_t)gc * 4096;
   if (2 * (xbytes + 8 * 2 * (8 * 512 + 8)) <= kSmemCta)
-    return fold_fwd_t<GRP, 8, 2>(p, X, Y, batch, gc, s);
-  const bool fits = 2 * (xbytes + 8 * (8 * 512 + 8)) <= kSmemCta;
-  if (GRP ? L.nrb * batch >= 2 * kFoldCtas : fits) return fold_fwd_t<GRP, 8, 1>(p, X, Y, batch, gc, s);
-  return fold_fwd_t<GRP, 4, 3>(p, X, Y, batch, gc, s);
+    return fold_fwd_t<true, 8, 2>(p, X, Y, batch, gc, false, s);
+  if (ctas >= 2 * kFoldCtas) return fold_fwd_t<true, 8, 1>(p, X, Y, batch, gc, false, s);
+  return fold_fwd_t<true, 4, 3>(p, X, Y, batch, gc, false, s);
 }
 
 template <bool GRP, int GPW, int SQ, int R>
@@ -771,7 +922,7 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
   auto fn = k_fold_adj<GRP, GPW, SQ, R>;
   cudaError_t e = allow_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)(nzc * batch), (unsigned)L.nrb);
+  const dim3 grid((unsigned)(GRP ? nzc * batch : nzc), (unsigned)L.nrb, GRP ? 1u : (unsigned)batch);
   return launch_pdl(fn, grid, dim3(nwarps * 32), smem, s, static_cast<const float4*>(p.table),
                     reinterpret_cast<const int4*>(p.rb_members),
                     static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(D),
@@ -784,11 +935,25 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
 // z-groups over more CTAs (64^2 x 32: 12.1 us in two, 16 in one; 32^2 x 16:
 // 5.8 us in four of one group per warp, 13 in one). A stage holds two quads of
 // D per warp along the time, or four from two waves of CTAs on (256^2 x 128 x
-// 512: 1175 us with two, 1154 with four; five volumes at 128^2 346 and 332).
+// 512: 1175 us with two, 1154 with four; five volumes at 128^2 346 and 332). In
+// rows a stage of one leaves L1 more room to gather bins (100^2 x 33 x 201: 64 us,
+// 76 with two, 123 with four; one shard of 128^2 x 32 x 128 36, 48, 50), but for a
+// shard from 64 depths on (64^2 x 128 x 256: 72 with one, 63 with two). With more
+// CTAs than SMs, 64 depths or more and few samples rows take no rings
+// (k_fold_adj_rows; 100^2 x 64 x 64 33 us, 38 through rings, one shard of 256^2 x
+// 64 x 128 227 and 241; but 128^2 x 64 x 256 107 and 105, five volumes of it 543
+// and 494, one shard of 256^2 x 128 x 512 1452 and 1327).
 template <bool GRP>
 cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStream_t s) {
   const Layout& L = p.L;
   const int64_t ctas = L.nrb * batch;
+  if (!GRP && ctas > kFoldCtas / 2 && L.nzg >= 16 && L.nt <= (L.nzg > 16 ? 256 : 128))
+    return launch_pdl(k_fold_adj_rows,
+                      dim3((unsigned)((L.nzg + 15) / 16), (unsigned)L.nrb, (unsigned)batch),
+                      dim3(kWarps * 32), 0, s, static_cast<const float4*>(p.table),
+                      reinterpret_cast<const int4*>(p.rb_members),
+                      static_cast<const int*>(p.rb_chunk), static_cast<const cx<float>*>(D),
+                      static_cast<cx<float>*>(Z), L.nz, L.nt, L.nzg, L.Kpad);
   const int units = (L.nzg + 1) / 2;
   int nzc = (units + 7) / 8;
   int zw = (units + nzc - 1) / nzc;
@@ -799,10 +964,13 @@ cudaError_t fold_adj(const Plan& p, const void* D, void* Z, int batch, cudaStrea
   if (zw == 1 && 2 * ctas * nzc <= 200) return fold_adj_t<GRP, 1, 1, 4>(p, D, Z, batch, 1, 8, s);
   static constexpr int kTw[8] = {8, 4, 2, 2, 1, 1, 1, 1};
   const int tw = kTw[zw - 1];
-  if (tw == 1 && ctas * nzc >= 2 * kFoldCtas)
-    return fold_adj_t<GRP, 2, 4, 2>(p, D, Z, batch, zw, tw, s);
-  return tw <= 2 ? fold_adj_t<GRP, 2, 2, 2>(p, D, Z, batch, zw, tw, s)
-                 : fold_adj_t<GRP, 2, 1, 2>(p, D, Z, batch, zw, tw, s);
+  if constexpr (GRP) {
+    if (tw == 1 && ctas * nzc >= 2 * kFoldCtas)
+      return fold_adj_t<GRP, 2, 4, 2>(p, D, Z, batch, zw, tw, s);
+  }
+  return tw <= 2 && (GRP || (p.shard_world && L.nzg >= 16))
+             ? fold_adj_t<GRP, 2, 2, 2>(p, D, Z, batch, zw, tw, s)
+             : fold_adj_t<GRP, 2, 1, 2>(p, D, Z, batch, zw, tw, s);
 }
 
 template <typename R, bool CPLX, int VB>
@@ -887,6 +1055,7 @@ __global__ void __launch_bounds__(256) k_regroup(const float2* __restrict__ in,
   const int64_t row = ((int64_t)v * n + g * kGroup) * Kpad + k;
   const int64_t grp = ((int64_t)vg * Kpad + k) * kGroup;
   float2 x[kGroup];
+  pdl_wait();
   if constexpr (TO) {
 #pragma unroll
     for (int j = 0; j < kGroup; ++j)
@@ -914,10 +1083,9 @@ cudaError_t regroup(const Plan& p, const void* in, void* out, int volumes, int n
   const int G = (n + kGroup - 1) / kGroup, kblocks = (int)((p.L.K + 255) / 256);
   const int64_t blocks = (int64_t)volumes * G * kblocks;
   if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
-  k_regroup<TO><<<(unsigned)blocks, 256, 0, s>>>(static_cast<const float2*>(in),
-                                                static_cast<float2*>(out), n, G, p.L.K, p.L.Kpad,
-                                                kblocks);
-  return cudaGetLastError();
+  return launch_pdl(k_regroup<TO>, dim3((unsigned)blocks), dim3(256), 0, s,
+                    static_cast<const float2*>(in), static_cast<float2*>(out), n, G, p.L.K,
+                    p.L.Kpad, kblocks);
 }
 
 cudaError_t launch_to_groups(const Plan& p, const void* in, void* out, int volumes, int n,
@@ -934,7 +1102,7 @@ cudaError_t launch_contract_fwd(const Plan& p, const void* X, void* Y, int batch
                                 bool grouped) {
   if (p.tc_fwd && p.tc_min_batch > 0 && batch >= p.tc_min_batch)
     return tc_contract(p, p.tc_fwd, p.tc_adj, X, Y, batch, false, p.tc_err, s, grouped);
-  if (p.L.fold) return grouped ? fold_fwd<true>(p, X, Y, batch, s) : fold_fwd<false>(p, X, Y, batch, s);
+  if (p.L.fold) return fold_fwd(p, X, Y, batch, grouped, s);
   if (p.L.fp64)
     return p.L.real ? fwd_vb<double, false>(p, X, Y, batch, s) : fwd_vb<double, true>(p, X, Y, batch, s);
   return p.L.real ? fwd_vb<float, false>(p, X, Y, batch, s) : fwd_vb<float, true>(p, X, Y, batch, s);
