@@ -903,11 +903,16 @@ cudaError_t fold_fwd(const Plan& p, const void* X, void* Y, int batch, bool grou
   // waves of CTAs on: two CTAs an SM up to 80 depths (128^2 x 64: 89 us in
   // blocks of 4 with three steps, 91 in blocks of 8; five volumes 402 and 351),
   // then one of 16 warps (256^2 x 128 x 512: 1212 and 1165; 71 CTAs at
-  // 64^2 x 128 x 256: 47 and 50).
+  // 64^2 x 128 x 256: 47 and 50). Blocks of 4 with three steps fit two CTAs an SM
+  // up to 64 depths; from 65 to 80 two with two steps are ahead once they fill
+  // three quarters of the SMs' places (128^2 x 80 x 200, 277 CTAs: 93 us, 106 in
+  // one CTA of 16 warps with three; 213 CTAs of 64^2 x 80 x 100: 47 and 41).
   const size_t xbytes = (size_t)gc * 4096;
   if (2 * (xbytes + 8 * 2 * (8 * 512 + 8)) <= kSmemCta)
     return fold_fwd_t<true, 8, 2>(p, X, Y, batch, gc, false, s);
   if (ctas >= 2 * kFoldCtas) return fold_fwd_t<true, 8, 1>(p, X, Y, batch, gc, false, s);
+  if (L.nzg > 16 && L.nzg <= 20 && 4 * ctas > 3 * kFoldCtas)
+    return fold_fwd_t<true, 4, 2>(p, X, Y, batch, gc, false, s);
   return fold_fwd_t<true, 4, 3>(p, X, Y, batch, gc, false, s);
 }
 
