@@ -1029,8 +1029,10 @@ cudaError_t adj_t(const Plan& p, const void* D, void* Z, int batch, cudaStream_t
 // groups of a block of bins are neighbouring CTAs, which share it through L2.
 template <typename R, bool CPLX>
 cudaError_t fwd_vb(const Plan& p, const void* X, void* Y, int batch, cudaStream_t s) {
-  if (batch >= 4) return fwd_t<R, CPLX, 4>(p, X, Y, batch, s);
-  if (batch >= 2) return fwd_t<R, CPLX, 2>(p, X, Y, batch, s);
+  // as many volumes as their spectra leave room for
+  const size_t one = sizeof(cx<R>) * (size_t)p.L.nzg * Elem<R, CPLX>::ZG * 32;
+  if (batch >= 4 && 4 * one <= kSmemCta) return fwd_t<R, CPLX, 4>(p, X, Y, batch, s);
+  if (batch >= 2 && 2 * one <= kSmemCta) return fwd_t<R, CPLX, 2>(p, X, Y, batch, s);
   return fwd_t<R, CPLX, 1>(p, X, Y, batch, s);
 }
 template <typename R, bool CPLX>
