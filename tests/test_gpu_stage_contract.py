@@ -82,3 +82,21 @@ def test_shard_forward_is_the_adjoint_of_the_adjoint(nz, nt):
     store = torch.zeros(nt * W + 1, dtype=torch.complex64, device="cuda")
     b = shard.shard_contract(X, store[1:].view(nt, W))  # 8-byte aligned: single stores
     assert torch.equal(Y, b)
+
+
+# rows of ragged groups converted in both directions (143 MB and past 32 depths)
+def test_converted_rows_of_ragged_groups():
+    import torch
+    n, nz, nt = 256, 35, 101
+    plan = Plan(n, n, nz, nt, 2 * n, 2 * n,
+                medium=Medium(MED_50UM.c, MED_50UM.dx, MED_50UM.dy, MED_50UM.dz, MED_50UM.dt,
+                              oracle.mz_for(nz, nt, MED_50UM), 1))
+    K, Kp = plan.info()["bins"], plan.info()["bins_padded"]
+    gen = torch.Generator(device="cuda").manual_seed(13)
+    X = torch.randn((nz, Kp), dtype=torch.complex64, device="cuda", generator=gen)
+    D = torch.randn((nt, Kp), dtype=torch.complex64, device="cuda", generator=gen)
+    Y = plan.stage_contract(X, torch.zeros_like(D))
+    Z = plan.stage_contract(D, torch.zeros_like(X), adjoint=True)
+    assert float(Y.abs().max()) > 0 and float(Z.abs().max()) > 0
+    # sums of at most 101 products: as above, over 131584 bins
+    assert per_bin_adjoint(X[:, :K], Y[:, :K], D[:, :K], Z[:, :K]) < 1e-5
