@@ -333,16 +333,14 @@ size_t dat_elems(const Layout& L, int batch) { return (size_t)batch * L.nt * L.m
 
 namespace pat {
 
-cudaError_t forward_dev(const Plan& p, const void* rho, void* d, int batch, cudaStream_t s,
-                        const void* sub, double* sumsq, int groups, double* group_sums) {
+cudaError_t forward_dev(const Plan& p, const void* rho, void* d, int batch, cudaStream_t s) {
   const Layout& L = p.L;
   const int64_t plane = (int64_t)L.ny * L.nx, scan = (int64_t)L.my * L.mx;
   const SpecRow zr = spec_row(p, L.nz), tr = spec_row(p, L.nt);
   cudaError_t e = launch_spectrum(p, rho, plane, L.nx, L.ny, p.X, zr, batch * L.nz, s);
   if (e != cudaSuccess) return e;
   if ((e = launch_contract_fwd(p, p.X, p.Y, batch, s, zr.group > 0)) != cudaSuccess) return e;
-  return launch_image(p, p.Y, tr, d, scan, batch * L.nt, sub, sumsq, s, groups, group_sums,
-                      sampling_of(L));
+  return launch_image(p, p.Y, tr, d, scan, batch * L.nt, nullptr, nullptr, s, sampling_of(L));
 }
 
 cudaError_t gradient_dev(const Plan& p, const void* x, const void* y, void* grad, int batch,

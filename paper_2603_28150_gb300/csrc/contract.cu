@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kWarps * 32)
 #pragma unroll
     for (int v = 0; v < VB; ++v) acc[v] = mk<R>(0, 0);
     const V* hp = tb + (int64_t)t * nzg * 32;
-#pragma unroll(CPLX && VB == 1 && sizeof(R) == 4 ? 4 : 4)
+#pragma unroll 4
     for (int g = 0; g < nzg; ++g) {
       E e[ZG];
       unpack<R, CPLX>(ld_stream(hp + g * 32), e);

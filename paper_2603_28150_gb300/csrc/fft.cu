@@ -55,16 +55,14 @@ cudaError_t spectrum_cols_t(const Plan& p, int ny_in, cx<R>* out, const SpecRow&
 
 template <typename R>
 cudaError_t image_t(const Plan& p, const cx<R>* in, const SpecRow& sr, R* out, int64_t out_stride,
-                    int S, const R* sub, double* sumsq, cudaStream_t st, int groups,
-                    double* group_sums, Samp sm) {
+                    int S, const R* sub, double* sumsq, cudaStream_t st, Samp sm) {
   const Layout& L = p.L;
   cx<R>* T = static_cast<cx<R>*>(p.T);
   const cx<R>* twx = static_cast<const cx<R>*>(p.twx);
   const cx<R>* twy = static_cast<const cx<R>*>(p.twy);
   cudaError_t e;
   int nblocks = 0;
-  const bool grouped = groups > 0 && group_sums != nullptr;
-  double* partials = (sumsq || grouped) ? p.red : nullptr;
+  double* partials = sumsq ? p.red : nullptr;
   auto col = [&]() -> cudaError_t {
     PAT_P_SWITCH(L.py, (FftLen<R, P_>::col_inv(in, sr, L.px / 2 + 1, S, T, L.tstride, L.tslice, L.ny,
                                         twy, st)))
@@ -75,17 +73,14 @@ cudaError_t image_t(const Plan& p, const cx<R>* in, const SpecRow& sr, R* out, i
                                         partials, twx, st, &nblocks, sm)))
   };
   if ((e = row()) != cudaSuccess) return e;
-  // partials are slice-major, so each group of S / groups slices owns a
-  // contiguous run of nblocks / groups partials
-  if (grouped) return launch_group_sums(p.red, nblocks / groups, groups, group_sums, st);
   if (sumsq) return launch_partials_sum(p.red, nblocks, sumsq, st);
   return cudaSuccess;
 }
 
 // Spectra of H x -> spectra of the residual r = S H x - y (S the measurement
 // operator, identity without sampling): column inverse pass into T, the fused
-// residual row pass in place, column forward pass into out; ||r||^2 summed as
-// image_t does.
+// residual row pass in place, column forward pass into out; ||r||^2 into *sumsq,
+// or per group of S / groups slices into group_sums.
 template <typename R>
 cudaError_t residual_t(const Plan& p, const cx<R>* in, const SpecRow& sr, const R* y,
                        int64_t y_stride, int S, double* sumsq, cudaStream_t st, int groups,
@@ -190,15 +185,13 @@ cudaError_t launch_spectrum(const Plan& p, const void* in, int64_t in_stride, in
 
 cudaError_t launch_image(const Plan& p, const void* in, const SpecRow& sr, void* out,
                          int64_t out_stride, int S, const void* sub, double* sumsq,
-                         cudaStream_t s, int groups, double* group_sums, Samp samp) {
+                         cudaStream_t s, Samp samp) {
   if (S <= 0) return cudaSuccess;
   if (p.L.fp64)
     return image_t<double>(p, static_cast<const cx<double>*>(in), sr, static_cast<double*>(out),
-                           out_stride, S, static_cast<const double*>(sub), sumsq, s, groups,
-                           group_sums, samp);
+                           out_stride, S, static_cast<const double*>(sub), sumsq, s, samp);
   return image_t<float>(p, static_cast<const cx<float>*>(in), sr, static_cast<float*>(out),
-                        out_stride, S, static_cast<const float*>(sub), sumsq, s, groups,
-                        group_sums, samp);
+                        out_stride, S, static_cast<const float*>(sub), sumsq, s, samp);
 }
 
 }  // namespace pat

@@ -287,12 +287,8 @@ struct PlanExt {
 
 struct FistaStep;  // below
 
-// d = H rho / rho = H* d on device buffers of the plan's precision; with `sub`,
-// the forward writes H rho - sub and sums its squares (FP64) into *sumsq, or,
-// with groups > 0, per group of nt slices into group_sums[groups].
-cudaError_t forward_dev(const Plan& p, const void* rho, void* d, int batch, cudaStream_t s,
-                        const void* sub = nullptr, double* sumsq = nullptr, int groups = 0,
-                        double* group_sums = nullptr);
+// d = H rho / rho = H* d on device buffers of the plan's precision.
+cudaError_t forward_dev(const Plan& p, const void* rho, void* d, int batch, cudaStream_t s);
 cudaError_t adjoint_dev(const Plan& p, const void* d, void* rho, int batch, cudaStream_t s);
 // grad = H*(S H x - y) (Eq. 15) with ||S H x - y||^2 summed into *sumsq, or per
 // group of nt slices into group_sums[groups]; the residual stays on the chip.
@@ -358,12 +354,12 @@ cudaError_t launch_spectrum(const Plan& p, const void* in, int64_t in_stride, in
 // *sumsq (FP64, via the plan's reduction scratch when sumsq != nullptr).
 cudaError_t launch_image(const Plan& p, const void* in, const SpecRow& sr, void* out,
                          int64_t out_stride, int S, const void* sub, double* sumsq,
-                         cudaStream_t s, int groups = 0, double* group_sums = nullptr,
-                         Samp samp = no_sampling());
+                         cudaStream_t s, Samp samp = no_sampling());
 // Stage iii then stage i on the data side of the gradient (Eq. 15): spectra
 // of H x -> spectra of r = S H x - y (both laid out as `sr` says; out may be
-// in), y [S][my][mx] with slice stride y_stride; ||r||^2 as in launch_image.
-// The residual image is never stored.
+// in), y [S][my][mx] with slice stride y_stride; ||r||^2 (FP64) into *sumsq, or
+// with groups > 0 per group of S / groups slices into group_sums[groups]. The
+// residual image is never stored.
 cudaError_t launch_residual(const Plan& p, const void* in, const SpecRow& sr, const void* y,
                             int64_t y_stride, int S, double* sumsq, cudaStream_t s, int groups,
                             double* group_sums, Samp samp, void* out);
@@ -502,9 +498,6 @@ cudaError_t launch_dot(const Plan& p, const void* a, const void* b, int64_t n, d
                        cudaStream_t s);
 // Sums n per-block partials (in order, FP64) into *out (device).
 cudaError_t launch_partials_sum(const double* partials, int n, double* out, cudaStream_t s);
-// out[g] = sum of partials[g * per, (g + 1) * per) for g < groups (in order, FP64).
-cudaError_t launch_group_sums(const double* partials, int per, int groups, double* out,
-                              cudaStream_t s);
 cudaError_t launch_scale_by_inv_norm(const Plan& p, const void* in, void* out, int64_t n,
                                      const double* sumsq_dev, cudaStream_t s);
 

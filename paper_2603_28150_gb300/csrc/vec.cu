@@ -47,17 +47,6 @@ __global__ void __launch_bounds__(1024) k_sum_partials(const double* __restrict_
   if (threadIdx.x == 0) *out = s;
 }
 
-// One block per group: out[blockIdx.x] = sum of its `per` partials.
-__global__ void __launch_bounds__(256) k_group_sums(const double* __restrict__ partials, int per,
-                                                    double* __restrict__ out) {
-  const double* p = partials + (int64_t)blockIdx.x * per;
-  pdl_wait();
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < per; i += 256) acc += p[i];
-  const double s = block_sum(acc);
-  if (threadIdx.x == 0) out[blockIdx.x] = s;
-}
-
 template <typename R>
 __global__ void __launch_bounds__(kBlock) k_scale(const R* __restrict__ in, R* __restrict__ out,
                                                   int64_t n, const double* __restrict__ sumsq) {
@@ -77,11 +66,6 @@ int grid_for(int64_t n, int cap) {
 
 cudaError_t launch_partials_sum(const double* partials, int n, double* out, cudaStream_t s) {
   return launch_pdl(k_sum_partials, dim3(1), dim3(1024), 0, s, partials, n, out);
-}
-
-cudaError_t launch_group_sums(const double* partials, int per, int groups, double* out,
-                              cudaStream_t s) {
-  return launch_pdl(k_group_sums, dim3(groups), dim3(256), 0, s, partials, per, out);
 }
 
 cudaError_t launch_dot(const Plan& p, const void* a, const void* b, int64_t n, double* out_dev,
