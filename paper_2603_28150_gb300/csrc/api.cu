@@ -303,6 +303,10 @@ int build_tensor_tables(pat_plan* pp, int flags, cudaStream_t s) {
     return fail(PAT_ERR_UNSUPPORTED,
                 "PAT_FLAG_BF16_SPLIT needs a real single-precision table, nz = 128 and nt a "
                 "multiple of 128 up to 512");
+  if (p.L.fold) {
+    const int rc = build_fold_order(p);
+    if (rc != PAT_OK) return rc;
+  }
   const size_t one = tc_table_bytes(p.L);
   PAT_CUDA(dev_alloc(&p.tc_fwd, one));
   PAT_CUDA(dev_alloc(&p.tc_adj, one));

@@ -477,6 +477,9 @@ inline bool fold_possible(const Layout& L) { return L.real && !L.fp64 && L.px ==
 // L.U / Upad / nub; members (optional) receives the host copy of the
 // representatives' bins [Upad][4].
 int build_fold_maps(Plan& p, std::vector<int>* members);
+// Order in which the tensor-core contraction takes the representatives (after
+// build_fold_maps).
+int build_fold_order(Plan& p);
 // Block layout of the CUDA-core contraction of a folded table (see
 // pat_fold_blocks): identity (one chunk per block) or radial sharing.
 struct FoldBlocks {

@@ -432,7 +432,22 @@ int build_fold_maps(Plan& p, std::vector<int>* members_out) {
   for (int64_t k = 0; k < L.K; ++k)
     if (rep[k] < 0) return fail(PAT_ERR_CUDA, "internal: a bin without representative");
   if (members_out) *members_out = members;
-  // processing order of the tensor-core contraction: 8 x 8 tiles of (a, b)
+  PAT_CUDA(dev_alloc(&p.fold_members, members.size() * sizeof(int)));
+  PAT_CUDA(dev_alloc(&p.fold_rep, rep.size() * sizeof(int)));
+  PAT_CUDA(cudaMemcpy(p.fold_members, members.data(), members.size() * sizeof(int),
+                      cudaMemcpyHostToDevice));
+  PAT_CUDA(cudaMemcpy(p.fold_rep, rep.data(), rep.size() * sizeof(int), cudaMemcpyHostToDevice));
+  return PAT_OK;
+}
+
+// Processing order of the tensor-core contraction: 8 x 8 tiles of (a, b). Only
+// plans with tensor tables pay for it (it took 5 % of the creation of a plan of
+// few depths).
+int build_fold_order(Plan& p) {
+  const Layout& L = p.L;
+  std::vector<int> members(4 * (size_t)L.U);
+  PAT_CUDA(cudaMemcpy(members.data(), p.fold_members, members.size() * sizeof(int),
+                      cudaMemcpyDeviceToHost));
   std::vector<int64_t> key((size_t)L.U);
   std::vector<int> order((size_t)L.U);
   for (int64_t u = 0; u < L.U; ++u) {
@@ -444,11 +459,6 @@ int build_fold_maps(Plan& p, std::vector<int>* members_out) {
   PAT_CUDA(dev_alloc(&p.fold_order, order.size() * sizeof(int)));
   PAT_CUDA(cudaMemcpy(p.fold_order, order.data(), order.size() * sizeof(int),
                       cudaMemcpyHostToDevice));
-  PAT_CUDA(dev_alloc(&p.fold_members, members.size() * sizeof(int)));
-  PAT_CUDA(dev_alloc(&p.fold_rep, rep.size() * sizeof(int)));
-  PAT_CUDA(cudaMemcpy(p.fold_members, members.data(), members.size() * sizeof(int),
-                      cudaMemcpyHostToDevice));
-  PAT_CUDA(cudaMemcpy(p.fold_rep, rep.data(), rep.size() * sizeof(int), cudaMemcpyHostToDevice));
   return PAT_OK;
 }
 
