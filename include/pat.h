@@ -418,7 +418,10 @@ int pat_stage_image(pat_plan* plan, const void* in, void* out, int slices,
  * bins_padded and bin index k = kx * py + ky (kx in [0, px/2]):
  *   adjoint = 0:  out[b][t][k] = sum_z Hh[k][t][z] in[b][z][k]        (Eq. 7)
  *   adjoint = 1:  out[b][z][k] = sum_t conj(Hh[k][t][z]) in[b][t][k]  (Eq. 11)
- * Hh carries the 1/(px py) factor of the inverse transform. */
+ * Hh carries the 1/(px py) factor of the inverse transform. The bins from K to
+ * bins_padded of out are left alone. On folded plans large spectra are converted
+ * to the operator's grouped layout in the plan's workspace and back, and batches
+ * on the tensor cores always are. */
 int pat_stage_contract(pat_plan* plan, const void* in, void* out, int batch, int adjoint,
                        pat_stream stream);
 

@@ -2,8 +2,8 @@
 device footprint): builds a plan with a device-generated real library and
 applies `--pairs` gradients H*(H x - y) (one forward and one adjoint each).
 
-  python profile_run.py [--n 128] [--nz 64] [--nt 256]
-         [--pairs 3] [--fista 0] [--batch 1] [--no-fold] [--no-radial] [--complex] [--tensor]
+  python profile_run.py [--n 128] [--nz 64] [--nt 256] [--pairs 3] [--fista 0]
+         [--stage 0] [--batch 1] [--no-fold] [--no-radial] [--complex] [--tensor]
 
 The data y = H x come first (4 FFT launches, 1 contraction). Each pair then
 launches, in order: stage i over depths (row, column FFT), the depth
@@ -11,7 +11,8 @@ contraction, stage iii over time samples (column, row inverse FFT), stage i
 over time samples, the time contraction, stage iii over depths; so a profiler
 skipping 12 FFT launches (or 3 contractions) starts at the second pair.
 With --fista N a power iteration (5 pairs) and an N-iteration FISTA solve
-follow (one CUDA graph of 8 kernels per iteration).
+follow (one CUDA graph of 8 kernels per iteration). With --stage N the
+contraction's stage entry runs N times in each direction at the end.
 """
 from __future__ import annotations
 
@@ -33,6 +34,7 @@ def main(argv=None):
     ap.add_argument("--nt", type=int, default=256)
     ap.add_argument("--pairs", type=int, default=3)
     ap.add_argument("--fista", type=int, default=0, help="FISTA iterations after the pairs")
+    ap.add_argument("--stage", type=int, default=0, help="stage contractions after the pairs")
     ap.add_argument("--batch", type=int, default=1)
     ap.add_argument("--no-fold", action="store_true")
     ap.add_argument("--no-radial", action="store_true",
@@ -60,6 +62,13 @@ def main(argv=None):
     if a.fista:
         L = 1.01 * plan.power_norm(torch.ones_like(x[0]), 5)
         plan.fista(y[0], iters=a.fista, L=L)
+    if a.stage:
+        Kp = plan.info()["bins_padded"]
+        X = torch.zeros((a.batch, a.nz, Kp), dtype=torch.complex64, device=dev)
+        Y = torch.zeros((a.batch, a.nt, Kp), dtype=torch.complex64, device=dev)
+        for _ in range(a.stage):
+            plan.stage_contract(X, Y, batch=a.batch)
+            plan.stage_contract(Y, X, batch=a.batch, adjoint=True)
     torch.cuda.synchronize()
     plan.check()
     info = plan.info()
