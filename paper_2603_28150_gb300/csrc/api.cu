@@ -1000,12 +1000,12 @@ int pat_stage_contract(pat_plan* plan, const void* in, void* out, int batch, int
   // A folded plan contracts grouped slices best; converting rows in and out (and
   // through X and Y) pays once the scattered rows outgrow the 129 MB of L2. The
   // forward scatters its larger side: all volumes' input and output count. Rows /
-  // converted, us: 128^2 x 64 x 256, 85 MB, 100 / 118, two volumes 215 / 221, five
-  // 639 / 484; 100^2 x 33 x 201, 62 MB, 59 / 69, three 209 / 178; five of
-  // 128^2 x 5 x 101, 140 MB, 120 / 93; 256^2 x 64 x 128, 202 MB, 385 / 270;
-  // 256^2 x 128 x 512, 674 MB, 2141 / 1412. The adjoint reads that side, one
-  // volume at a time, and scatters the depths: 105 / 119, 201 / 217, 494 / 488;
-  // 64 / 80, 161 / 199; 100 / 148; 317 / 255; 1653 / 1395; 202^2 x 17 x 201,
+  // converted, us: 128^2 x 64 x 256, 85 MB, 100 / 118, two volumes 215 / 218, five
+  // 639 / 479; 100^2 x 33 x 201, 62 MB, 59 / 69, three 209 / 175; five of
+  // 128^2 x 5 x 101, 140 MB, 120 / 89; 256^2 x 64 x 128, 202 MB, 385 / 268;
+  // 256^2 x 128 x 512, 674 MB, 2141 / 1367. The adjoint reads that side, one
+  // volume at a time, and scatters the depths: 104 / 119, 201 / 217, 494 / 488;
+  // 64 / 80, 161 / 199; 100 / 148; 317 / 253; 1653 / 1408; 202^2 x 17 x 201,
   // 229 MB, 212 / 226.
   const int64_t bytes = 8 * p.L.Kpad * (p.L.nz + p.L.nt);  // of one volume
   const int64_t l2 = (int64_t)128 << 20;

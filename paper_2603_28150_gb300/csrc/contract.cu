@@ -242,13 +242,13 @@ __global__ void __launch_bounds__(kWarps * 32, (sizeof(R) == 4 && !CPLX && VB ==
 // every bank once.
 //
 // Measured per launch (one GB300, forward / adjoint): 128^2 -> 256^2 x 64 x
-// 256, 0.40 GB stored: 83 / 89 us, from 110 / 113 with bin rows and the table
-// loaded into registers; 256^2 -> 512^2 x 128 x 512, 5.8 GB: 1154 / 1154 from
-// 2270 / 1915; 202^2 -> 512^2 x 17 x 201: 118 / 146 from 507 / 316; five
-// volumes at 64^2 -> 128^2 x 32 x 128: 31 / 37 from 57 / 76. What bounds them
+// 256, 0.40 GB stored: 87 / 88 us, from 110 / 113 with bin rows and the table
+// loaded into registers; 256^2 -> 512^2 x 128 x 512, 5.8 GB: 1170 / 1176 from
+// 2270 / 1915; 202^2 -> 512^2 x 17 x 201: 119 / 147 from 507 / 316; five
+// volumes at 64^2 -> 128^2 x 32 x 128: 32 / 38 from 57 / 76. What bounds them
 // is the load / store unit: a block of 4 samples reads its spectra (32 cycles
 // a step and warp), the ring (16), stages and stores scattered sectors (a cycle
-// per line): 64 us of the 83 at 128^2, beside 62 us of DRAM traffic and 34 us
+// per line): 64 us of the 87 at 128^2, beside 62 us of DRAM traffic and 34 us
 // of multiply-adds.
 constexpr int kFoldThreads = 512;  // most threads of a CTA (caps the registers at 128)
 
@@ -404,7 +404,8 @@ struct TableRing {
   // slot, ordinary loads before a __syncwarp, come before the copies that
   // overwrite it: different proxies, so a fence. It costs what the loads still
   // in flight take (forward / adjoint 83 / 89 us without, 87 / 88 with it at
-  // 128^2 x 64 x 256; 1154 / 1154 and 1225 / 1165 at 256^2 x 128 x 512).
+  // 128^2 x 64 x 256; 1154 / 1154 and 1225 / 1165 at 256^2 x 128 x 512, both in
+  // blocks of 4). Later in the step it costs more: the copies then start late.
   __device__ __forceinline__ float4* open(int i, uint32_t bytes) {
     fence_proxy_async();
     mbar_arrive_expect_tx(&full[i], bytes);
@@ -846,7 +847,8 @@ cudaError_t fold_fwd_t(const Plan& p, const void* X, void* Y, int batch, int gc,
   // Splits of the time blocks over CTAs, by waves of CTAs x (blocks of the
   // busiest warp + the CTA's load of its SM + its prologue): the order of the
   // measured times at 71 to 1059 blocks (64^2: 9.2 us in 2, 14.5 in 1; 128^2:
-  // 83 us in 1, 91 in 2; 5 volumes at 64^2: 31 us in 2, 33.5 in 1).
+  // 83 us in 1, 91 in 2; 5 volumes at 64^2: 31 us in 2, 33.5 in 1; all without
+  // the fence of a refill).
   const int nb = (L.nt + T - 1) / T, slots = two ? (int)kFoldCtas : (int)kFoldCtas / 2;
   const int64_t ctas = L.nrb * batch;
   int tb = nb;
@@ -940,7 +942,8 @@ cudaError_t fold_adj_t(const Plan& p, const void* D, void* Z, int batch, int zw,
 // z-groups over more CTAs (64^2 x 32: 12.1 us in two, 16 in one; 32^2 x 16:
 // 5.8 us in four of one group per warp, 13 in one). A stage holds two quads of
 // D per warp along the time, or four from two waves of CTAs on (256^2 x 128 x
-// 512: 1175 us with two, 1154 with four; five volumes at 128^2 346 and 332). In
+// 512: 1175 us with two, 1154 with four; five volumes at 128^2 346 and 332; so
+// far without the fence of a refill). In
 // rows a stage of one leaves L1 more room to gather bins (100^2 x 33 x 201: 64 us,
 // 76 with two, 123 with four; one shard of 128^2 x 32 x 128 36, 48, 50), but for a
 // shard from 64 depths on (64^2 x 128 x 256: 72 with one, 63 with two). With more
